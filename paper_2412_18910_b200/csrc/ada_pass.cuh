@@ -62,7 +62,15 @@ constexpr int kXBytes = 80 * 1024;               // the buffers' area
 __host__ __device__ constexpr int xbuf_boxes(int TP) { return TP <= 40 ? 4 : 2; }
 __host__ __device__ constexpr int xbuf_bytes(int TP) { return xbuf_boxes(TP) * TP * 256; }
 __host__ __device__ constexpr int xbuf_count(int TP) { return xbuf_bytes(TP) * kXBufs <= kXBytes ? kXBufs : kXBytes / xbuf_bytes(TP); }
-constexpr int kTmemCols = 256;                   // two accumulators of 2 TP <= 96 columns, 128 apart
+// Tensor memory.  The tensor core drops what lies below the last bit of an accumulator at every addition, so an accumulator
+// takes one section of K only (see Slab::per): two places of 2 TP columns per m tile take turns, and while the products fill
+// one, the workers add the other to the sums so far (rounded to nearest), TP columns per m tile from kTmemSums on.  Two layers
+// of 7B width, features of decode rows against 64-bit sums: 1.1e-5 off with one accumulator over K, 6.2e-6 so (7.0e-6 in the
+// multi-row kernels, whose K splits are of up to 1365 k).  It costs 2 % of a pass (7B, 11 rows at context 3801: 4.95 -> 5.03 ms a block).
+constexpr int kTmemCols = 512;
+__host__ __device__ constexpr uint32_t acc_cols(uint32_t TP) { return (2 * TP + 31) & ~31u; }
+constexpr uint32_t kTmemSums = 384;
+static_assert(2 * 2 * acc_cols(kPassRowsMax) <= kTmemSums && kTmemSums + 2 * kPassRowsMax <= kTmemCols, "tensor memory");
 constexpr int kRedBytes = (kPassRowsMax / 8) * 128 * 16;
 constexpr int kMiscBytes = 6144;                 // mbarriers and small per-CTA arrays
 // attention scratch lives where the activation buffers and the reduction buffer are (both idle
@@ -312,20 +320,32 @@ __device__ __forceinline__ bool elect_one() {
 __device__ __forceinline__ void umma_commit(uint64_t *bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
-// sums of 8 + 8 accumulator columns of this thread's tensor-memory lane: the hi and the lo parts of eight pass rows
-__device__ __forceinline__ void tmem_ld_sum8(uint32_t hi, uint32_t lo, float (&v)[8]) {
-  uint32_t a[8], b[8];
+__device__ __forceinline__ void tmem_ld8_issue(uint32_t taddr, uint32_t (&r)[8]) {   // (valid after tcgen05.wait::ld)
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-               : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3]), "=r"(a[4]), "=r"(a[5]), "=r"(a[6]), "=r"(a[7])
-               : "r"(hi)
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr)
                : "memory");
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-               : "=r"(b[0]), "=r"(b[1]), "=r"(b[2]), "=r"(b[3]), "=r"(b[4]), "=r"(b[5]), "=r"(b[6]), "=r"(b[7])
-               : "r"(lo)
+}
+__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&r)[8]) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]),
+               "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
                : "memory");
+}
+// Sums of eight pass rows: those so far (where there are any, `more`) plus the accumulator's hi and lo parts, 8 + 8 columns of this
+// thread's tensor-memory lane.
+__device__ __forceinline__ void tmem_sum8(bool more, uint32_t sums, uint32_t hi, uint32_t lo, float (&v)[8]) {
+  uint32_t a[8], b[8], c[8];
+  tmem_ld8_issue(hi, a);
+  tmem_ld8_issue(lo, b);
+  if (more) {   // (warp-uniform)
+    tmem_ld8_issue(sums, c);
+  } else {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) c[i] = 0u;
+  }
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-  for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(a[i]) + __uint_as_float(b[i]);
+  for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(c[i]) + (__uint_as_float(a[i]) + __uint_as_float(b[i]));
 }
 __device__ __forceinline__ void named_bar(int id, int threads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
@@ -490,6 +510,7 @@ struct Slab {
   int ks, kj;       // K splits of this GEMM and this CTA's split
   int c0, c1;       // this CTA's 256-k chunks [c0, c1)
   int rot;          // ... which it walks from c0 + rot, around the end
+  int per, nsec;    // chunks per section of K (in the order of the walk), sections
   int group;        // index of the slab (= group of ks CTAs)
 };
 __host__ __device__ __forceinline__ int slab_rpc(int Nseg, int nseg, int ncta) {
@@ -547,6 +568,12 @@ __device__ __forceinline__ Slab make_slab(const GemmDesc &g, int cta, int ncta) 
   // queue at the few level-2 slices that hold them.  7B, 5 rows: QKV 20.1 -> 19.4 us, gate/up 32.8 -> 31.9 us per layer,
   // verify pass 3167 -> 3112 us; eight starts are no better, and K halves (already two starts) gain nothing.
   s.rot = s.ks == 1 && s.c1 > s.c0 ? ((cta & 3) * (s.c1 - s.c0)) >> 2 : 0;
+  // Sections of 512 k, 32 additions to an accumulator; of 256 k where a CTA has 2048 or less, as the K splits of the multi-row
+  // kernels are there (512 k throughout: features 4 % further off at d_model 512 and 1 % at 1536).  Of the shape alone: a row's
+  // sums do not depend on the rows of its pass.
+  const int nch = s.c1 - s.c0;
+  s.per = nch <= 8 ? 1 : 2;
+  s.nsec = nch <= 8 ? max(1, nch) : (nch + 1) >> 1;
   return s;
 }
 // A GEMM phase as a CTA sees it, for all layers: made once, in shared memory.  (Every role worked this out again after every
@@ -556,6 +583,10 @@ struct PhaseGemm {
   Slab s;
 };
 constexpr int kPhaseGemms = PH_LM - PH_FC + 1;
+// Parities of the two accumulator places after a phase of nsec sections, all but the last of which were handed on.
+__device__ __forceinline__ uint32_t sections_done(uint32_t sphase, int nsec) {
+  return sphase ^ (uint32_t)(((nsec >> 1) & 1) | ((((nsec - 1) >> 1) & 1) << 1));
+}
 // m tile mi -> weight map index and first row
 __device__ __forceinline__ void tile_source(const GemmDesc &g, const Slab &s, int mi, int &map, int &row0) {
   if (g.epi == EPI_SWIGLU_ACT) { map = g.wmap[mi]; row0 = s.r0; }
@@ -718,6 +749,45 @@ __device__ __forceinline__ int draft_first(const PassParams &p, const SeqState &
   return j - p0 < 1 || j - p0 > p.nmax + 1 || q.stale ? -1 : p0;
 }
 
+// The issuing warp between section sec - 1 of K and section sec, whose place must have been added up.
+__device__ __noinline__ void next_section(uint64_t *secfull, uint64_t *secempty, int sec, uint32_t sphase, Counters *cnt, volatile int *abort_flag) {
+  if (elect_one()) umma_commit(&secfull[(sec - 1) & 1]);
+  __syncwarp();
+  if (sec >= 2) {
+    mbar_wait(&secempty[sec & 1], ((sphase >> (sec & 1)) ^ ((unsigned)(sec - 2) >> 1)) & 1u, cnt, abort_flag);
+    tc_fence_after();
+  }
+}
+// Column of the accumulators at `place` for rows t8 .. t8 + 7 of one m tile (t8 < TP) or of the second one.
+__device__ __forceinline__ uint32_t acc_column(uint32_t place, int TP, int t8) {
+  return place + (uint32_t)t8 + (t8 < TP ? 0u : acc_cols((uint32_t)TP) - (uint32_t)TP);
+}
+// All sections of K but the last, one after another under the products of the next (one worker warp; t_end = 0: it has no rows,
+// but its arrivals must not run ahead of the sections).  Out of line: models whose K is one section jump over it.
+__device__ __noinline__ uint32_t add_sections(uint64_t *secfull, uint64_t *secempty, uint32_t sphase, int nsec, int t_end, int TP,
+                                              uint32_t taddr, uint32_t place, uint32_t sums, Counters *cnt, volatile int *abort_flag) {
+#pragma unroll 1
+  for (int q = 0; q + 1 < nsec; ++q) {
+    mbar_wait(&secfull[q & 1], ((sphase >> (q & 1)) ^ ((unsigned)q >> 1)) & 1u, cnt, abort_flag);
+    tc_fence_after();
+#pragma unroll 1
+    for (int t8 = 0; t8 < t_end; t8 += 8) {
+      const uint32_t acc = acc_column(taddr + (uint32_t)(q & 1) * place, TP, t8);
+      float v[8];
+      uint32_t r[8];
+      tmem_sum8(q > 0, sums + (uint32_t)t8, acc, acc + (uint32_t)TP, v);
+#pragma unroll
+      for (int u = 0; u < 8; ++u) r[u] = __float_as_uint(v[u]);
+      tmem_st8(sums + (uint32_t)t8, r);
+    }
+    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+    tc_fence_before();
+    __syncwarp();
+    if ((threadIdx.x & 31) == 0) mbar_arrive(&secempty[q & 1]);
+  }
+  return sections_done(sphase, nsec);
+}
+
 // ---------------------------------------------------------------------------------- the kernel
 
 // PROMPT: the rows are a short prompt (p.prompt); a kernel of its own, for the extra tests cost the decode passes 1 %.
@@ -759,7 +829,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
   unsigned char *ring = smem;
   uint64_t *bars = reinterpret_cast<uint64_t *>(smem + kRingBytes);
   uint64_t *full = bars, *empty = bars + kSlots, *xfull = bars + 2 * kSlots, *xempty = bars + 2 * kSlots + kXBufs;
-  float *inv_rms = reinterpret_cast<float *>(bars + 2 * kSlots + 2 * kXBufs + 4 + 2 * kNumCWarps);   // [rows] (after the single barriers)
+  float *inv_rms = reinterpret_cast<float *>(bars + 2 * kSlots + 2 * kXBufs + 8 + 2 * kNumCWarps);   // [rows] (after the single barriers)
   float *ssw = inv_rms + kPassRowsMax;                                             // [rows][8] (log-probabilities: [8][16])
   int *flag_s = reinterpret_cast<int *>(ssw + 8 * kPassRowsMax);
   volatile int *abort_s = flag_s + 1;
@@ -767,12 +837,13 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
   float *red = reinterpret_cast<float *>(xbuf + kXBytes);   // [rows / 8][128 threads][4 rows] sums of the K-split pair's other CTA
   Top2 *topw = reinterpret_cast<Top2 *>(red);   // [8][rows] (LM head, which has no pairs)
   static_assert(8 * kPassRowsMax * sizeof(Top2) <= kRedBytes, "room for the warps' candidates");
-  static_assert((2 * kSlots + 2 * kXBufs + 4 + 2 * kNumCWarps) * 8 + 9 * kPassRowsMax * 4 + 16 + 4 * kFlight * 4 + sizeof(PassRows) + 8 + kPhaseGemms * sizeof(PhaseGemm) <= kMiscBytes, "misc area");
+  static_assert((2 * kSlots + 2 * kXBufs + 8 + 2 * kNumCWarps) * 8 + 9 * kPassRowsMax * 4 + 16 + 4 * kFlight * 4 + sizeof(PassRows) + 8 + kPhaseGemms * sizeof(PhaseGemm) <= kMiscBytes, "misc area");
 
   uint64_t *accfull = xempty + kXBufs;                     // accumulator of the phase complete
   uint64_t *attn_bar = accfull + 1;                        // attention: per worker warp, its 16 keys and its 16 values have landed
   uint64_t *kbar = attn_bar + 2 * kNumCWarps;                           // K-split pair: the sums of the other CTA are here
   uint64_t *step_bar = kbar + 1;                           // stopping rule: the draft length after a step is decided
+  uint64_t *secfull = step_bar + 1, *secempty = secfull + 2;   // the two places of the accumulators: a section of K is complete, has been added up by the eight workers
   uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(const_cast<int *>(abort_s) + 1);
   uint32_t *st_rec = tmem_slot + 1;   // [2 producers][offsets, ends][kFlight]: records of the stages in flight
   PassRows *rows = reinterpret_cast<PassRows *>(st_rec + 4 * kFlight);
@@ -785,6 +856,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
     for (int i = 0; i < 2 * kNumCWarps; ++i) mbar_init(attn_bar + i, 1);
     mbar_init(kbar, 1);
     mbar_init(step_bar, 1);
+    for (int i = 0; i < 2; ++i) { mbar_init(&secfull[i], 1); mbar_init(&secempty[i], kNumCWarps); }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 2) tmem_alloc(tmem_slot, kTmemCols);
@@ -901,8 +973,8 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
 
   // ================================================================= tensor-core issuer (warp 2)
   // One elected thread issues every product, in schedule order (about 58 cycles per tcgen05.mma when the
-  // products of a stage are issued back to back), so stages are also released in order.  M tile mi
-  // accumulates in tensor-memory columns [32 mi, 32 mi + 32).
+  // products of a stage are issued back to back), so stages are also released in order.  M tile mi of section q of K
+  // accumulates in the acc_cols(TP) tensor-memory columns from (mtiles (q & 1) + mi) acc_cols(TP) on.
   if (warp == 2) {
     {
       RingCursor cur{0, 0};
@@ -915,6 +987,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
       // to issue instead of 45, and the loops were bound by it (7B, 5 rows: QKV 22 400 of its 28 800 cycles).
       const int nsteps = (int)__reduce_max_sync(0xffffffffu, (unsigned)nstep);
       unsigned decisions = 0;
+      uint32_t sphase = 0;     // per place of the accumulators the parity of its next release in this phase
       for (int step = first_step;
            step < nsteps || (p.ddd_thr < 0.f && step < (int)__reduce_max_sync(0xffffffffu, (unsigned)await_length(step_bar, decisions, rows, p.cnt, abort_s)));
            ++step, xslot = 0)
@@ -939,8 +1012,13 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
           const uint32_t idesc = umma_idesc_mn(s.m64 ? 64u : 128u, 2 * TP);
           const uint32_t region16 = (uint32_t)s.region >> 4;
           const int kb = min(s.kb, kxb);
-          uint32_t started = 0;   // bit mi: the accumulator of m tile mi holds a product of this phase
+          uint32_t started = 0;   // bit mi: the accumulator of m tile mi holds a product of this section
+          uint32_t col = tmem_base;   // accumulators of the section
+          const uint32_t step_cols = (uint32_t)s.mtiles * acc_cols(TP);
+          int sec = 0, left = s.per;  // section, chunks left in it
           for (int i = s.c0, c = s.c0 + s.rot; i < s.c1; ++i, c = c + 1 == s.c1 ? s.c0 : c + 1) {
+            if (left == 0) { next_section(secfull, secempty, ++sec, sphase, p.cnt, abort_s); col = tmem_base + (sec & 1 ? step_cols : 0u); started = 0; left = s.per; }
+            --left;
             const int kleft = min(kKc, K - c * kKc);
             const int nbox = (kleft + kBoxK - 1) / kBoxK;
 #pragma unroll 1
@@ -954,7 +1032,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
                   const uint32_t off = cur.take((uint32_t)(nb * s.region));
                   const unsigned slot = (cur.n - 1) % kSlots, parity = ((cur.n - 1) / kSlots) & 1u;
                   const uint64_t adesc0 = umma_desc(ring_u + off);
-                  const uint32_t dcol = tmem_base + (uint32_t)mi * 128;
+                  const uint32_t dcol = col + (uint32_t)mi * acc_cols(TP);
                   mbar_wait(&full[slot], parity, p.cnt, abort_s);
                   tc_fence_after();
                   if (elect_one()) {   // one thread issues the stage's products and the commit that frees it
@@ -1000,8 +1078,16 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
           constexpr uint32_t xbox16 = (TP * 256) >> 4;
           const uint32_t idesc = umma_idesc_mn(s.m64 ? 64u : 128u, 2 * TP);
           const uint32_t region16 = (uint32_t)s.region >> 4, bytes = (uint32_t)(KB * s.region);
-          uint32_t acc = 0;
+          uint32_t acc = 0, col = tmem_base;        // accumulators of the section
+          const int per = s.per * (4 / kxb);
+          int sec = 0, left = per;                  // section, activation buffers left in it
           for (int n = (s.c1 - s.c0) * (4 / kxb); n > 0; --n) {   // activation buffers
+            if (left == 0) {
+              next_section(secfull, secempty, ++sec, sphase, p.cnt, abort_s);
+              col = tmem_base + (sec & 1 ? MT * acc_cols(TP) : 0u);
+              left = per; acc = 0;
+            }
+            --left;
             const uint64_t bdesc0 = umma_desc(xbuf_u + (uint32_t)(xslot * xbuf_bytes(TP)));
             mbar_wait(&xfull[xslot], (xphase >> xslot) & 1u, p.cnt, abort_s);
 #pragma unroll
@@ -1013,7 +1099,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
               tc_fence_after();
               if (elect_one()) {
                 const uint64_t ad = umma_desc(ring_u + off);
-                const uint32_t dcol = tmem_base + (uint32_t)mi * 128;
+                const uint32_t dcol = col + (uint32_t)mi * acc_cols(TP);
 #pragma unroll
                 for (int b = 0; b < KB; ++b)
 #pragma unroll
@@ -1052,6 +1138,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
         else dispatch(products);
         if (elect_one()) umma_commit(accfull);
         __syncwarp();
+        sphase = sections_done(sphase, s.nsec);
       }
     }
     __syncwarp();
@@ -1094,6 +1181,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
     bulk_g2s_hint(wst + (values ? 16 * 128 : 0), (values ? p.vpool : p.kpool) + off, bytes, bar, l2_policy_evict_first());
   };
   unsigned kuses = 0;               // completed phases of the K-split pair barrier
+  uint32_t sphase = 0;              // per place of the accumulators the parity of its next section of this phase
   (void)g8; (void)q4;
 
   for (int step = first_step; step < nstep; ++step) {
@@ -1590,6 +1678,12 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
       attn_pages(sq, at_kfirst, kend, 0);
       if (at_kfirst < kend) at_hh = hh;
     }
+    // accumulators of section q of K and this warp's m tile from taddr + (q & 1) place on, its sums from `sums` on
+    const uint32_t cols = acc_cols((uint32_t)TP), place = (uint32_t)s.mtiles * cols;
+    const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)mi * cols;
+    const uint32_t sums = tmem_base + ((uint32_t)(quarter * 32) << 16) + kTmemSums + (uint32_t)(mi * TP);
+    const int t_end = sw ? 2 * TP : TP;                  // (SwiGLU: the gate rows, then the up rows)
+    if (s.nsec > 1 && s.rows > 0) sphase = add_sections(secfull, secempty, sphase, s.nsec, active_warp ? t_end : 0, TP, taddr, place, sums, p.cnt, abort_s);
     if (s.rows > 0) {
       mbar_wait(accfull, acc_phase & 1u, p.cnt, abort_s);
       ++acc_phase;
@@ -1617,27 +1711,24 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
     const bool sends = pair && cw < 4;
     if (sends && ctid == 0) mbar_expect_tx(kbar, (unsigned)(128 * 16 * (TP >> 3)));
     if (active_warp) {
-      const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(mi * 128);
       const unsigned other = (unsigned)(s.kj ^ 1);
       const uint32_t dst = peer_addr(red + ctid * 4, other), bar = peer_addr(kbar, other);
+      const bool more = s.nsec > 1;
+      const uint32_t last = taddr + (uint32_t)((s.nsec - 1) & 1) * place;   // the last section's accumulators
+      float *y = ys + rslab;
 #pragma unroll 1
-      for (int t8 = 0; t8 < TP; t8 += 8) {
+      for (int t8 = 0; t8 < t_end; t8 += 8, y += 8 * 256) {
+        if (t8 == TP) y = ys + 128 + rslab;
+        const uint32_t acc = acc_column(last, TP, t8);   // accumulator column = pass row
         float v[8];
-        tmem_ld_sum8(taddr + (uint32_t)t8, taddr + (uint32_t)(TP + t8), v);   // accumulator column = pass row
+        tmem_sum8(more, sums + (uint32_t)t8, acc, acc + (uint32_t)TP, v);
         if (sends) {
           if (s.kj) st_async_peer(dst + (uint32_t)t8 * 256u, bar, v[0], v[2], v[4], v[6]);
           else st_async_peer(dst + (uint32_t)t8 * 256u, bar, v[1], v[3], v[5], v[7]);
         }
         if (valid) {
 #pragma unroll
-          for (int u = 0; u < 8; ++u) ys[(t8 + u) * 256 + rslab] = v[u];
-        }
-        if (sw) {
-          tmem_ld_sum8(taddr + 128u + (uint32_t)t8, taddr + 128u + (uint32_t)(TP + t8), v);
-          if (valid) {
-#pragma unroll
-            for (int u = 0; u < 8; ++u) ys[(t8 + u) * 256 + 128 + rslab] = v[u];
-          }
+          for (int u = 0; u < 8; ++u) y[u * 256] = v[u];
         }
       }
     }
