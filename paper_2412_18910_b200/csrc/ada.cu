@@ -236,6 +236,11 @@ size_t part_need_tc(int epi, int nseg, int Nseg, int K) {
 // that of the kernel (750 clocks a box at nb = 64, 820 at 96, little more than the products' time at 128).  At 60 bytes tiles
 // of 64 rows came out too cheap: a prompt of 512 tokens 14.4 -> 13.4 ms (7B), 333 tokens 10.7 -> 10.3; 16 layers of 2048: 333
 // tokens 2033 -> 1932 us, 129 tokens 1563 -> 1496, 640 tokens 2785 -> 2820.
+// 64-k boxes per accumulator, so that a prompt's features are no further from 64-bit sums than with the 128-row kernel, whose K
+// splits get shorter with K.  Two layers, 333 tokens, 128-row kernel in chunks -> pairs: d_model 4096 6.8e-6 -> 6.3e-6 with 4
+// boxes, 2048 4.54e-6 -> 4.48e-6 with 4 (4.89e-6 with 8), 1024 1.99e-6 -> 2.01e-6 and 256 2.64e-7 -> 2.58e-7 with 2 (2.76e-7 with 4).  With
+// 8 boxes the middle model's 333 tokens took 1.97 ms (2.09 with 4, 2.52 with 2), 2001 tokens of 7B 50.9 (52.2 with 4, 60.4 with 2).
+int pair_chunk(int K) { return K < 2048 ? 2 : 4; }
 struct PairPlan { int nb, token_tiles, S; };
 constexpr int kPairs = 74;
 constexpr int kPairSplitRows = 2048;    // S x rows of the partial sums at most (scratch is sized for it)
@@ -379,7 +384,7 @@ bool gemm_prompt(ada_ctx *x, int epi, const bf16 *W0, const bf16 *W1, const bf16
   memset(&t, 0, sizeof(t));
   const bool sw = r.kind == Reduce::SWIGLU;
   const int kind = sw ? PAIR_SWIGLU : r.kind == Reduce::QKV_ROPE ? PAIR_QKV : PAIR_PART;
-  t.nseg = nseg; t.Nseg = Nseg; t.K = K; t.T = x->TM;
+  t.nseg = nseg; t.Nseg = Nseg; t.K = K; t.T = x->TM; t.chunk = pair_chunk(K);
   t.weight_tiles = sw ? (Nseg + 127) / 128 : nseg * ((Nseg + 255) / 256);
   const PairPlan plan = plan_pair(x->TM, t.weight_tiles, sw ? 2 * Nseg : nseg * Nseg, K, kind == PAIR_PART);
   t.nb = plan.nb; t.token_tiles = plan.token_tiles; t.S = plan.S;

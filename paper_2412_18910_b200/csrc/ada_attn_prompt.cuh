@@ -137,7 +137,7 @@ __global__ void __launch_bounds__(kPaThreads, 1) k_attn_prompt(const AttnPromptA
         const uint32_t q = smem_u32(smem + i * Sh::kQTile), k = smem_u32(stages + (t & 1) * Sh::kStage), d = tmem_base + 256u * i;
         uint32_t acc = 0;
 #pragma unroll
-        for (int pl = 0; pl < 2; ++pl)
+        for (int pl = 1; pl >= 0; --pl)    // lo first: an addition drops what lies below the accumulator's last bit
 #pragma unroll
           for (int h = 0; h < Sh::kHalves; ++h) {
             const uint64_t ad = umma_desc(q + (uint32_t)((pl * Sh::kHalves + h) * Sh::kQBox)), bd = umma_desc(k + (uint32_t)(h * Sh::kBox));
@@ -155,7 +155,7 @@ __global__ void __launch_bounds__(kPaThreads, 1) k_attn_prompt(const AttnPromptA
         const uint32_t v = smem_u32(stages + (t & 1) * Sh::kStage + Sh::kHalves * Sh::kBox), d = tmem_base + 256u * i + 128u;
         uint32_t acc = 0;
 #pragma unroll
-        for (int pl = 0; pl < 2; ++pl)
+        for (int pl = 1; pl >= 0; --pl)
 #pragma unroll
           for (int k4 = 0; k4 < 4; ++k4) {   // 16 keys
             umma_f16_ta(d, tmem_base + 256u * i + 64u + 32u * pl + 8u * k4, pa_desc_mn(v + (uint32_t)(k4 * 2048), Sh::kBox), id_o, acc);

@@ -18,9 +18,9 @@
 //   warps 4..11 epilogue: thread = one weight row (tensor-memory lane) x nb of the tile's prompt rows
 //
 // The accumulator of the tensor cores drops what lies below its last bit at every addition: over K = 4096, hi and lo in
-// one accumulator, sums came out 8e-6 short (measured; 2.5e-5 over K = 11008).  So an accumulator takes kPairChunk x 64 k
-// only; the epilogue warps add it to fp32 sums in their registers (round to nearest) while the products go on in the
-// other accumulator.
+// one accumulator, sums came out 8e-6 short (measured; 2.5e-5 over K = 11008).  So an accumulator takes a few boxes of 64 k
+// only (GemmPairArgs::chunk, see pair_chunk), in each the lo products before the hi ones; the epilogue warps add it to fp32
+// sums in their registers (round to nearest) while the products go on in the other accumulator.
 //
 // Epilogues (template parameter): PART leaves fp32 sums of a K split for k_reduce_h (O, down, the draft head's fc: their
 // consumer needs the sums of squares of whole rows); QKV applies 1/rms, rotary embedding and writes q and the cache rows;
@@ -33,7 +33,6 @@
 namespace ada {
 
 constexpr int kPairThreads = 12 * 32;
-constexpr int kPairChunk = 8;                                 // 64-k boxes per accumulator
 constexpr int kPairStageMax = kTcABytes + 2 * 128 * 128;      // weight box + hi and lo boxes of 128 prompt rows
 constexpr int kPairRing = 4 * kPairStageMax;                  // 192 KB
 constexpr int kPairSlots = 8;                                 // barrier pairs (stages in flight at most)
@@ -51,6 +50,7 @@ struct GemmPairArgs {
   int T;                                   // rows of the pass (known on the host)
   int nb;                                  // prompt rows per CTA and tile: 32, 64, 96 or 128
   int token_tiles, weight_tiles, S;        // S: K splits (PART only)
+  int chunk;                               // 64-k boxes per accumulator
   float *part; int part_rows;              // PART: [S][part_rows][Nseg]
   // QKV and SWIGLU
   const float *ss_part; float eps; int d;
@@ -239,8 +239,8 @@ __global__ void __launch_bounds__(kPairThreads, 1) k_gemm_pair(const GemmPairArg
     for (int item = pair; item < items; item += npairs) {
       int seg, tile, tok0, kb0, kb1, split;
       decode(item, seg, tile, tok0, kb0, kb1, split);
-      for (int kc = kb0; kc < kb1; kc += kPairChunk, ++n) {
-        const int buf = n & 1, kc1 = min(kb1, kc + kPairChunk);
+      for (int kc = kb0; kc < kb1; kc += a.chunk, ++n) {
+        const int buf = n & 1, kc1 = min(kb1, kc + a.chunk);
         if (n >= 2) mbar_wait_inline(&accempty[buf], ((unsigned)(n >> 1) & 1u) ^ 1u, a.cnts, abort_s);
         tc_fence_after();
         const uint32_t dcol = tb + (uint32_t)buf * 256;
@@ -253,16 +253,13 @@ __global__ void __launch_bounds__(kPairThreads, 1) k_gemm_pair(const GemmPairArg
             const uint32_t acc = kb > kc ? 1u : 0u;
             if (kb * 64 + 64 <= a.K) {
 #pragma unroll
-              for (int k4 = 0; k4 < 4; ++k4) {
-                umma_bf16_pair(dcol, ad + 2 * k4, bh + 2 * k4, idesc, k4 > 0 ? 1u : acc);
-                umma_bf16_pair(dcol, ad + 2 * k4, bl + 2 * k4, idesc, 1u);
-              }
+              for (int k4 = 0; k4 < 4; ++k4) umma_bf16_pair(dcol, ad + 2 * k4, bl + 2 * k4, idesc, k4 > 0 ? 1u : acc);
+#pragma unroll
+              for (int k4 = 0; k4 < 4; ++k4) umma_bf16_pair(dcol, ad + 2 * k4, bh + 2 * k4, idesc, 1u);
             } else {
               const int nstep = (a.K - kb * 64 + 15) >> 4;   // k16 steps holding any k < K
-              for (int k4 = 0; k4 < nstep; ++k4) {
-                umma_bf16_pair(dcol, ad + 2 * k4, bh + 2 * k4, idesc, k4 > 0 ? 1u : acc);
-                umma_bf16_pair(dcol, ad + 2 * k4, bl + 2 * k4, idesc, 1u);
-              }
+              for (int k4 = 0; k4 < nstep; ++k4) umma_bf16_pair(dcol, ad + 2 * k4, bl + 2 * k4, idesc, k4 > 0 ? 1u : acc);
+              for (int k4 = 0; k4 < nstep; ++k4) umma_bf16_pair(dcol, ad + 2 * k4, bh + 2 * k4, idesc, 1u);
             }
             umma_commit_pair(&empty[slot]);
           }
@@ -311,7 +308,7 @@ __global__ void __launch_bounds__(kPairThreads, 1) k_gemm_pair(const GemmPairArg
       for (int blk = 0; blk < 4; ++blk)
 #pragma unroll
         for (int i = 0; i < 32; ++i) sum[blk][i] = 0.f;
-      for (int kc = kb0; kc < kb1; kc += kPairChunk, ++n) {
+      for (int kc = kb0; kc < kb1; kc += a.chunk, ++n) {
         const int buf = n & 1;
         const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * 256 + ch * a.nb);
         mbar_wait_inline(&accfull[buf], (unsigned)(n >> 1) & 1u, a.cnts, abort_s);

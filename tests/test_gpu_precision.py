@@ -103,7 +103,7 @@ def measure(model):
     return _prompt_error(model, 100)
 
 
-@pytest.mark.parametrize("m", [31, 48])
+@pytest.mark.parametrize("m", [31, 48, 129, 333])
 def test_prompt_routes(model, measure, m):
     assert _prompt_error(model, m) < 1.05 * measure
 
