@@ -635,29 +635,14 @@ __device__ __forceinline__ void stamp(const PassParams &p, int ph, int k, bool o
 
 // ---------------------------------------------------------------------------------- row lists
 
-// Attention items of the sequences in s_* (one thread).  A single sequence keeps the split size fixed when its prompt was
-// read.  The draft rows of a batch choose one for the step: 32 heads of 8 sequences are more items than CTAs, so the splits
-// are as long as balances their fixed cost (about five rounds of 64 keys for staging and merging) against an even load.
-__device__ __noinline__ void pass_items(PassRows *r, int H, int ncta, bool choose) {
-  int chunk = 0;
-  if (choose) {
-    int best = 1 << 30;
-    for (int c = 128; c <= 4096; c *= 2) {
-      int items = 0, most = 0;
-      for (int i = 0; i < r->nseq; ++i) {
-        const int nsp = (r->s_pos0[i] + r->s_rows[i] + c - 1) / c;
-        items += H * nsp;
-        most = max(most, nsp);
-      }
-      const int cost = ((items + ncta - 1) / ncta) * (c / 64 + 5);
-      if (most <= kPassMaxSplits && cost < best) { best = cost; chunk = c; }
-    }
-    if (!chunk) choose = false;
-  }
+// Attention items of the sequences in s_* (one thread).  A sequence keeps the split size fixed when its prompt was read, in every
+// pass and whatever the sequences beside it: the split a key falls in is part of the arithmetic.  (Split sizes chosen for a
+// batch's draft step from all its sequences balance the items over the CTAs better, 0.6 % of a block of eight ragged sequences
+// of 7B, but then a sequence's draft depends on its batch mates.)
+__device__ __noinline__ void pass_items(PassRows *r, int H) {
   int item0 = 0, part0 = 0;
   for (int i = 0; i < r->nseq; ++i) {
     const int nkeys = r->s_pos0[i] + r->s_rows[i];
-    if (choose) r->s_chunk[i] = chunk;
     r->s_nsp[i] = min(kPassMaxSplits, (nkeys + r->s_chunk[i] - 1) / r->s_chunk[i]);
     r->s_item0[i] = item0; r->s_part0[i] = part0;
     item0 += H * r->s_nsp[i];
@@ -679,7 +664,7 @@ __device__ __noinline__ int await_length(uint64_t *step_bar, unsigned &decisions
 // Rows of draft step `step` (Eq. 2; one thread).  Step 0: the catch-up rows p = p0 .. j - 1 of every sequence, row p pairs
 // the target feature of p with the embedding of token p + 1, a sequence's last row feeds the LM head.  Step s >= 1: one row per
 // sequence with n > s at position j + s - 1, its token the newest draft token.
-__device__ __noinline__ void draft_rows_of_step(PassRows *r, const PassParams &p, int step, int ncta) {
+__device__ __noinline__ void draft_rows_of_step(PassRows *r, const PassParams &p, int step) {
   int T = 0, ns = 0;
   for (int b = 0; b < p.B; ++b) {
     if (r->n[b] <= step) continue;
@@ -695,12 +680,12 @@ __device__ __noinline__ void draft_rows_of_step(PassRows *r, const PassParams &p
     ++ns;
   }
   r->T = T; r->lmT = ns; r->nseq = ns; r->TP = (T + 7) & ~7;
-  pass_items(r, p.H, ncta, p.B > 1);
+  pass_items(r, p.H);
 }
 
 // Rows of a target pass (Eq. 1; one warp): the pending token of every sequence that takes part, then its draft, positions
 // j .. j + n.  A sequence that is full takes no further step.
-__device__ __noinline__ void verify_rows(PassRows *r, const PassParams &p, int ncta, bool record) {
+__device__ __noinline__ void verify_rows(PassRows *r, const PassParams &p, bool record) {
   const int lane = threadIdx.x & 31;
   int R = 0, j = 0, chunk = 0;
   if (lane < p.B && (p.only_seq < 0 || lane == p.only_seq)) {
@@ -733,7 +718,7 @@ __device__ __noinline__ void verify_rows(PassRows *r, const PassParams &p, int n
   }
   if (lane == 0) {
     r->T = r->lmT = T; r->TP = (T + 7) & ~7; r->nseq = ns;
-    pass_items(r, p.H, ncta, false);
+    pass_items(r, p.H);
   }
 }
 
@@ -879,10 +864,10 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
       if (lane == 0) {
         rows->T = T; rows->TP = (T + 7) & ~7; rows->nseq = (T + 15) >> 4;
         rows->lmT = 1; rows->lm_row[0] = T - 1; rows->lm_out[0] = 0;
-        pass_items(rows, p.H, ncta, true);
+        pass_items(rows, p.H);
       }
     } else if (p.mode == 0) {
-      verify_rows(rows, p, ncta, cta == 0);
+      verify_rows(rows, p, cta == 0);
     } else {
       if (lane < p.B) {
         const SeqState q = p.st[lane];
@@ -894,7 +879,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
         rows->cur[lane] = first_step > 0 ? __ldcg(p.tok_out + lane * p.nmax + first_step - 1) : 0;
       }
       __syncwarp();
-      if (lane == 0) draft_rows_of_step(rows, p, first_step, ncta);
+      if (lane == 0) draft_rows_of_step(rows, p, first_step);
     }
   }
   tc_fence_before();
@@ -1924,7 +1909,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
       } else if (p.ddd_thr < 0.f) {
         rows->cum = (step == 0 ? 0.f : rows->cum) + rows->lp;
       }
-      if (p.ddd_thr < 0.f ? made < n : made < nstep) draft_rows_of_step(rows, p, made, ncta);
+      if (p.ddd_thr < 0.f ? made < n : made < nstep) draft_rows_of_step(rows, p, made);
       else if (cta == 0) {   // the draft is complete
         for (int b = 0; b < p.B; ++b)
           if (rows->n[b] > 0 && p.step0 == 0) {

@@ -114,3 +114,33 @@ def test_small_models_on_part_of_the_chip(vocab):
         assert e.ada_get_counters()["status"] == 0
     finally:
         e.close()
+
+
+@pytest.mark.parametrize("batch", [1, 3, 6])
+def test_drafts_do_not_depend_on_batch_mates(batch):
+    """A sequence's drafts and draft features bit for bit beside short and beside long sequences (three sequences: every step in
+    the persistent pass, and the same bits as alone; six: the first step on the multi-row path), and whatever the length of
+    the draft that they belong to.  Sixteen heads: the items of the long batch are more than the thread blocks."""
+    from paper_2412_18910_b200 import Engine
+    sh = si.scaled(si.SHAPES["tiny"], d_model=1024, n_heads=16, d_ffn=1408)
+    w = si.make_weights(sh)
+    prompt = si.uniform_ids(31, "mates", 300, sh.vocab)
+
+    def draft(B, mate_len, n):
+        e = Engine(sh, w, max_batch=B, kv_capacity=512)
+        try:
+            for b in range(B):
+                e.prefill(b, prompt if b == 0 else si.uniform_ids(32 + b, "mate", mate_len, sh.vocab))
+            e.d_n.fill_(sh.n_max)
+            e.d_n[0] = n
+            e.ada_draft(e.d_n, e.d_draft)
+            f = e.ada_debug_buffer(4, torch.float32, (B, sh.n_max, sh.d_model))[0, :n].clone()
+            assert e.ada_get_counters()["status"] == 0
+            return e.d_draft[0, :n].clone(), f
+        finally:
+            e.close()
+
+    tokens, feats = draft(1 if batch == 3 else batch, 20, sh.n_max)
+    for mate_len, n in ((20, sh.n_max), (450, sh.n_max), (450, 3)):
+        t, f = draft(batch, mate_len, n)
+        assert torch.equal(t, tokens[:n]) and torch.equal(f, feats[:n]), (mate_len, n)
