@@ -125,10 +125,10 @@ int ada_label(ada_ctx *ctx, int32_t *d_k);
  * the target's own continuation).  For j = j0 .. j0 + count - 1, with token j of sequence `seq` taken as the pending
  * token and tokens 0..j as the committed prefix, the draft head drafts n_max tokens (fewer at the end of the cache), the
  * target verifies them, and d_k[j - j0] receives the accepted length; d_drafts [count][n_max] and d_targets
- * [count][n_max+1] (optional) receive the drafts and the target's choices, -1 past the draft length.  The positions
- * run one after another, last first, each through the draft and verify kernels of the decode iteration; afterwards
- * the cache rows and features from j0 on are recomputed from the committed tokens (multi-row chunks), so the sequence
- * continues exactly as if the call had not been made.  1 <= j0, j0 + count - 1 <= index of the pending token; the
+ * [count][n_max+1] (optional) receive the drafts and the target's choices, -1 past the draft length.  Up to eight
+ * positions are drafted and verified together, in cache pages that the sequence does not use yet; where the cache is
+ * too full for that, and with teacher forcing, they run one by one in the sequence's own pages, whose rows are kept
+ * aside and put back.  The sequences continue exactly as if the call had not been made.  1 <= j0, j0 + count - 1 <= index of the pending token; the
  * draft head must be up to date (the sequence was decoded with drafts): ADA_ERR_STATE otherwise.  Teacher forcing
  * (ada_force_draft) applies as in ada_label.  This call reads the sequence's length from the device: it synchronises
  * the stream once before it enqueues. */

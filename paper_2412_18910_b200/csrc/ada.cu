@@ -84,6 +84,8 @@ struct ada_ctx {
   SeqState *lb_st;
   int *lb_pages, *lb_draft, *lb_target;
   float *lb_dfeat;
+  bf16 *lb_rows;                      // rows of a sequence kept aside while a start position's passes run in its own pages
+  float *lb_feat;
   float2 *lb_top;
   float4 *amax2;
   unsigned *gbar;
@@ -325,6 +327,8 @@ size_t carve(ada_ctx *x, const ada_config *c, char *base) {
   x->lb_target = w.take<int>(kMaxBatch * (c->n_max + 1));
   x->lb_dfeat = w.take<float>((size_t)kMaxBatch * c->n_max * d);
   x->lb_top = w.take<float2>(kMaxBatch * (c->n_max + 1) + 1);
+  x->lb_rows = w.take<bf16>(((c->n_max + 1) * L + 2 * c->n_max + 1) * 2 * d);
+  x->lb_feat = w.take<float>((c->n_max + 1) * d);
   x->out_acc = w.take<int>(B);
   x->out_emit = w.take<int>(B * (c->n_max + 1));
   x->out_nemit = w.take<int>(B);
@@ -777,7 +781,8 @@ void enqueue_verify(ada_ctx *x, int only_seq, float *d_logits, bool accept = fal
 int enqueue_labels(ada_ctx *x, int seq, int j0, int count, const SeqState &s0, int *d_k, int *d_drafts, int *d_targets) {
   const ada_config &c = x->c;
   if (x->force_draft) return 0;   // (forced drafts belong to the sequence itself)
-  const int ps = c.page_size, unused = x->pages_per_seq - ((s0.len - 1) / ps + 1);
+  // (the rows of a verify that is not accepted yet reach up to n_max positions past the pending one)
+  const int ps = c.page_size, unused = std::max(0, x->pages_per_seq - ((s0.len - 1 + c.n_max) / ps + 1));
   const int most = std::min(kMaxBatch, kTcRows / (c.n_max + 1));
   int done = 0;
   while (done < count) {
@@ -825,34 +830,32 @@ int enqueue_labels(ada_ctx *x, int seq, int j0, int count, const SeqState &s0, i
   return done;
 }
 
-// Multi-row passes over committed positions of one sequence: the target over positions [p_begin, p_end) (cache rows and
-// features), the draft head over those of them below d_end (each needs the token after its position), in equal chunks of
-// at most kMaxRows rows.  with_choice: the greedy choice after position p_end - 1 goes to chunk_tok.  chunk: the sequence's
-// attention split size.
-void enqueue_chunks(ada_ctx *x, int seq, int p_begin, int p_end, int d_end, bool with_choice, int chunk) {
+// The prompt of a sequence, m tokens: the target over all of them (cache rows and features; the greedy choice after the last
+// goes to chunk_tok), the draft head over all but the last (each needs the token after its position), in equal chunks of at
+// most kMaxRows rows.  chunk: the sequence's attention split size.
+void enqueue_prompt(ada_ctx *x, int seq, int m, int chunk) {
   const ada_config &c = x->c;
-  const int TM0 = x->TM, total = p_end - p_begin, chunks = (total + kMaxRows - 1) / kMaxRows;
+  const int TM0 = x->TM, chunks = (m + kMaxRows - 1) / kMaxRows;
   x->prompt_seq = seq;
-  if (total <= kPassRowsMax && x->pass_ok) {   // few rows: a persistent pass each for the target and the draft head
-    LAUNCH(x, k_rows_chunk, 1, 256, 0, x->pass, x->tok, c.kv_capacity, seq, p_begin, total, 0, x->B, chunk);
+  if (m <= kPassRowsMax && x->pass_ok) {   // few rows: a persistent pass each for the target and the draft head
+    LAUNCH(x, k_rows_chunk, 1, 256, 0, x->pass, x->tok, c.kv_capacity, seq, 0, m, 0, x->B, chunk);
     run_pass(x, 0, 0, nullptr, x->chunk_tok, x->vtop + x->B * (c.n_max + 1), nullptr, 1);
-    const int Rd = std::min(p_end, d_end) - p_begin;
-    if (Rd > 0) {
-      LAUNCH(x, k_rows_chunk, 1, 256, 0, x->pass, x->tok, c.kv_capacity, seq, p_begin, Rd, 1, x->B, chunk);
+    if (m > 1) {
+      LAUNCH(x, k_rows_chunk, 1, 256, 0, x->pass, x->tok, c.kv_capacity, seq, 0, m - 1, 1, x->B, chunk);
       run_pass(x, 1, 0, nullptr, nullptr, nullptr, nullptr, 1);
     }
     x->prompt_seq = -1;
     return;
   }
   for (int i = 0; i < chunks; ++i) {
-    const int p0 = p_begin + (int)((long long)total * i / chunks), R = p_begin + (int)((long long)total * (i + 1) / chunks) - p0;
+    const int p0 = (int)((long long)m * i / chunks), R = (int)((long long)m * (i + 1) / chunks) - p0;
     x->TM = R;
     x->prompt_pos0 = p0;
     LAUNCH(x, k_rows_chunk, 1, 256, 0, x->pass, x->tok, c.kv_capacity, seq, p0, R, 0, x->B, chunk);
     target_rows(x);
-    if (i + 1 == chunks && with_choice)   // greedy choice after the last position
+    if (i + 1 == chunks)   // greedy choice after the last position
       lm_head(x, x->xhi, x->xlo, 1, x->chunk_tok, x->vtop + x->B * (c.n_max + 1), nullptr, nullptr);
-    const int Rd = (p0 + R <= d_end) ? R : (d_end - p0);
+    const int Rd = i + 1 < chunks ? R : R - 1;
     if (Rd > 0) {
       x->TM = Rd;
       LAUNCH(x, k_rows_chunk, 1, 256, 0, x->pass, x->tok, c.kv_capacity, seq, p0, Rd, 1, x->B, chunk);
@@ -1072,7 +1075,7 @@ extern "C" int ada_prefill(ada_ctx *x, int seq, const int32_t *d_prompt, int32_t
   if (m + c.n_max + 2 > c.kv_capacity) return fail(x, ADA_ERR_KV_FULL, "ada_prefill: prompt does not fit the cache");
   LAUNCH(x, k_copy_prompt, 8, 256, 0, x->tok, c.kv_capacity, seq, d_prompt, m);
   const int chunk = attn_chunk_for_prompt(m, c.kv_capacity, c.n_heads);   // attention split size of this sequence from now on
-  enqueue_chunks(x, seq, 0, m, m - 1, true, chunk);
+  enqueue_prompt(x, seq, m, chunk);
   LAUNCH(x, k_finish_prefill, 1, 32, 0, x->st, x->tok, c.kv_capacity, seq, m, chunk, x->chunk_tok, d_first_token);
   return finish(x, "ada_prefill");
 }
@@ -1124,21 +1127,31 @@ extern "C" int ada_label_positions(ada_ctx *x, int seq, int32_t j0, int32_t coun
     return fail(x, ADA_ERR_STATE, "ada_label_positions: the draft head is behind the sequence (it was decoded without drafts)");
   const int packed = enqueue_labels(x, seq, j0, count, s0, d_k, d_drafts, d_targets);
   if (packed == count) return finish(x, "ada_label_positions");
-  // What did not fit beside the sequence, one by one in its own pages, start positions from the last to the first: the passes of position j write cache rows and features at positions
-  // >= j only (draft head: >= j - 1, that row from true inputs), which no earlier start position reads.
-  for (int j = j0 + count - 1; j >= j0 + packed; --j) {
-    const int dl = s0.dlen < j - 1 ? s0.dlen : j - 1;
+  // What did not fit beside the sequence, one by one in its own pages.  The rows and features that a start position's passes
+  // write are kept aside and put back, and so are all states; drafts and choices go to buffers of their own.
+  auto swap_out = [&] { std::swap(x->draft, x->lb_draft); std::swap(x->target, x->lb_target); std::swap(x->dfeat, x->lb_dfeat); };
+  float2 *const dtop0 = x->dtop, *const vtop0 = x->vtop;
+  swap_out();
+  x->dtop = x->vtop = x->lb_top;
+  cudaMemcpyAsync(x->lb_st, x->st, sizeof(SeqState) * x->B, cudaMemcpyDeviceToDevice, x->stream);
+  for (int j = j0 + packed; j < j0 + count; ++j) {
+    const int dl = s0.dlen < j - 1 ? s0.dlen : j - 1, n = std::max(0, std::min(c.n_max, c.kv_capacity - j - 2));
+    const LabelRows keep{j, n + 1, dl, j - dl + n, c.n_layers, c.n_heads, c.head_dim, x->page_table + (size_t)seq * x->pages_per_seq,
+                         x->tk, x->tv, x->dk, x->dv, x->lb_rows, x->feat + (size_t)seq * c.kv_capacity * c.d_model, x->lb_feat};
+    const dim3 g(std::max(keep.nt, keep.nd), c.n_layers + 1);
+    LAUNCH(x, k_label_rows, g, 128, 0, keep, 0);
     LAUNCH(x, k_label_begin, 1, 32, 0, x->st, seq, x->B, j + 1, dl, c.n_max, c.kv_capacity);
     enqueue_draft(x);
     enqueue_verify(x, seq, nullptr);
     const int i = j - j0;
-    LAUNCH(x, k_label_one, 1, 32, 0, x->st, x->draft, x->target, c.n_max, seq, d_k + i,
+    LAUNCH(x, k_label_many, 1, 32, 0, x->st + seq, x->draft + seq * c.n_max, x->target + seq * (c.n_max + 1), c.n_max, d_k + i,
            d_drafts ? d_drafts + (size_t)i * c.n_max : (int *)nullptr,
            d_targets ? d_targets + (size_t)i * (c.n_max + 1) : (int *)nullptr);
+    LAUNCH(x, k_label_rows, g, 128, 0, keep, 1);
   }
-  // the sequence's own state again: cache rows and features from the first start position on, from the committed tokens
-  LAUNCH(x, k_label_end, 1, 32, 0, x->st, seq, s0.len, s0.dlen, s0.n, s0.j_prev);
-  enqueue_chunks(x, seq, j0 + packed, s0.len - 1, s0.dlen, false, s0.chunk);
+  cudaMemcpyAsync(x->st, x->lb_st, sizeof(SeqState) * x->B, cudaMemcpyDeviceToDevice, x->stream);
+  swap_out();
+  x->dtop = dtop0; x->vtop = vtop0;
   return finish(x, "ada_label_positions");
 }
 

@@ -666,29 +666,36 @@ __global__ void k_label_begin(SeqState *st, int seq, int B, int len_j, int dlen_
   st[b].j_prev = -1;
   st[b].n = max(0, min(nmax, cap - len_j - 1));
 }
-// ... the label of that start position (and, optionally, the drafts and the target's choices it came from) ...
-__global__ void k_label_one(const SeqState *st, const int *draft, const int *target, int nmax, int seq, int *k_out,
-                            int *draft_out, int *target_out) {
-  if (threadIdx.x != 0) return;
-  const int n = st[seq].n;
-  int k = 0;
-  while (k < n && draft[seq * nmax + k] == target[seq * (nmax + 1) + k]) ++k;
-  *k_out = k;
-  for (int i = 0; i < nmax; ++i) {
-    if (draft_out) draft_out[i] = i < n ? draft[seq * nmax + i] : -1;
+// Rows of one sequence that the passes of a start position write, kept aside (restore = 0) and put back (1): cache rows and
+// features of positions t0 .. t0 + nt - 1 of the target, cache rows of positions d0 .. d0 + nd - 1 of the draft head.  Block
+// (row, layer; layer L: the draft head); `rows` holds nt rows per layer, then the draft head's, a row its keys and its values.
+struct LabelRows {
+  int t0, nt, d0, nd, L, H, hd;
+  const int *pages;                      // page table of the sequence
+  __nv_bfloat16 *tk, *tv, *dk, *dv, *rows;
+  float *feat, *feat_rows;               // features of position 0, kept features
+};
+__global__ void __launch_bounds__(128) k_label_rows(const LabelRows a, int restore) {
+  const int r = blockIdx.x, layer = blockIdx.y, d = a.H * a.hd;
+  const bool head = layer == a.L;
+  if (r >= (head ? a.nd : a.nt)) return;
+  const int pos = (head ? a.d0 : a.t0) + r, page = a.pages[pos / kPageSize], slot = pos % kPageSize;
+  const size_t base = head ? (size_t)page * a.H : ((size_t)page * a.L + layer) * a.H;
+  uint4 *kept = reinterpret_cast<uint4 *>(a.rows + ((size_t)layer * a.nt + r) * 2 * d);
+  for (int i = threadIdx.x; i < d / 8; i += 128) {
+    const int hh = 8 * i / a.hd;
+    const size_t o = ((base + hh) * kPageSize + slot) * a.hd + (8 * i - hh * a.hd);
+    uint4 *k = reinterpret_cast<uint4 *>((head ? a.dk : a.tk) + o), *v = reinterpret_cast<uint4 *>((head ? a.dv : a.tv) + o);
+    if (restore) { *k = kept[i]; *v = kept[d / 8 + i]; }
+    else { kept[i] = *k; kept[d / 8 + i] = *v; }
   }
-  for (int i = 0; i <= nmax; ++i) {
-    if (target_out) target_out[i] = i <= n ? target[seq * (nmax + 1) + i] : -1;
+  if (layer == 0) {
+    float *f = a.feat + (size_t)pos * d, *g = a.feat_rows + (size_t)r * d;
+    for (int i = threadIdx.x; i < d; i += 128) {
+      if (restore) f[i] = g[i];
+      else g[i] = f[i];
+    }
   }
-}
-// ... and the sequence's own state back (the cache rows and features past the first start position are recomputed
-// by the caller's chunk passes).
-__global__ void k_label_end(SeqState *st, int seq, int len0, int dlen0, int n0, int j_prev0) {
-  if (threadIdx.x != 0) return;
-  st[seq].len = len0;
-  st[seq].dlen = dlen0;
-  st[seq].n = n0;
-  st[seq].j_prev = j_prev0;
 }
 
 // Label collection, packed: up to kMaxBatch start positions of one sequence as sequences of their own, which share the
