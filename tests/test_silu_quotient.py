@@ -1,5 +1,6 @@
 """The prompt GEMM's silu divides by an approximate reciprocal and adds the quotient's remainder: its bound of 0.51 units in
-the last place, for every reciprocal within the two units that CUDA documents for the fast division."""
+the last place, for every reciprocal within the two units that CUDA documents for the fast division.  (The arithmetic alone, in
+numpy; test_gpu_silu.py runs the device function.)"""
 import numpy as np
 
 
