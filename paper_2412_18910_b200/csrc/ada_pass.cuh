@@ -235,6 +235,10 @@ __device__ __forceinline__ void bulk_g2s_hint(void *dst, const void *src, unsign
                "l"(src), "r"(bytes), "r"(smem_u32(bar)), "l"(pol)
                : "memory");
 }
+// Bulk copies read global memory through the async proxy: what this kernel's ordinary stores have written to it, here or (seen
+// through a barrier) in another thread block, is ordered before the copies that this thread issues afterwards.  One fence a phase
+// and reading thread: 0.2 to 0.5 % of a pass (as much as one by every writer before the barrier).
+__device__ __forceinline__ void fence_global_copies() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
 __device__ __forceinline__ void tma_load_2d(void *dst, const TensorMap128 *map, int x, int y, uint64_t *bar) {
   asm volatile(
       "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
@@ -1159,7 +1163,6 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
     const unsigned bytes = (unsigned)(16 * p.hd * 2);
     const size_t off = ((((size_t)page * p.cache_layers + layer) * p.H + hh) * kPageSize + k0 % kPageSize) * p.hd;
     uint64_t *bar = attn_bar + 2 * cw + (values ? 1 : 0);
-    if (PROMPT) asm volatile("fence.proxy.async;" ::: "memory");   // a prompt's new cache rows come first (as does what follows; 0.4 us a piece)
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // earlier generic accesses to the buffer come first
     mbar_expect_tx(bar, bytes);
     // (a layer's cache rows are read once per pass: evict-first, like the weights)
@@ -1236,6 +1239,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
           }
         }
         grid_barrier(p, epoch, tid, abort_s);
+        if (!is_xprod && lane == 0) fence_global_copies();   // the new cache rows
       }
       if (!is_xprod) {
         // Items (sequence, head, KV split) round-robin over CTAs.  Worker warp w takes the 16-key pieces w, w + 8, ... of the
@@ -1245,7 +1249,8 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
         // pair of halves, so each product is issued twice and the sums are fp32.
         //
         // The phase is bound by latency, so it is a short chain: the first pieces of a CTA's first item are requested during
-        // the QKV phase's epilogue (old keys depend on no phase of this pass), a warp's next keys fly under its softmax and
+        // the QKV phase's epilogue (old keys depend on no phase of this step; those of the draft steps before it lie a fence
+        // back), a warp's next keys fly under its softmax and
         // values and its next values under its scores, the merge over the warps and the merge over the splits are one step
         // each with all loads in flight, and an item that is its head's only split writes the result straight away.
         // Phase per layer, 5 rows, before -> after: small model 10.2 -> 6.6 us (context 100), 7B 13.9 -> 9.5 us (512) and
@@ -1558,6 +1563,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
       // ---- activation producer: the input tiles of this GEMM, one bulk copy per 256-k chunk
       if (s.rows > 0) {
         const int kxb = xbuf_boxes(TP), nx = xbuf_count(TP);      // boxes per buffer, buffers (of this step)
+        if (lane == 0) fence_global_copies();   // the input tiles that the phase before stored
         for (int i = s.c0, c = s.c0 + s.rot; i < s.c1; ++i, c = c + 1 == s.c1 ? s.c0 : c + 1) {
           const int nbox = (min(kKc, g.K - c * kKc) + kBoxK - 1) / kBoxK;
           for (int b0 = 0; b0 < nbox; b0 += kxb) {
@@ -1669,6 +1675,8 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
     const uint32_t sums = tmem_base + ((uint32_t)(quarter * 32) << 16) + kTmemSums + (uint32_t)(mi * TP);
     const int t_end = sw ? 2 * TP : TP;                  // (SwiGLU: the gate rows, then the up rows)
     if (s.nsec > 1 && s.rows > 0) sphase = add_sections(secfull, secempty, sphase, s.nsec, active_warp ? t_end : 0, TP, taddr, place, sums, p.cnt, abort_s);
+    // (the cache rows of the draft steps before this one, under the products)
+    if (kind == PH_QKV && step > first_step && lane == 0) fence_global_copies();
     if (s.rows > 0) {
       mbar_wait(accfull, acc_phase & 1u, p.cnt, abort_s);
       ++acc_phase;
