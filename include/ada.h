@@ -80,11 +80,12 @@ typedef struct {
   const void *ldlp_wr, *ldlp_br; /* ldlp_mode 1: [ldlp_blocks][hid][hid], [ldlp_blocks][hid]; else unused (may be NULL) */
 } ada_weights;
 
-/* Bytes of device workspace (KV pools, feature rows, scratch) ada_init needs for this config;
- * 0 if the config is invalid. */
+/* Bytes of device workspace (KV pools, feature rows, scratch) for this config; 0 if the config is invalid.  The
+ * scratch holds prompt chunks of min(1024, kv_capacity) rows; ada_init also accepts a workspace that has room for
+ * shorter ones only, down to 128 rows, and then reads longer prompts in more chunks (ADA_ERR_WORKSPACE below that). */
 size_t ada_workspace_bytes(const ada_config *cfg);
 
-/* Validates cfg, carves d_workspace (256-byte aligned, >= ada_workspace_bytes) and builds the
+/* Validates cfg, carves d_workspace (256-byte aligned, see ada_workspace_bytes for its size) and builds the
  * rotary table.  cuda_stream is a cudaStream_t (NULL = default stream).
  * A verify pass of at most 48 rows (max_batch * (n_max + 1)) is one persistent kernel and so are all steps
  * of a draft, launched cooperatively in thread-block clusters of two, one CTA per SM; ada_init checks that the
@@ -98,7 +99,7 @@ int ada_init(ada_ctx **out, const ada_config *cfg, const ada_weights *w, void *d
              size_t workspace_bytes, void *cuda_stream);
 
 /* Algorithm 1, first pass (draft length 0): the target reads the m prompt tokens of sequence
- * `seq` (in chunks of up to 128 positions), fills its cache and emits the first new token, which
+ * `seq` (in chunks of up to 1024 positions, see ada_workspace_bytes), fills its cache and emits the first new token, which
  * becomes the pending token; the draft head is brought up to date on prompt positions 0..m-2.  d_first_token (optional)
  * receives that token.  1 <= m, m + n_max + 2 <= kv_capacity. */
 int ada_prefill(ada_ctx *ctx, int seq, const int32_t *d_prompt, int32_t m, int32_t *d_first_token);

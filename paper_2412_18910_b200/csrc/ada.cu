@@ -41,6 +41,7 @@ struct ada_ctx {
   int B, TM;              // batch; rows of the pass being enqueued at most (a decode pass of the multi-kernel path, or a prompt chunk)
   int prompt_seq, prompt_pos0;   // sequence whose prompt chunk is being enqueued (-1: a decode pass), position of its first row
   int pages_per_seq, n_pages;
+  int prompt_rows, max_splits;    // rows of a prompt chunk at most; attention splits of a sequence at most
   std::vector<LayerW> layers;
   LayerW eagle;
   const bf16 *embed, *lm_head, *final_norm, *eagle_fc, *ldlp_w1, *ldlp_b1, *ldlp_w2, *ldlp_b2, *ldlp_wr, *ldlp_br;
@@ -246,13 +247,13 @@ int pair_chunk(int K) { return K < 2048 ? 2 : 4; }
 struct PairPlan { int nb, token_tiles, S; };
 constexpr int kPairs = 74;
 constexpr int kPairSplitRows = 2048;    // S x rows of the partial sums at most (scratch is sized for it)
-PairPlan plan_pair(int T, int weight_tiles, int N, int K, bool may_split) {
+PairPlan plan_pair(int T, int weight_tiles, int N, int K, bool may_split, size_t split_rows) {
   PairPlan best{128, (T + 255) / 256, 1};
   double best_us = 1e30;
   const int kboxes = (K + 63) / 64;
   for (int nb = 32; nb <= 128; nb += 32) {
     const int tt = (T + 2 * nb - 1) / (2 * nb);
-    for (int S = 1; S <= (may_split ? 8 : 1) && S <= kboxes && (S == 1 || S * T <= kPairSplitRows); ++S) {
+    for (int S = 1; S <= (may_split ? 8 : 1) && S <= kboxes && (S == 1 || (S * T <= kPairSplitRows && S * (size_t)T <= split_rows)); ++S) {
       const int items = tt * weight_tiles * S, waves = (items + kPairs - 1) / kPairs;
       const double clk_box = fmax(8.0 * nb, (16384.0 + 256.0 * nb) / 48.0);
       double us = waves * ((double)((kboxes + S - 1) / S) * clk_box / 1900.0 + 2.0);
@@ -263,13 +264,20 @@ PairPlan plan_pair(int T, int weight_tiles, int N, int K, bool may_split) {
   return best;
 }
 
-// Lays the workspace out; with base == nullptr only measures it.
-size_t carve(ada_ctx *x, const ada_config *c, char *base) {
+// Rows of a prompt chunk (and of the row scratch) that an engine asks for; ada_init takes the most, down to 128, that the
+// caller's workspace has room for, so that a workspace of the size asked for when chunks had 128 rows still does.
+int prompt_rows_wanted(const ada_config *c) { return std::max(kTcRowsMax, std::min(kMaxRows, (int)c->kv_capacity)); }
+
+// Lays the workspace out for prompt chunks of up to `rows` rows; with base == nullptr only measures it.
+size_t carve(ada_ctx *x, const ada_config *c, int rows, char *base) {
   Carver w{base, 0};
   const size_t d = c->d_model, F = c->d_ffn, V = c->vocab, L = c->n_layers, H = c->n_heads, hd = c->head_dim;
   const size_t B = c->max_batch, cap = c->kv_capacity, ps = c->page_size;
   const int TM = rows_per_pass(c);
-  const size_t TP = kMaxRows;   // row scratch holds the largest pass of any engine: a prompt chunk
+  const size_t TP = rows;   // row scratch holds the largest pass of any engine: a prompt chunk
+  x->prompt_rows = rows;
+  // attention splits of a sequence at most (attn_chunk_for_prompt: 256 keys and a 32nd of the capacity at least)
+  x->max_splits = (int)std::min<size_t>(kPassMaxSplits, (cap + 255) / 256);
   const size_t pps = cap / ps, pages = pps * B;
   x->B = (int)B; x->TM = TM; x->seq_stride = (int)cap; x->pages_per_seq = (int)pps; x->n_pages = (int)pages;
   x->tk = w.take<bf16>(pages * L * H * ps * hd);
@@ -285,10 +293,11 @@ size_t carve(ada_ctx *x, const ada_config *c, char *base) {
   x->cnt = w.take<Counters>(1);
   x->pass = w.take<Pass>(1);
   x->h = w.take<float>(TP * d);
-  x->qkv = w.take<float>(kPassRowsMax * 3 * d);   // the persistent pass kernel's q, k, v rows
   x->ss_rows = w.take<float>(TP * kSsSegs);
-  x->qrot = w.take<float>(TP * d);
-  x->attn_part = w.take<float>(H * kAttnSplits * (size_t)kTcRows * (hd + 2));
+  // the persistent pass kernel's q, k, v rows and its partial attention results share their space with those of the other kernels
+  x->qrot = x->qkv = w.take<float>(std::max(TP, (size_t)kPassRowsMax * 3) * d);
+  x->attn_part = x->attn_part2 =
+      w.take<float>(H * std::max(kAttnSplits * (size_t)kTcRows, x->max_splits * (size_t)kPassRowsMax) * (hd + 2));
   const size_t ldx = 2 * d, ldx2 = ((F + 63) / 64) * 64 > d ? ((F + 63) / 64) * 64 : d;
   x->ldx = (int)ldx; x->ldx2 = (int)ldx2;
   x->xhi = w.take<bf16>(TP * ldx);
@@ -304,7 +313,8 @@ size_t carve(ada_ctx *x, const ada_config *c, char *base) {
     upd(part_need_tc(EPI_RESID, 1, (int)d, (int)F));
     upd(part_need_tc(EPI_ARGMAX, 1, (int)V, (int)d));
     upd(part_need_tc(EPI_STORE, 1, (int)d, (int)(2 * d)));
-    upd((size_t)kPairSplitRows * d);   // prompt passes: K splits of the GEMMs with d columns
+    // prompt passes on CTA pairs: K splits of the GEMMs with d columns
+    upd((size_t)(rows <= kTcRowsMax ? 0 : rows == prompt_rows_wanted(c) ? kPairSplitRows : rows) * d);
   }
   x->part_floats = pf;
   x->gemm_part = w.take<float>(pf ? pf : 1);
@@ -344,7 +354,6 @@ size_t carve(ada_ctx *x, const ada_config *c, char *base) {
   x->ac = w.take<bf16>(((F + 63) / 64) * (kPassRowsMax * 128));
   x->fc = w.take<bf16>(((2 * d + 63) / 64) * (kPassRowsMax * 128));
   x->ss_part = w.take<float>(kSsStride * kPassRowsMax);
-  x->attn_part2 = w.take<float>(H * kPassMaxSplits * kPassRowsMax * (hd + 2));
   x->attn_cnt = w.take<int>(kMaxBatch * H);
   x->amax2 = w.take<float4>(256 * kPassRowsMax);
   x->gbar = w.take<unsigned>(64);
@@ -390,7 +399,7 @@ bool gemm_prompt(ada_ctx *x, int epi, const bf16 *W0, const bf16 *W1, const bf16
   const int kind = sw ? PAIR_SWIGLU : r.kind == Reduce::QKV_ROPE ? PAIR_QKV : PAIR_PART;
   t.nseg = nseg; t.Nseg = Nseg; t.K = K; t.T = x->TM; t.chunk = pair_chunk(K);
   t.weight_tiles = sw ? (Nseg + 127) / 128 : nseg * ((Nseg + 255) / 256);
-  const PairPlan plan = plan_pair(x->TM, t.weight_tiles, sw ? 2 * Nseg : nseg * Nseg, K, kind == PAIR_PART);
+  const PairPlan plan = plan_pair(x->TM, t.weight_tiles, sw ? 2 * Nseg : nseg * Nseg, K, kind == PAIR_PART, x->part_floats / c.d_model);
   t.nb = plan.nb; t.token_tiles = plan.token_tiles; t.S = plan.S;
   const bf16 *Ws[3] = {W0, W1, W2};
   for (int i = 0; i < 3; ++i)
@@ -635,8 +644,9 @@ bool build_tc_maps(ada_ctx *x, std::vector<TensorMap128> &maps) {
   layer(x->eagle);
   add(x->eagle_fc, d, 2 * d, 128);
   add(x->lm_head, V, d, 128);
-  add(x->xhi, kMaxRows, x->ldx, kTcRows); add(x->xlo, kMaxRows, x->ldx, kTcRows);
-  add(x->x2hi, kMaxRows, x->ldx2, kTcRows); add(x->x2lo, kMaxRows, x->ldx2, kTcRows);
+  const size_t rows = x->prompt_rows;
+  add(x->xhi, rows, x->ldx, kTcRows); add(x->xlo, rows, x->ldx, kTcRows);
+  add(x->x2hi, rows, x->ldx2, kTcRows); add(x->x2lo, rows, x->ldx2, kTcRows);
   // the cache pools as rows of head_dim 16-bit elements, whose chunks are stored swizzled already (attention of prompts)
   auto add_pool = [&](const void *base, size_t rows) {
     ok = ok && next < x->n_tcmaps && encode_map(fn, &maps[next], base, rows, c.head_dim, 64, false);
@@ -654,10 +664,10 @@ bool build_tc_maps(ada_ctx *x, std::vector<TensorMap128> &maps) {
   auto gate_up = [&](const LayerW &a) { add_pair(a.wg, F, d, 64); add_pair(a.wu, F, d, 64); };
   for (int l = 0; l < c.n_layers; ++l) gate_up(x->layers[l]);
   gate_up(x->eagle);
-  for (unsigned box = 32; box <= 128; box += 32) add_pair(x->xhi, kMaxRows, x->ldx, box);
-  for (unsigned box = 32; box <= 128; box += 32) add_pair(x->xlo, kMaxRows, x->ldx, box);
-  for (unsigned box = 32; box <= 128; box += 32) add_pair(x->x2hi, kMaxRows, x->ldx2, box);
-  for (unsigned box = 32; box <= 128; box += 32) add_pair(x->x2lo, kMaxRows, x->ldx2, box);
+  for (unsigned box = 32; box <= 128; box += 32) add_pair(x->xhi, rows, x->ldx, box);
+  for (unsigned box = 32; box <= 128; box += 32) add_pair(x->xlo, rows, x->ldx, box);
+  for (unsigned box = 32; box <= 128; box += 32) add_pair(x->x2hi, rows, x->ldx2, box);
+  for (unsigned box = 32; box <= 128; box += 32) add_pair(x->x2lo, rows, x->ldx2, box);
   return ok;
 }
 
@@ -698,7 +708,7 @@ void run_pass(ada_ctx *x, int mode, int step0, float *logits, int *tok_out, floa
   p.rope = x->rope;
   p.kpool = mode == 0 ? x->tk : x->dk; p.vpool = mode == 0 ? x->tv : x->dv;
   p.page_table = x->page_table; p.pages_per_seq = x->pages_per_seq; p.page_size = c.page_size;
-  p.attn_part = x->attn_part2; p.attn_part_floats = (size_t)c.n_heads * kPassMaxSplits * kPassRowsMax * c.head_dim; p.attn_cnt = x->attn_cnt;
+  p.attn_part = x->attn_part2; p.attn_part_floats = (size_t)c.n_heads * x->max_splits * kPassRowsMax * c.head_dim; p.max_splits = x->max_splits; p.attn_cnt = x->attn_cnt;
   p.amax = x->amax2; p.logits = logits; p.tok_out = tok_out; p.top_out = top_out; p.forced = forced;
   p.gbar = x->gbar; p.cnt = x->cnt;
   p.lp_out = p.ddd_thr < 0.f ? x->dlp : nullptr; p.tok_logit = x->dfl;
@@ -832,10 +842,10 @@ int enqueue_labels(ada_ctx *x, int seq, int j0, int count, const SeqState &s0, i
 
 // The prompt of a sequence, m tokens: the target over all of them (cache rows and features; the greedy choice after the last
 // goes to chunk_tok), the draft head over all but the last (each needs the token after its position), in equal chunks of at
-// most kMaxRows rows.  chunk: the sequence's attention split size.
+// most prompt_rows rows.  chunk: the sequence's attention split size.
 void enqueue_prompt(ada_ctx *x, int seq, int m, int chunk) {
   const ada_config &c = x->c;
-  const int TM0 = x->TM, chunks = (m + kMaxRows - 1) / kMaxRows;
+  const int TM0 = x->TM, chunks = (m + x->prompt_rows - 1) / x->prompt_rows;
   x->prompt_seq = seq;
   if (m <= kPassRowsMax && x->pass_ok) {   // few rows: a persistent pass each for the target and the draft head
     LAUNCH(x, k_rows_chunk, 1, 256, 0, x->pass, x->tok, c.kv_capacity, seq, 0, m, 0, x->B, chunk);
@@ -889,7 +899,7 @@ int finish(ada_ctx *x, const char *what) {
 extern "C" size_t ada_workspace_bytes(const ada_config *cfg) {
   if (!config_ok(cfg)) return 0;
   ada_ctx tmp;
-  return carve(&tmp, cfg, nullptr);
+  return carve(&tmp, cfg, prompt_rows_wanted(cfg), nullptr);
 }
 
 extern "C" int ada_init(ada_ctx **out, const ada_config *cfg, const ada_weights *w, void *d_workspace,
@@ -912,8 +922,9 @@ extern "C" int ada_init(ada_ctx **out, const ada_config *cfg, const ada_weights 
   ada_ctx *x = new ada_ctx();
   x->c = *cfg;
   x->stream = (cudaStream_t)cuda_stream;
-  const size_t need = carve(x, cfg, (char *)d_workspace);
-  if (workspace_bytes < need) {
+  int rows = prompt_rows_wanted(cfg);
+  while (rows > kTcRowsMax && carve(x, cfg, rows, nullptr) > workspace_bytes) rows = (rows - 1) / kTcRowsMax * kTcRowsMax;
+  if (carve(x, cfg, rows, (char *)d_workspace) > workspace_bytes) {
     delete x;
     return ADA_ERR_WORKSPACE;
   }
@@ -969,10 +980,10 @@ extern "C" int ada_init(ada_ctx **out, const ada_config *cfg, const ada_weights 
   if (e == cudaSuccess) e = cudaMemsetAsync(x->target, 0, sizeof(int) * x->B * (cfg->n_max + 1), x->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(x->force_n_dev, 0, sizeof(int) * x->B, x->stream);
   // activation staging rows beyond the live ones are read by the tensor-core tiles: keep them finite
-  if (e == cudaSuccess) e = cudaMemsetAsync(x->xhi, 0, sizeof(bf16) * (size_t)kMaxRows * x->ldx, x->stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(x->xlo, 0, sizeof(bf16) * (size_t)kMaxRows * x->ldx, x->stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(x->x2hi, 0, sizeof(bf16) * (size_t)kMaxRows * x->ldx2, x->stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(x->x2lo, 0, sizeof(bf16) * (size_t)kMaxRows * x->ldx2, x->stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(x->xhi, 0, sizeof(bf16) * (size_t)x->prompt_rows * x->ldx, x->stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(x->xlo, 0, sizeof(bf16) * (size_t)x->prompt_rows * x->ldx, x->stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(x->x2hi, 0, sizeof(bf16) * (size_t)x->prompt_rows * x->ldx2, x->stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(x->x2lo, 0, sizeof(bf16) * (size_t)x->prompt_rows * x->ldx2, x->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(x->stream);  // host vectors go out of scope
   // Persistent pass kernel: decode passes of at most 48 rows (all sequences of the engine at n_max + 1 rows each).  Measured
   // against the multi-row path, 7B verify: 15 rows 2.83 against 3.79 ms, 24 rows 3.02, 32 rows 3.26, 40 rows 3.72 against

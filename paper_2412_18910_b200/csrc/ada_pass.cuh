@@ -156,6 +156,7 @@ struct PassParams {
   __nv_bfloat16 *kpool, *vpool;
   const int *page_table; int pages_per_seq, page_size;
   float *attn_part;            // partial results per (sequence, head, split) and row of the sequence: [rows][hd] sums, then [rows] (m, l)
+  int max_splits;              // attention splits of a sequence at most
   size_t attn_part_floats;     // where the (m, l) pairs start
   int *attn_cnt;               // [sequences][H] arrival counters (zero between passes)
   // LM head
@@ -643,11 +644,11 @@ __device__ __forceinline__ void stamp(const PassParams &p, int ph, int k, bool o
 // pass and whatever the sequences beside it: the split a key falls in is part of the arithmetic.  (Split sizes chosen for a
 // batch's draft step from all its sequences balance the items over the CTAs better, 0.6 % of a block of eight ragged sequences
 // of 7B, but then a sequence's draft depends on its batch mates.)
-__device__ __noinline__ void pass_items(PassRows *r, int H) {
+__device__ __noinline__ void pass_items(PassRows *r, int H, int max_splits) {
   int item0 = 0, part0 = 0;
   for (int i = 0; i < r->nseq; ++i) {
     const int nkeys = r->s_pos0[i] + r->s_rows[i];
-    r->s_nsp[i] = min(kPassMaxSplits, (nkeys + r->s_chunk[i] - 1) / r->s_chunk[i]);
+    r->s_nsp[i] = min(max_splits, (nkeys + r->s_chunk[i] - 1) / r->s_chunk[i]);
     r->s_item0[i] = item0; r->s_part0[i] = part0;
     item0 += H * r->s_nsp[i];
     part0 += H * r->s_nsp[i] * r->s_rows[i];
@@ -684,7 +685,7 @@ __device__ __noinline__ void draft_rows_of_step(PassRows *r, const PassParams &p
     ++ns;
   }
   r->T = T; r->lmT = ns; r->nseq = ns; r->TP = (T + 7) & ~7;
-  pass_items(r, p.H);
+  pass_items(r, p.H, p.max_splits);
 }
 
 // Rows of a target pass (Eq. 1; one warp): the pending token of every sequence that takes part, then its draft, positions
@@ -722,7 +723,7 @@ __device__ __noinline__ void verify_rows(PassRows *r, const PassParams &p, bool 
   }
   if (lane == 0) {
     r->T = r->lmT = T; r->TP = (T + 7) & ~7; r->nseq = ns;
-    pass_items(r, p.H);
+    pass_items(r, p.H, p.max_splits);
   }
 }
 
@@ -868,7 +869,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
       if (lane == 0) {
         rows->T = T; rows->TP = (T + 7) & ~7; rows->nseq = (T + 15) >> 4;
         rows->lmT = 1; rows->lm_row[0] = T - 1; rows->lm_out[0] = 0;
-        pass_items(rows, p.H);
+        pass_items(rows, p.H, p.max_splits);
       }
     } else if (p.mode == 0) {
       verify_rows(rows, p, cta == 0);

@@ -60,3 +60,45 @@ def test_prompt_features_match_the_oracle(model, plen):
         assert e.ada_get_counters()["status"] == 0
     finally:
         e.close()
+
+
+@pytest.mark.parametrize("cap,budget", [(512, 5769216), (1280, 12000000), (64, 3817728)])
+def test_workspaces_of_shorter_chunks(monkeypatch, cap, budget):
+    """Workspaces that hold prompt chunks of 128 rows (of the sizes that the small model asked for when chunks had 128 rows) or of
+    some more: the same features as with all the scratch.  One that holds none is refused."""
+    from paper_2412_18910_b200 import Engine, binding
+    sh = si.SHAPES["tiny"]
+    w = si.make_weights(sh)
+    real = binding.lib()
+
+    class Budget:
+        def __init__(self, nbytes):
+            self.nbytes = nbytes
+
+        def __getattr__(self, name):
+            return (lambda cfg: self.nbytes) if name == "ada_workspace_bytes" else getattr(real, name)
+
+    def features(nbytes):
+        if nbytes:
+            monkeypatch.setattr(binding, "lib", lambda: Budget(nbytes))
+        try:
+            e = Engine(sh, w, max_batch=1, kv_capacity=cap)
+        finally:
+            monkeypatch.setattr(binding, "lib", lambda: real)
+        try:
+            m = cap - sh.n_max - 2
+            first = e.prefill(0, si.uniform_ids(9, "budget", m, sh.vocab))
+            e.step()
+            assert e.ada_get_counters()["status"] == 0
+            return first, e.ada_debug_buffer(0, torch.float32, (1, cap, sh.d_model))[0, :m].double().clone()
+        finally:
+            e.close()
+
+    t0, f0 = features(None)
+    t1, f1 = features(budget)
+    assert t0 == t1
+    # another order of 32-bit sums moves about one cache element in 60 by a unit (2^-11 of the element): as a share of the norm
+    # 2^-11 / sqrt(60), which no layer passes on whole
+    assert float((f1 - f0).norm() / f0.norm()) < 2.0 ** -11 / 60 ** 0.5
+    with pytest.raises(binding.AdaError, match="WORKSPACE"):
+        features(1000000)
