@@ -420,7 +420,7 @@ def main():
     if c1["status"] != 0:     # a device-side error (a wait that gave up, a full cache) invalidates the timing
         raise RuntimeError("device status word %d after the timed region" % c1["status"])
     tokens = c1["n_tokens"] - c0["n_tokens"]
-    launches = c1["kernels"] - c0["kernels"]
+    launches = c1["launches"] - c0["launches"]
     n_draft = c1["n_draft"] - c0["n_draft"]
     n_target = c1["n_target"] - c0["n_target"]
     job_ms, job_tokens = aggregate(dist, total_ms, float(tokens), dev)

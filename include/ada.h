@@ -182,8 +182,8 @@ int ada_force_commit(ada_ctx *ctx, int seq, const int32_t *d_tokens, int32_t cou
 /* Synchronises the stream and returns, summed over sequences:
  * out[0] N_target (verify passes), out[1] N_draft, out[2] N_waste, out[3] tokens emitted
  * (Table 2's counters), out[4] device status word (0 = no device-side error),
- * out[5] kernels launched by this context so far, where the one launch that runs all draft steps counts
- * as the launches of each step it stands for, out[6] kernels launched as they are, out[7] 0. */
+ * out[5] kernels launched by this context so far (a launch that runs all draft steps is one), out[6] the same,
+ * out[7] 0. */
 int ada_get_counters(ada_ctx *ctx, int64_t out[8]);
 
 /* Clears the device status word (stream-ordered).  After a device-side error (out[4] of ada_get_counters non-zero)

@@ -92,10 +92,9 @@ struct ada_ctx {
   unsigned *gbar;
   unsigned long long *phase_ns;
   // bookkeeping
-  long long launches;               // kernel launches, the persistent draft launch counted as the steps it stands for
-  long long kernels;                // kernel launches as they are
+  long long launches;               // kernel launches
   cudaGraphExec_t graph;
-  int graph_launches, graph_kernels;
+  int graph_launches;
   int graph_key;                    // configuration the graph was captured for
   int *out_acc, *out_emit, *out_nemit, *out_nused;   // internal outputs of ada_step
   // per-kernel timing for roofline reports (off by default): event pairs around GEMM / attention launches
@@ -120,7 +119,6 @@ int fail(ada_ctx *ctx, int code, const char *msg) {
   do {                                                                      \
     kernel<<<grid, block, smem, (ctx)->stream>>>(__VA_ARGS__);              \
     (ctx)->launches++;                                                      \
-    (ctx)->kernels++;                                                       \
   } while (0)
 
 // Launch with the programmatic-serialization attribute: the kernel may begin while the kernel before it in the stream
@@ -137,7 +135,6 @@ void launch_pdl(ada_ctx *x, void (*kernel)(KArgs...), dim3 grid, dim3 block, siz
   cfg.attrs = at; cfg.numAttrs = 1;
   cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
   x->launches++;
-  x->kernels++;
 }
 
 // The same for a kernel on CTA pairs (clusters of two).
@@ -154,7 +151,6 @@ void launch_pair(ada_ctx *x, void (*kernel)(KArgs...), int pairs, int block, siz
   cfg.attrs = at; cfg.numAttrs = 2;
   cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
   x->launches++;
-  x->kernels++;
 }
 
 // Event pair around the launches made by `body` when profiling is on.
@@ -729,10 +725,7 @@ void run_pass(ada_ctx *x, int mode, int step0, float *logits, int *tok_out, floa
     lc.attrs = at; lc.numAttrs = noncoop ? 1 : 2;
     if (prompt) cudaLaunchKernelEx(&lc, k_pass<true>, p);
     else cudaLaunchKernelEx(&lc, k_pass<false>, p);
-    x->kernels++;
-    // a target pass stands for its row list too (and for accepting), a step of the draft for a row list and a pass, and a
-    // length decision with the stopping rule
-    x->launches += prompt ? 1 : mode == 0 ? 2 + accept : (c.n_max - step0) * (c.ddd_threshold < 0.f ? 3 : 2);
+    x->launches++;
   });
 }
 
@@ -941,7 +934,7 @@ extern "C" int ada_init(ada_ctx **out, const ada_config *cfg, const ada_weights 
   x->ldlp_w1 = (const bf16 *)w->ldlp_w1; x->ldlp_b1 = (const bf16 *)w->ldlp_b1;
   x->ldlp_w2 = (const bf16 *)w->ldlp_w2; x->ldlp_b2 = (const bf16 *)w->ldlp_b2;
   x->ldlp_wr = (const bf16 *)w->ldlp_wr; x->ldlp_br = (const bf16 *)w->ldlp_br;
-  x->force_draft = nullptr; x->has_force_n = 0; x->launches = x->kernels = 0; x->graph = nullptr; x->graph_launches = 0;
+  x->force_draft = nullptr; x->has_force_n = 0; x->launches = 0; x->graph = nullptr; x->graph_launches = 0;
   x->graph_key = -1;
   x->capture_stream = nullptr;
   x->prof = 0; x->ev_used = 0; x->enqueue_failed = 0; x->prompt_seq = -1;
@@ -1201,7 +1194,7 @@ extern "C" int ada_step(ada_ctx *x, int32_t *d_emitted, int32_t *d_n_emitted, in
   const int key = (x->has_force_n ? 1 : 0) | (x->force_draft ? 2 : 0) | (all_ar ? 4 : 0);
   if (!x->graph || x->graph_key != key) {
     if (x->graph) { cudaGraphExecDestroy(x->graph); x->graph = nullptr; }
-    const long long before = x->launches, before_k = x->kernels;
+    const long long before = x->launches;
     cudaGraph_t g = nullptr;
     // record on the private stream (the caller's may be the legacy default stream, which cannot be
     // captured); the graph is then replayed on the caller's stream
@@ -1226,9 +1219,7 @@ extern "C" int ada_step(ada_ctx *x, int32_t *d_emitted, int32_t *d_n_emitted, in
     x->stream = user_stream;
     x->prof = user_prof;
     x->graph_launches = (int)(x->launches - before);
-    x->graph_kernels = (int)(x->kernels - before_k);
     x->launches = before;
-    x->kernels = before_k;
     if (e != cudaSuccess || !g) return fail(x, ADA_ERR_CUDA, "ada_step: stream capture failed");
     e = cudaGraphInstantiate(&x->graph, g, 0);
     cudaGraphDestroy(g);
@@ -1237,7 +1228,6 @@ extern "C" int ada_step(ada_ctx *x, int32_t *d_emitted, int32_t *d_n_emitted, in
   }
   if (cudaGraphLaunch(x->graph, x->stream) != cudaSuccess) return fail(x, ADA_ERR_CUDA, "ada_step: graph launch failed");
   x->launches += x->graph_launches;
-  x->kernels += x->graph_kernels;
   CopyMany out = {{d_emitted, d_n_emitted, d_n_used, d_accept_len},
                   {x->out_emit, x->out_nemit, x->out_nused, x->out_acc},
                   {x->B * (c.n_max + 1), x->B, x->B, x->B}};
@@ -1290,7 +1280,7 @@ extern "C" int ada_get_counters(ada_ctx *x, int64_t out[8]) {
   if (cudaMemcpy(&h, x->cnt, sizeof(h), cudaMemcpyDeviceToHost) != cudaSuccess)
     return fail(x, ADA_ERR_CUDA, "ada_get_counters: copy failed");
   out[0] = (int64_t)h.n_target; out[1] = (int64_t)h.n_draft; out[2] = (int64_t)h.n_waste; out[3] = (int64_t)h.n_tokens;
-  out[4] = h.status; out[5] = x->launches; out[6] = x->kernels; out[7] = 0;
+  out[4] = h.status; out[5] = out[6] = x->launches; out[7] = 0;
   return ADA_OK;
 }
 

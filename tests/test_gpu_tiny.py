@@ -176,7 +176,8 @@ def test_counters_and_launch_count(tiny, eng):
     assert c1["n_draft"] - c0["n_draft"] == tot["n"]
     assert c1["n_waste"] - c0["n_waste"] == tot["n"] - tot["k"]
     assert c1["n_tokens"] - c0["n_tokens"] == tot["e"]
-    assert c1["launches"] > c0["launches"] + 5 * 20
+    # a step: the predictor's two kernels, all draft steps, the verify pass, the copy of the results
+    assert c1["launches"] - c0["launches"] == 5 * 5
     assert c1["status"] == 0
 
 
