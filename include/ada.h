@@ -218,8 +218,8 @@ int ada_debug_buffer(ada_ctx *ctx, int which, void **d_ptr, size_t *bytes);
  * brackets every GEMM launch and every attention launch pair of the separately called steps
  * (not of the ada_step graph) with CUDA events on the context's stream; ada_profile(ctx, 0) stops.
  * ada_get_profile synchronises and returns out[0] GEMM launches, out[1] their summed duration (ms),
- * out[2] the weight bytes they streamed (each weight once per launch), out[3] attention launch
- * pairs, out[4] their summed duration (ms), out[5..7] 0.  At most 4096 launches are recorded. */
+ * out[2] the weight bytes they streamed (each weight once per launch; a launch that runs draft steps: the draft
+ * head's once per step that ran), out[3] attention launch pairs, out[4] their summed duration (ms), out[5..7] 0.  At most 4096 launches are recorded. */
 int ada_profile(ada_ctx *ctx, int enable);
 int ada_get_profile(ada_ctx *ctx, double out[8]);
 

@@ -91,6 +91,7 @@ struct ada_ctx {
   float4 *amax2;
   unsigned *gbar;
   unsigned long long *phase_ns;
+  int *prof_steps;
   // bookkeeping
   long long launches;               // kernel launches
   cudaGraphExec_t graph;
@@ -153,7 +154,10 @@ void launch_pair(ada_ctx *x, void (*kernel)(KArgs...), int pairs, int block, siz
   x->launches++;
 }
 
-// Event pair around the launches made by `body` when profiling is on.
+// Event pair around the launches made by `body` when profiling is on.  cls: 0 GEMM, 1 attention, kProfDraft: a GEMM launch of
+// draft steps, `bytes` for each.
+constexpr int kProfDraft = 2;
+constexpr int kProfRecords = 4096;
 template <typename F>
 void timed(ada_ctx *x, int cls, double bytes, F body) {
   if (!x->prof || x->ev_used + 2 > (int)x->ev_pool.size()) { body(); return; }
@@ -354,6 +358,7 @@ size_t carve(ada_ctx *x, const ada_config *c, int rows, char *base) {
   x->amax2 = w.take<float4>(256 * kPassRowsMax);
   x->gbar = w.take<unsigned>(64);
   x->phase_ns = w.take<unsigned long long>(512 + 4 * 512);
+  x->prof_steps = w.take<int>(kProfRecords);
   return (w.off + 255) & ~(size_t)255;
 }
 
@@ -667,13 +672,14 @@ bool build_tc_maps(ada_ctx *x, std::vector<TensorMap128> &maps) {
   return ok;
 }
 
-// Bytes of weights one pass streams (each once): for the per-launch roofline record.
-double pass_weight_bytes(const ada_ctx *x, int mode) {
+// Bytes of weights one pass, or one draft step, streams (each once): for the per-launch roofline record.  The draft head's pass
+// over a short prompt has no LM head.
+double pass_weight_bytes(const ada_ctx *x, int mode, int prompt) {
   const ada_config &c = x->c;
   const double d = c.d_model, F = c.d_ffn, V = c.vocab;
   const double layer = 4 * d * d + 3 * d * F;
   double p = mode == 0 ? c.n_layers * layer : 2 * d * d + layer;
-  p += V * d;
+  if (mode == 0 || !prompt) p += V * d;
   return 2.0 * p;
 }
 
@@ -709,7 +715,10 @@ void run_pass(ada_ctx *x, int mode, int step0, float *logits, int *tok_out, floa
   p.gbar = x->gbar; p.cnt = x->cnt;
   p.lp_out = p.ddd_thr < 0.f ? x->dlp : nullptr; p.tok_logit = x->dfl;
   p.phase_ns = (x->prof && mode == 0) ? x->phase_ns : nullptr;
-  timed(x, 0, pass_weight_bytes(x, mode), [&] {
+  // a launch of draft steps streams the head once per step that runs: the kernel leaves their number in the record's place
+  const bool steps = mode == 1 && !prompt;
+  if (x->prof && steps && x->ev_used + 2 <= (int)x->ev_pool.size()) p.steps_out = x->prof_steps + x->ev_used / 2;
+  timed(x, steps ? kProfDraft : 0, pass_weight_bytes(x, mode, prompt), [&] {
     // cooperative (all CTAs resident: they meet at grid barriers) in clusters of two (K-split pairs)
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3(x->n_sm); lc.blockDim = dim3(kPassThreads); lc.dynamicSmemBytes = kPassSmemBytes; lc.stream = x->stream;
@@ -1326,7 +1335,7 @@ extern "C" int ada_debug_buffer(ada_ctx *x, int which, void **d_ptr, size_t *byt
 extern "C" int ada_profile(ada_ctx *x, int enable) {
   if (!x) return ADA_ERR_NULL;
   if (enable && x->ev_pool.empty()) {
-    x->ev_pool.resize(8192);
+    x->ev_pool.resize(2 * kProfRecords);
     for (auto &e : x->ev_pool)
       if (cudaEventCreate(&e) != cudaSuccess) return fail(x, ADA_ERR_CUDA, "ada_profile: cannot create events");
   }
@@ -1340,11 +1349,14 @@ extern "C" int ada_get_profile(ada_ctx *x, double out[8]) {
   if (!x || !out) return ADA_ERR_NULL;
   if (cudaStreamSynchronize(x->stream) != cudaSuccess) return fail(x, ADA_ERR_CUDA, "ada_get_profile: stream error");
   for (int i = 0; i < 8; ++i) out[i] = 0.0;
+  std::vector<int> steps(kProfRecords);
+  if (cudaMemcpy(steps.data(), x->prof_steps, sizeof(int) * kProfRecords, cudaMemcpyDeviceToHost) != cudaSuccess)
+    return fail(x, ADA_ERR_CUDA, "ada_get_profile: copy failed");
   for (const auto &r : x->prof_recs) {
     float ms = 0.f;
     if (cudaEventElapsedTime(&ms, x->ev_pool[r.ev], x->ev_pool[r.ev + 1]) != cudaSuccess) continue;
-    const int o = r.cls == 0 ? 0 : 3;
-    out[o] += 1.0; out[o + 1] += ms; out[o + 2] += r.bytes;
+    const int o = r.cls == 1 ? 3 : 0;
+    out[o] += 1.0; out[o + 1] += ms; out[o + 2] += r.bytes * (r.cls == kProfDraft ? steps[r.ev / 2] : 1);
   }
   return ADA_OK;
 }

@@ -168,6 +168,7 @@ struct PassParams {
   // sync
   unsigned *gbar;              // [0] grid barrier count, [16] CTAs that have left: both zero between launches
   Counters *cnt;
+  int *steps_out;              // optional: the draft steps that the launch ran
   unsigned long long *phase_ns;  // optional [512]: [0] = start, [i+1] = time CTA 0 left barrier i (globaltimer)
 };
 
@@ -811,6 +812,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
     }
   }
   const int first_step = p.mode == 0 || PROMPT ? 0 : p.step0;
+  if (!PROMPT && p.steps_out && nstep <= first_step && cta == 0 && tid == 0) *p.steps_out = 0;
   if (nstep <= first_step) return;
 
   extern __shared__ __align__(128) unsigned char pass_smem[];
@@ -1931,6 +1933,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
     if (p.ddd_thr < 0.f) nstep = rows->n[0];
   }
   }
+  if (!PROMPT && p.steps_out && cta == 0 && tid == 32) *p.steps_out = nstep - first_step;
   // the last CTA to leave clears the barrier count for the next launch (all have passed the last barrier)
   if (tid == 32 && atomicAdd(p.gbar + 16, 1u) == (unsigned)ncta - 1u) {
     p.gbar[0] = 0;

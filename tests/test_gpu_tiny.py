@@ -538,3 +538,28 @@ def test_labels_over_start_positions_match_the_oracle_and_leave_the_state_alone(
         assert e.ada_get_counters()["status"] == 0
     finally:
         e.close()
+
+
+def test_profile_counts_the_bytes_of_the_steps_that_ran(tiny):
+    """ada_get_profile: a draft launch streams the head's weights once per step, the head over a short prompt has no LM head."""
+    from paper_2412_18910_b200 import Engine
+    sh, w, prompt, _ = tiny
+    d, F, V, L = sh.d_model, sh.d_ffn, sh.vocab, sh.n_layers
+    layer = 2 * (4 * d * d + 3 * d * F)
+    e = Engine(sh, w, max_batch=1, kv_capacity=sh.kv_capacity)
+    try:
+        def profiled(f):
+            e.ada_profile(True)
+            f()
+            r = e.ada_get_profile()
+            e.ada_profile(False)
+            return r["gemm_launches"], r["gemm_bytes"]
+
+        ids = torch.as_tensor(prompt[:20], dtype=torch.int32).to(e.dev)
+        assert profiled(lambda: e.ada_prefill(0, ids)) == (2, (L + 1) * layer + 2 * V * d + 4 * d * d)
+        for n in (1, 3, sh.n_max):
+            e.d_n.fill_(n)
+            assert profiled(lambda: e.ada_draft(e.d_n, e.d_draft)) == (1, n * (layer + 4 * d * d + 2 * V * d))
+            assert profiled(lambda: e.ada_verify(e.d_draft, e.d_n, e.d_target)) == (1, L * layer + 2 * V * d)
+    finally:
+        e.close()
