@@ -116,6 +116,7 @@ __global__ void __launch_bounds__(kPaThreads, 1) k_attn_prompt(const AttnPromptA
       for (int t = 0; t < nmax; ++t) {
         const int s = t & 1;
         if (t >= 2) mbar_wait_inline(&empty[s], ((unsigned)(t >> 1) & 1u) ^ 1u, a.cnt, abort_s);
+        if (*abort_s) break;
         const int row = ((a.pages[t] * a.L + a.layer) * a.H + hh) * kPageSize;
         unsigned char *st = stages + s * Sh::kStage;
         mbar_expect_tx(&full[s], (unsigned)Sh::kStage);
@@ -306,6 +307,7 @@ __global__ void __launch_bounds__(kPaThreads, 1) k_attn_prompt(const AttnPromptA
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  await_copies(abort_s);
   if (warp == 9) tmem_dealloc(tmem_base, 512);
 }
 

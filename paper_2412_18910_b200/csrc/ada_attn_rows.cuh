@@ -256,6 +256,7 @@ __global__ void __launch_bounds__(128) k_attn_rows(const Pass *pass, const float
       pp[c] = oo;
       if (c == 0) { pp[HD] = M; pp[HD + 1] = lo; }
     }
+    await_copies(&abort_s);
   }
 }
 

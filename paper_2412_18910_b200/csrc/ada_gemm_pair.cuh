@@ -217,6 +217,7 @@ __global__ void __launch_bounds__(kPairThreads, 1) k_gemm_pair(const GemmPairArg
       }
       for (; kb < kb1; ++kb, ++it) {
         if (it >= nstage) mbar_wait_inline(&empty[slot], ((unsigned)(it / nstage) & 1u) ^ 1u, a.cnts, abort_s);
+        if (*abort_s) break;
         load_w(kb, slot);
         load_x(kb, slot);
         slot = slot + 1 == nstage ? 0 : slot + 1;
@@ -434,6 +435,7 @@ __global__ void __launch_bounds__(kPairThreads, 1) k_gemm_pair(const GemmPairArg
   __syncwarp();
   tc_fence_before();
   __syncthreads();
+  await_copies(abort_s);
   cluster_sync_all();
   tc_fence_after();
   if (warp == 2) tmem_dealloc_pair(tmem_base, 512);

@@ -177,6 +177,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_gemm_tc(const GemmTcArgs a) {
       for (int kb = kb0 + nfirst, i = nfirst; kb < kb1 && !idle; ++kb, ++i) {
         const int s = i % kTcStages;
         mbar_wait(&empty[s], ((unsigned)(i / kTcStages) & 1u) ^ 1u, a.cnts, abort_s);
+        if (*abort_s) break;
         load_weights(kb, s);
         load_planes(kb, s);
       }
@@ -308,6 +309,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_gemm_tc(const GemmTcArgs a) {
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  await_copies(abort_s);
   if (warp == 2) tmem_dealloc(tmem_base, kTcTmemCols);
 }
 

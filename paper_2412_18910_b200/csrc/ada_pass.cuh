@@ -225,6 +225,12 @@ __device__ __forceinline__ void mbar_wait(uint64_t *bar, unsigned parity, Counte
   if (mbar_test(bar, parity)) return;
   mbar_spin(bar, parity, cnt, abort_flag, limit);
 }
+// Where a wait gave up, copies into shared memory (this thread block's, or its peer's sums) may still be under way: the thread
+// block stays for a millisecond, in which they land.  Called once, at a kernel's end.
+__device__ __forceinline__ void await_copies(volatile int *abort_flag) {
+  if (*abort_flag)
+    for (int i = 0; i < 1000; ++i) __nanosleep(1000);
+}
 __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, unsigned bytes, uint64_t *bar) {
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
                    smem_u32(dst)),
@@ -914,7 +920,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
     const int TP0 = *reinterpret_cast<const volatile int *>(&rows->TP);
     unsigned decisions = 0;
     for (int step = first_step; step < nstep || (p.ddd_thr < 0.f && step < await_length(step_bar, decisions, rows, p.cnt, abort_s)); ++step)
-    for (int ph = 0; ph < nphase; ++ph) {
+    for (int ph = 0; ph < nphase && !*abort_s; ++ph) {
       int layer;
       const int kind = phase_kind(p, ph, layer);
       if (!is_gemm(kind)) continue;
@@ -1941,6 +1947,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
   }
   // let warp 2 free the tensor memory once every worker has made its last read
   if (!is_xprod) {
+    await_copies(abort_s);
     tc_fence_before();
     named_bar(5, 32 + kNumCWarps * 32);
   }
@@ -1963,6 +1970,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_wait_selftest(unsigned *gba
   if (mode == 0) {
     if (tid == 0) {
       mbar_wait(&bar, 0u, cnt, &abort_flag, limit);
+      await_copies(&abort_flag);
       result[0] = 1;
     }
   } else if (warp == 1 || warp >= kFirstWorker) {   // the threads that take part in the pass kernel's grid barrier
