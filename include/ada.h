@@ -87,8 +87,8 @@ size_t ada_workspace_bytes(const ada_config *cfg);
 
 /* Validates cfg, carves d_workspace (256-byte aligned, see ada_workspace_bytes for its size) and builds the
  * rotary table.  cuda_stream is a cudaStream_t (NULL = default stream).
- * A verify pass of at most 48 rows (max_batch * (n_max + 1)) is one persistent kernel and so are all steps
- * of a draft, launched cooperatively in thread-block clusters of two, one CTA per SM; ada_init checks that the
+ * A verify pass of at most 48 rows (max_batch * (n_max + 1)) and 128 heads (max_batch * n_heads) is one persistent
+ * kernel and so are all steps of a draft, launched cooperatively in thread-block clusters of two, one CTA per SM; ada_init checks that the
  * whole grid can be resident and uses the multi-kernel path otherwise.  Larger batches take that kernel
  * for the draft steps after the first.  Their other passes and the prompt of every engine run the
  * multi-kernel path with its tensor-core GEMMs, whose weight boxes are 128 rows high: d_model, d_ffn and

@@ -68,7 +68,7 @@ struct ada_ctx {
   size_t part_floats;
   // persistent pass kernel: device copies of the layer pointer tables and its scratch
   int pass_ok, n_sm;   // it can run here: draft steps of one row per sequence go through it
-  int use_pass;        // so do all decode passes (max_batch * (n_max + 1) <= 48)
+  int use_pass;        // so do all decode passes (see pass_takes)
   // tensor-core GEMM of the multi-row path (passes of up to 88 rows): tensor maps of every weight matrix and of
   // the activation planes, found by base pointer
   TensorMap128 *d_tcmaps;
@@ -786,6 +786,17 @@ void enqueue_verify(ada_ctx *x, int only_seq, float *d_logits, bool accept = fal
            (const int *)nullptr, 0, x->out_acc, x->out_emit, x->out_nemit, (int *)nullptr);
 }
 
+// Whether the decode passes of B sequences go through the persistent kernel: at most 48 rows (n_max + 1 a sequence), which is what
+// its shared memory holds, and at most 128 heads in all, for its attention takes one item (head, cache split) per SM at a time.
+// Fixed by the configuration, so that a row's sums do not depend on the pass.  Verify of 7B at context 512, persistent against
+// multi-row path: 3 sequences 24 rows 3.42 against 4.01 ms, 33 rows 3.72 / 4.08; 4 sequences 24 rows 3.55 / 3.97, 44 rows 4.39 / 4.22.
+// Verify and a draft of half length at contexts 100, 512, 2000: 16 layers of 2048 with 32 heads, 4 sequences 1.22 / 1.46, 1.51 /
+// 1.58, 2.02 / 1.73 ms, 5 sequences 1.35 / 1.47, 1.72 / 1.61, 2.34 / 1.85; 8 layers of 4096 with 32 heads, 6 sequences 1.17 / 1.34, 1.37 /
+// 1.42, 2.33 / 1.96 (before batches took this kernel: 1.88); 8 layers of 2048 with 16 heads, 8 sequences 0.67 / 0.80, 0.83 / 0.88, 1.17 / 1.04.
+bool pass_takes(const ada_ctx *x, int B) {
+  return x->pass_ok && B * (x->c.n_max + 1) <= kPassRowsMax && B * x->c.n_heads <= 128;
+}
+
 // Labels of start positions j0 .. j0 + count - 1 of a sequence in packed passes: up to eight start positions at a time are
 // drafted and verified together, each with pages of its own from the sequence's unused ones.  Returns how many positions
 // were done, from j0 on; fewer than `count` where the cache is too full.  One draft and one verify pass for eight positions:
@@ -827,7 +838,7 @@ int enqueue_labels(ada_ctx *x, int seq, int j0, int count, const SeqState &s0, i
     float2 *const dtop0 = x->dtop, *const vtop0 = x->vtop;
     swap_in();
     x->B = pl.G; x->TM = (pl.G * (c.n_max + 1) + 7) / 8 * 8; x->seq_stride = 0;
-    x->use_pass = x->pass_ok && pl.G * (c.n_max + 1) <= kPassRowsMax;
+    x->use_pass = pass_takes(x, pl.G);
     x->tok = tok0 + (size_t)seq * c.kv_capacity; x->feat = feat0 + (size_t)seq * c.kv_capacity * c.d_model;
     x->dtop = x->vtop = x->lb_top;
     enqueue_draft(x);
@@ -987,9 +998,6 @@ extern "C" int ada_init(ada_ctx **out, const ada_config *cfg, const ada_weights 
   if (e == cudaSuccess) e = cudaMemsetAsync(x->x2hi, 0, sizeof(bf16) * (size_t)x->prompt_rows * x->ldx2, x->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(x->x2lo, 0, sizeof(bf16) * (size_t)x->prompt_rows * x->ldx2, x->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(x->stream);  // host vectors go out of scope
-  // Persistent pass kernel: decode passes of at most 48 rows (all sequences of the engine at n_max + 1 rows each).  Measured
-  // against the multi-row path, 7B verify: 15 rows 2.83 against 3.79 ms, 24 rows 3.02, 32 rows 3.26, 40 rows 3.72 against
-  // about 3.8, 44 rows 4.05 against about 4.0; beyond, the activations that every CTA reads outgrow the weights.
   x->use_pass = x->pass_ok = 0;
   if (e == cudaSuccess) {
     int dev = 0, sms = 0, per_sm = 0;
@@ -1023,7 +1031,7 @@ extern "C" int ada_init(ada_ctx **out, const ada_config *cfg, const ada_weights 
     }
     if (e == cudaSuccess && per_sm >= 1 && sms <= 256 && fits && max_clusters >= grid / 2) {
       x->pass_ok = 1;
-      x->use_pass = cfg->max_batch * (cfg->n_max + 1) <= kPassRowsMax;
+      x->use_pass = pass_takes(x, cfg->max_batch);
       x->n_sm = grid;
       std::vector<LayerPtrs> lp(cfg->n_layers);
       for (int l = 0; l < cfg->n_layers; ++l) {
