@@ -345,7 +345,7 @@ size_t carve(ada_ctx *x, const ada_config *c, int rows, char *base) {
   x->out_nused = w.take<int>(B);
   x->d_layers = w.take<LayerPtrs>(L);
   x->d_eagle = w.take<LayerPtrs>(1);
-  x->n_maps = (int)(7 * (L + 1) + 2 + 8);
+  x->n_maps = (int)(7 * (L + 1) + 2);
   x->d_maps = w.take<TensorMap128>(x->n_maps);
   x->n_tcmaps = (int)(9 * (L + 1) + 2 + 4 + 4 + 16);   // weights (gate and up twice), planes of decode passes, cache pools, planes of prompt passes
   x->d_tcmaps = w.take<TensorMap128>(x->n_tcmaps);
@@ -696,11 +696,11 @@ void run_pass(ada_ctx *x, int mode, int step0, float *logits, int *tok_out, floa
   p.layers = mode == 0 ? x->d_layers : x->d_eagle;
   p.maps = x->d_maps;
   p.map_layer0 = mode == 0 ? 0 : 7 * c.n_layers;
-  p.map_fc = 7 * (c.n_layers + 1); p.map_lm = p.map_fc + 1; p.map_planes = p.map_fc + 2;
+  p.map_fc = 7 * (c.n_layers + 1); p.map_lm = p.map_fc + 1;
   p.n_layers = mode == 0 ? c.n_layers : 1;
   p.cache_layers = p.n_layers;
   p.d = c.d_model; p.H = c.n_heads; p.hd = c.head_dim; p.F = c.d_ffn; p.V = c.vocab; p.eps = c.rms_eps;
-  p.embed = x->embed; p.lm_head = x->lm_head; p.final_norm = x->final_norm; p.eagle_fc = x->eagle_fc;
+  p.embed = x->embed; p.final_norm = x->final_norm;
   p.mode = mode; p.prompt = prompt; p.step0 = step0; p.st = x->st; p.B = x->B; p.tok = x->tok; p.tok_stride = x->seq_stride;
   p.draft = x->draft; p.only_seq = only_seq; p.accept = accept; p.acc_out = x->out_acc; p.emit_out = x->out_emit; p.nemit_out = x->out_nemit;
   p.ddd_thr = mode == 1 && x->B == 1 && !prompt ? c.ddd_threshold : 0.f;   // (packed start positions: full-length drafts)

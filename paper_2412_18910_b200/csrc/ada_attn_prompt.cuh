@@ -18,7 +18,7 @@
 // 7B, layer of 1000 rows at positions 1000 .. 1999, before -> after: 245 us on mma.sync (tensor products at 200 TFLOP/s) -> 87 us.
 // What bounds it now is a page's chain, 2.4 us for both tiles: 1.7 us of products (hi and lo parts; 64 keys are a narrow N for
 // queries that are read from shared memory each time) with the softmax in turn.  Scores a page ahead and sums kept in
-// tensor memory filled the tensor pipe and took as long (and hundreds of additions in one accumulator are less exact).
+// tensor memory made 333 tokens of 16 layers of 2048 2.5 % faster, but hundreds of additions in one accumulator are less exact.
 #pragma once
 #include <type_traits>
 

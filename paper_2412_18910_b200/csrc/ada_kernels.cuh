@@ -442,7 +442,7 @@ __global__ void k_set_n(SeqState *st, const int *n_in, int B, int nmax, int cap,
 }
 
 // ---------------------------------------------------------------------------------------------
-// Row lists.  One thread block of one warp; B <= 8, rows <= kMaxRows.
+// Row lists.  One thread block; B <= 8, rows <= kMaxRows.
 //
 // Verify (Eq. 1): rows of sequence b = pending token then its n drafts, positions j..j+n.
 // tok[seq * tok_stride + position]: committed tokens (stride 0: all sequences are start positions of one text).

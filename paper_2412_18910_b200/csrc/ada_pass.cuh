@@ -94,10 +94,8 @@ struct LayerPtrs {
 };
 
 // Tensor maps (CUtensorMap, 128 bytes each) live in a device array, in this order:
-//   7 per target layer (wq wk wv wo w_gate w_up w_down), 7 for the draft head's layer, then
-//   eagle_fc, lm_head, then the activation planes xa_hi xa_lo at_hi at_lo ac_hi ac_lo fc_hi fc_lo.
-// Weight maps: dims {K, N}, box {64, rows of one m tile of that matrix's slabs}; plane maps: dims {K, 16},
-// box {64, 16}; 128-byte swizzle.
+//   7 per target layer (wq wk wv wo w_gate w_up w_down), 7 for the draft head's layer, then eagle_fc, lm_head.
+// Dims {K, N}, box {64, rows of one m tile of that matrix's slabs}, 128-byte swizzle.
 struct alignas(64) TensorMap128 {
   unsigned long long opaque[16];
 };
@@ -117,19 +115,18 @@ struct PassRows {
   float lp, cum;                        // log-probability of the newest token, of the draft (stopping rule)
 };
 enum { MAP_WQ = 0, MAP_WK, MAP_WV, MAP_WO, MAP_WG, MAP_WU, MAP_WD };
-enum { MAPX_XA = 0, MAPX_AT = 2, MAPX_AC = 4, MAPX_FC = 6 };
 
 struct PassParams {
   const Pass *pass;            // prompt: the rows
   const TensorMap128 *maps;    // device array, see above
   int map_layer0;              // index of the first map of this pass's first layer
-  int map_fc, map_lm, map_planes;
+  int map_fc, map_lm;
   const LayerPtrs *layers;     // device array
   int n_layers;                // layers of this pass (target: L, draft head: 1)
   int cache_layers;            // layers in the KV pool (stride)
   int d, H, hd, F, V;
   float eps;
-  const __nv_bfloat16 *embed, *lm_head, *final_norm, *eagle_fc;
+  const __nv_bfloat16 *embed, *final_norm;
   int mode;                    // 0 target pass over the pending tokens and drafts, 1 draft-head steps step0 .. (longest draft length) - 1
   int prompt;                  // 1: the rows of `pass` are a short prompt of one sequence (mode 0: greedy choice after the last
                                // row; mode 1: the draft head over its rows, no LM head)
@@ -143,7 +140,7 @@ struct PassParams {
   float ddd_thr;               // < 0: the draft grows while its running log-probability is at least this (one sequence)
   // activations: fp32 residual stream and qkv; bf16 (hi, lo) planes of every GEMM input
   float *h, *qkv;              // [rows][d], [rows][3d]
-  // each input is stored as tensor-core-ready tiles (see xstore): per 64 k one 4 KB box of 32 rows
+  // each input is stored as tensor-core-ready tiles (see xstore): per 64 k one box of 2 TP rows
   __nv_bfloat16 *xa;              // K = d    h * gain of the norm that follows
   __nv_bfloat16 *at;              // K = d    attention output
   __nv_bfloat16 *ac;              // K = F    SwiGLU output
@@ -231,12 +228,6 @@ __device__ __forceinline__ void await_copies(volatile int *abort_flag) {
   if (*abort_flag)
     for (int i = 0; i < 1000; ++i) __nanosleep(1000);
 }
-__device__ __forceinline__ void bulk_g2s(void *dst, const void *src, unsigned bytes, uint64_t *bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                   smem_u32(dst)),
-               "l"(src), "r"(bytes), "r"(smem_u32(bar))
-               : "memory");
-}
 __device__ __forceinline__ void bulk_g2s_hint(void *dst, const void *src, unsigned bytes, uint64_t *bar, uint64_t pol) {
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;" ::"r"(
                    smem_u32(dst)),
@@ -283,17 +274,12 @@ __device__ __forceinline__ void ldmatrix_x4_trans(uint32_t addr, uint32_t &r0, u
                : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3)
                : "r"(addr));
 }
-// warp-level products on 16-bit halves with fp32 sums (attention): c[16 x 8] += a[16 x 16] b[16 x 8], and k = 8
+// warp-level products on 16-bit halves with fp32 sums (attention): c[16 x 8] += a[16 x 16] b[16 x 8]
 __device__ __forceinline__ void mma_f16_k16(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
                                             uint32_t b1) {
   asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
                : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
                : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
-__device__ __forceinline__ void mma_f16_k8(float *c, uint32_t a0, uint32_t a1, uint32_t b0) {
-  asm volatile("mma.sync.aligned.m16n8k8.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5}, {%6}, {%0,%1,%2,%3};"
-               : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-               : "r"(a0), "r"(a1), "r"(b0));
 }
 // ---- tcgen05 (5th generation tensor cores, accumulators in tensor memory)
 __device__ __forceinline__ void tmem_alloc(uint32_t *smem_slot, uint32_t ncols) {   // whole warp
@@ -509,8 +495,8 @@ __device__ __forceinline__ const __nv_bfloat16 *gain_after(const PassParams &p, 
 // GEMMs with only d output columns (O, down, the draft head's fc) would leave each CTA a slab of ~28
 // rows: the tensor core then spends a whole instruction per 28 x 16 weights and every CTA re-reads the
 // whole activation.  They are cut along K too: the two CTAs of a thread-block cluster share a slab of
-// twice the rows, each takes one half of K (whole 256-k chunks), and the CTA of the second half adds the
-// first half's partial sums, read through distributed shared memory, to its own and runs the epilogue.
+// twice the rows, each takes one half of K (whole 256-k chunks); they exchange their sums through distributed shared memory and
+// each finishes half of the pass rows.
 struct Slab {
   int seg;          // matrix (segment) of this CTA
   int r0, rows;     // rows [r0, r0 + rows) inside that matrix
@@ -1151,7 +1137,6 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
   // ================================================================= activation producer + workers
   const bool is_xprod = warp == 1;
   const int cw = warp - kFirstWorker;      // worker warp index 0..7 (workers only)
-  const int g8 = lane >> 2, q4 = lane & 3;
   const int ntid = is_xprod ? lane : 32 + (tid - kFirstWorker * 32);   // index among the 288 barrier participants
   const int ctid = tid - kFirstWorker * 32;   // index among the 256 worker threads
   unsigned epoch = 0;
@@ -1179,7 +1164,6 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
   };
   unsigned kuses = 0;               // completed phases of the K-split pair barrier
   uint32_t sphase = 0;              // per place of the accumulators the parity of its next section of this phase
-  (void)g8; (void)q4;
 
   for (int step = first_step; step < nstep; ++step) {
   const int T = rows->T, lmT = rows->lmT, TP = rows->TP;

@@ -32,10 +32,21 @@ def test_batches_match_their_sequences(tiny, lengths):
             e.d_n.copy_(n)
             e.ada_draft(e.d_n, e.d_draft)
             drafts = []
+            dfeat = e.ada_debug_buffer(4, torch.float32, (B, sh.n_max, sh.d_model)).cpu().numpy()
+            g_draft = e.d_draft.cpu().numpy()
             for b in range(B):
                 nb = int(n[b])
-                d_o = seqs[b].draft(nb)[0] if nb else np.zeros(0, dtype=np.int32)
-                if nb:   # a sequence's own draft: equal, or a flip inside the oracle's margin (then the oracle's is used)
+                d_o = np.zeros(0, dtype=np.int32)
+                if nb:   # a sequence's own draft: equal, or a flip inside the oracle's margin; then on with the oracle's
+                    d_o, d1, d2 = seqs[b].draft(nb)
+                    f_o = seqs[b].draft_features(nb)
+                    rms = np.sqrt((f_o.astype(np.float64) ** 2).mean(axis=1))
+                    for i in range(nb):
+                        scale = max(1.0, float(rms[i]))
+                        assert np.abs(dfeat[b, i] - f_o[i]).max() < 2e-2 * scale, (it, b, i)
+                        if g_draft[b, i] != d_o[i]:
+                            assert d1[i] - d2[i] <= lockstep.TOKEN_MARGIN * scale, (it, b, i)
+                            break
                     e.d_draft[b, :nb] = torch.from_numpy(np.asarray(d_o, dtype=np.int32)).to(e.dev)
                 drafts.append(d_o)
             e.ada_verify(e.d_draft, e.d_n, e.d_target, logits)

@@ -221,8 +221,7 @@ def test_ragged_batch_matches_per_sequence_oracle(tiny):
 
 
 def test_batch_of_two_with_sixteen_rows_matches_per_sequence_oracle():
-    """max_batch = 2 with n_max = 7: a decode pass has at most 16 rows, as at batch 1, but two sequences: it must take
-    the multi-kernel path (the persistent pass kernel's attention reads one sequence's cache)."""
+    """max_batch = 2 with n_max = 7: a decode pass has at most 16 rows, as at batch 1, but of two sequences."""
     from paper_2412_18910_b200 import Engine
     sh = si.scaled(si.SHAPES["tiny"], n_max=7)
     w = si.make_weights(sh)
