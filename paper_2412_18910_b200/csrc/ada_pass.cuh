@@ -28,8 +28,8 @@
 //   warps 0, 3    weight producers, one thread each: both walk the static schedule of (phase, k chunk,
 //                 k boxes, m tile) stages; warp 0 loads the even stages, warp 3 the odd ones (a single
 //                 thread's mbarrier / TMA issue latency, about 700 cycles per stage, was the limit of the loops)
-//   warp 1        activation producer: per GEMM phase (after the grid barrier that makes its input
-//                 visible) copies the input planes chunk by chunk into shared memory
+//   warp 1        stands for the thread block at the grid barriers, and produces activations: per GEMM phase (after the
+//                 barrier that makes its input visible) copies the input planes chunk by chunk into shared memory
 //   warp 2        one elected thread issues every tcgen05.mma and commit, in schedule order; the warp
 //                 also owns the tensor-memory allocation
 //   warps 4..11   workers: epilogues out of tensor memory (tcgen05.ld: one weight row per thread),
@@ -593,33 +593,29 @@ __device__ __forceinline__ void tile_source(const GemmDesc &g, const Slab &s, in
 
 // ---------------------------------------------------------------------------------- grid barrier
 
-// Warp 1 and the eight worker warps (288 threads) take part; the producers' and the issuer's warps do not.
-__device__ __noinline__ void grid_barrier_body(unsigned *gbar, Counters *cnt, unsigned long long *phase_ns, unsigned epoch, int tid,
-                                              volatile int *abort_flag, unsigned limit = kSpinLimit) {
-  named_bar(2, (kNumXWarps + kNumCWarps) * 32);
-  if (tid == 32) {
-    // arrive with release semantics (the named barrier above ordered the other threads' writes before this
-    // thread; the release makes them visible with the count), poll with acquire loads
-    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(gbar) : "memory");
-    const unsigned target = epoch * gridDim.x;
-    bool ok = false;
-    for (unsigned i = 0; i < limit && !*abort_flag; ++i) {
-      if (ld_acquire(gbar) >= target) { ok = true; break; }
-      if ((i & 63) == 63 && (ld_acquire(reinterpret_cast<const unsigned *>(&cnt->status)) & kStatTimeout)) break;
-      if (i > 4096) __nanosleep(64);   // a barrier normally completes within a few polls
-    }
-    if (!ok) { *abort_flag = 1; atomicOr(&cnt->status, kStatTimeout); }
-    if (phase_ns && blockIdx.x == 0 && epoch < 511) {
-      unsigned long long t;
-      asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-      phase_ns[epoch] = t;
-    }
-  }
-  named_bar(2, (kNumXWarps + kNumCWarps) * 32);
+// Warp 1 and the eight worker warps (288 threads) take part; the producers' and the issuer's warps do not.  Workers announce
+// that their stores are done and later await the release; in between they may do what depends on no other CTA's results of the
+// phase.  Warp 1 stands between them and the other CTAs.
+__device__ __forceinline__ void named_arrive(int id, int threads) {
+  asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
-__device__ __forceinline__ void grid_barrier(const PassParams &p, unsigned &epoch, int tid, volatile int *abort_flag) {
-  ++epoch;
-  grid_barrier_body(p.gbar, p.cnt, p.phase_ns, epoch, tid, abort_flag);
+constexpr int kBarThreads = (kNumXWarps + kNumCWarps) * 32;
+__device__ __forceinline__ void phase_arrive() { named_arrive(2, kBarThreads); }
+__device__ __forceinline__ void phase_await() { named_bar(4, kBarThreads); }
+
+// One thread of the CTA: arrives with release semantics (a named barrier has ordered the other threads' writes before this
+// thread; the release makes them visible with the count), polls with acquire loads until `target` arrivals.
+__device__ __forceinline__ void grid_wait(unsigned *gbar, Counters *cnt, unsigned target, volatile int *abort_flag,
+                                          unsigned limit = kSpinLimit) {
+  asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(gbar) : "memory");
+#pragma unroll 1
+  for (unsigned i = 0; i < limit && !*abort_flag; ++i) {
+    if (ld_acquire(gbar) >= target) return;
+    if ((i & 63) == 63 && (ld_acquire(reinterpret_cast<const unsigned *>(&cnt->status)) & kStatTimeout)) break;
+    if (i > 4096) __nanosleep(64);   // a barrier normally completes within a few polls
+  }
+  *abort_flag = 1;
+  atomicOr(&cnt->status, kStatTimeout);
 }
 
 // optional fine-grained clock of CTA 0's first consumer lane: 4 stamps per phase after the 512 barrier stamps
@@ -1134,19 +1130,97 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
     return;
   }
 
-  // ================================================================= activation producer + workers
-  const bool is_xprod = warp == 1;
-  const int cw = warp - kFirstWorker;      // worker warp index 0..7 (workers only)
-  const int ntid = is_xprod ? lane : 32 + (tid - kFirstWorker * 32);   // index among the 288 barrier participants
+  // ================================================================= grid barriers and activation producer (warp 1)
+  // A small loop of its own: what follows a barrier's last poll is the release of the workers and the first copies of the next
+  // phase's input, whose description was worked out before the barrier.  (As part of the workers' loop over the phases it was
+  // 1950 clocks from the last poll to the first copy, most of them waits for instructions that every phase had to fetch again;
+  // now 850.  Draft of four + its verify: small model 163 + 74.8 -> 148 + 64.7 us, middle model 352 + 783 -> 336 + 735, 7B 612 +
+  // 2825 -> 595 + 2738.)
+  if (warp == 1) {
+    const uint64_t pol_x = l2_policy_evict_last();   // (every CTA reads the same input tiles)
+    uint32_t xused = 0, xphase = 0;                  // buffers used before, parity of their next release
+    unsigned target = 0, epoch = 0;
+    for (int step = first_step; step < nstep; ++step) {
+      const int TP = *reinterpret_cast<const volatile int *>(&rows->TP);
+      const int kxb = xbuf_boxes(TP), nx = xbuf_count(TP);    // boxes per buffer, buffers (of this step)
+      const unsigned xbytes = (unsigned)xbuf_bytes(TP);
+      int xslot = 0;   // (all buffers are free between steps)
+      const __nv_bfloat16 *src = nullptr;
+      int beg = 0, end = 0, b = 0, parts = 0;        // boxes of this CTA's part of K, the next one, copies to make
+      for (int ph = 0; ph < nphase; ++ph) {
+        if (lane == 0 && parts > 0 && !*abort_s) {
+          fence_global_copies();   // the input tiles that the phase before stored
+          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the buffers double as scratch of the workers
+#pragma unroll 1
+          for (int i = parts; i > 0; --i) {
+            if ((xused >> xslot) & 1u) {
+              mbar_wait(&xempty[xslot], (xphase >> xslot) & 1u, p.cnt, abort_s);
+              xphase ^= 1u << xslot;
+            }
+            xused |= 1u << xslot;
+            const unsigned bytes = (unsigned)(min(kxb, end - b) * TP * 256);
+            mbar_expect_tx(&xfull[xslot], bytes);
+            bulk_g2s_hint(xbuf + (size_t)xslot * xbytes, src + (size_t)b * (TP * 128), bytes, &xfull[xslot], pol_x);
+            xslot = xslot + 1 == nx ? 0 : xslot + 1;
+            b += kxb;
+            if (b >= end) b = beg;
+          }
+        }
+        __syncwarp();
+        // the next phase's copies
+        int layer;
+        const int kind = phase_kind(p, ph, layer);
+        parts = 0;
+        if (ph + 1 < nphase) {
+          const int next = phase_kind(p, ph + 1, layer);
+          if (is_gemm(next)) {
+            const GemmDesc &g = gemms[next - PH_FC].g;
+            const Slab &s = gemms[next - PH_FC].s;
+            src = g.xt;
+            beg = s.c0 * (kKc / kBoxK);
+            end = min(s.c1 * (kKc / kBoxK), (g.K + kBoxK - 1) / kBoxK);
+            b = beg + s.rot * (kKc / kBoxK);
+            parts = s.rows > 0 ? (end - beg + kxb - 1) / kxb : 0;
+          }
+        }
+        for (int k = PROMPT && kind == PH_ATTN ? 2 : 1; k > 0; --k) {   // (a prompt's new cache rows have a barrier of their own)
+          target += (unsigned)ncta;
+          named_bar(2, kBarThreads);
+          if (lane == 0) grid_wait(p.gbar, p.cnt, target, abort_s);
+          __syncwarp();
+          named_arrive(4, kBarThreads);
+          ++epoch;
+          if (p.phase_ns && cta == 0 && lane == 0 && epoch < 511) {
+            unsigned long long t;
+            asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+            p.phase_ns[epoch] = t;
+          }
+        }
+      }
+      if (p.mode == 1 && !PROMPT) {   // the next step's rows, and whether there is one
+        named_bar(6, kBarThreads);
+        if (p.ddd_thr < 0.f) nstep = *reinterpret_cast<const volatile int *>(&rows->n[0]);
+      }
+    }
+    if (lane == 0) {
+      if (!PROMPT && p.steps_out && cta == 0) *p.steps_out = nstep - first_step;
+      // the last CTA to leave clears the barrier count for the next launch (all have passed the last barrier)
+      if (atomicAdd(p.gbar + 16, 1u) == (unsigned)ncta - 1u) {
+        p.gbar[0] = 0;
+        p.gbar[16] = 0;
+      }
+    }
+    return;
+  }
+
+  // ================================================================= workers
+  const int cw = warp - kFirstWorker;         // worker warp index 0..7
   const int ctid = tid - kFirstWorker * 32;   // index among the 256 worker threads
-  unsigned epoch = 0;
-  int xslot = 0;                    // activation producer: next buffer, buffers used before, parity of their next release
-  uint32_t xused = 0, xphase = 0;
   unsigned acc_phase = 0;   // GEMM phases of this CTA whose accumulator has been awaited
   unsigned attn_uses = 0;           // completed phases of this warp's two attention barriers
   // Keys and values of a worker warp: 16-key pieces cw, cw + 8, ... of an item's split, one bulk copy each into the warp's
   // own two buffers (a piece is contiguous in its cache page).  No warp waits for another inside an item.
-  __nv_bfloat16 *const wst = reinterpret_cast<__nv_bfloat16 *>(xbuf) + 4 * 16 * 128 + (is_xprod ? 0 : cw) * 2 * 16 * 128;
+  __nv_bfloat16 *const wst = reinterpret_cast<__nv_bfloat16 *>(xbuf) + 4 * 16 * 128 + cw * 2 * 16 * 128;
   int pages = 0;                    // cache pages of the warp's pieces 32 i + lane of the current item
   auto attn_pages = [&](int sq, int kfirst, int kend, int i0) {   // (fetched 32 at a time: no copy waits for a table lookup)
     const int k0 = kfirst + 128 * (i0 + lane);
@@ -1167,7 +1241,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
 
   for (int step = first_step; step < nstep; ++step) {
   const int T = rows->T, lmT = rows->lmT, TP = rows->TP;
-  xslot = 0;   // (all buffers are free between steps)
+  bool arrived = false;             // at a grid barrier whose release has not been awaited
   for (int ph = 0; ph < nphase; ++ph) {
     int layer;
     const int kind = phase_kind(p, ph, layer);
@@ -1176,15 +1250,15 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
     if (kind == PH_EMBED || kind == PH_EAGLE_IN) {
       // EMBED: h = embedding rows, planes = split(h * gain of layer 0), partial sums of squares.
       // EAGLE_IN: planes of [e(token) ; feature] for the draft head's fc.  Column slices per CTA.
-      // Sixteen lanes per pass row, 18 rows at once (row by row, each row waited for its own chain of lookups: 5 rows of the
+      // Sixteen lanes per pass row, 16 rows at once (row by row, each row waited for its own chain of lookups: 5 rows of the
       // small model took 6.6 us here); the row's sum of squares is a fixed shuffle tree over its lanes.
       const int width = kind == PH_EMBED ? p.d : 2 * p.d;
       const int cpc = (((width + ncta - 1) / ncta) + 3) & ~3;
       const int c0 = cta * cpc, c1 = min(width, c0 + cpc);
       const __nv_bfloat16 *gain = p.layers[0].na;
-      const int l16 = ntid & 15;
-      for (int t0 = 0; t0 < T; t0 += (kNumXWarps + kNumCWarps) * 2) {
-        const int t = t0 + (ntid >> 4);
+      const int l16 = ctid & 15;
+      for (int t0 = 0; t0 < T; t0 += kNumCWarps * 2) {
+        const int t = t0 + (ctid >> 4);
         float ss = 0.f;
         if (t < T) {
           const __nv_bfloat16 *e = p.embed + (size_t)rows->tok[t] * p.d;
@@ -1208,14 +1282,16 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
           if (l16 == 0 && t < T) p.ss_part[t * kSsStride + cta] = ss;
         }
       }
-      grid_barrier(p, epoch, tid, abort_s);
+      phase_arrive();
+      arrived = true;
       continue;
     }
 
     // ------------------------------------------------------------- attention
     if (kind == PH_ATTN) {
+      phase_await();
       if (PROMPT) {
-        if (!is_xprod) {
+        {
           const int half = p.hd >> 1, per_row = p.H * half, b = rows->seq[0];
           for (int i = cta * (kNumCWarps * 32) + ctid; i < T * per_row; i += ncta * (kNumCWarps * 32)) {
             const int r = i / per_row, e = i - r * per_row, hh = e / half, c = e - hh * half, pos = rows->pos[r];
@@ -1231,10 +1307,11 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
             p.vpool[base + o1] = kv_store(vb);
           }
         }
-        grid_barrier(p, epoch, tid, abort_s);
-        if (!is_xprod && lane == 0) fence_global_copies();   // the new cache rows
+        phase_arrive();
+        phase_await();
+        if (lane == 0) fence_global_copies();   // the new cache rows
       }
-      if (!is_xprod) {
+      {
         // Items (sequence, head, KV split) round-robin over CTAs.  Worker warp w takes the 16-key pieces w, w + 8, ... of the
         // split for all 16 query rows with mma.sync: scores = q k^T (m16n8k16 per 16 channels, two tiles of 8 keys), online
         // softmax on the accumulator fragments, weighted values (m16n8k16 over the 16 keys per 8 channels).  Cache elements
@@ -1543,7 +1620,8 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
           }
         }
       }
-      grid_barrier(p, epoch, tid, abort_s);
+      phase_arrive();
+      arrived = true;
       continue;
     }
 
@@ -1552,37 +1630,47 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
     const Slab &s = gemms[kind - PH_FC].s;
     const int Tg = g.lm_rows ? lmT : T;
 
-    if (is_xprod) {
-      // ---- activation producer: the input tiles of this GEMM, one bulk copy per 256-k chunk
-      if (s.rows > 0) {
-        const int kxb = xbuf_boxes(TP), nx = xbuf_count(TP);      // boxes per buffer, buffers (of this step)
-        if (lane == 0) fence_global_copies();   // the input tiles that the phase before stored
-        for (int i = s.c0, c = s.c0 + s.rot; i < s.c1; ++i, c = c + 1 == s.c1 ? s.c0 : c + 1) {
-          const int nbox = (min(kKc, g.K - c * kKc) + kBoxK - 1) / kBoxK;
-          for (int b0 = 0; b0 < nbox; b0 += kxb) {
-            if (lane == 0) {
-              if ((xused >> xslot) & 1u) {
-                mbar_wait(&xempty[xslot], (xphase >> xslot) & 1u, p.cnt, abort_s);
-                xphase ^= 1u << xslot;
-              }
-              xused |= 1u << xslot;
-              const unsigned bytes = (unsigned)(min(kxb, nbox - b0) * TP * 256);
-              asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the buffer doubles as attention scratch
-              mbar_expect_tx(&xfull[xslot], bytes);
-              // (every CTA reads the same input tiles: evict-last)
-              bulk_g2s_hint(xbuf + (size_t)xslot * xbuf_bytes(TP), g.xt + (size_t)(c * (kKc / kBoxK) + b0) * (TP * 128), bytes,
-                            &xfull[xslot], l2_policy_evict_last());
-            }
-            __syncwarp();
-            xslot = xslot + 1 == nx ? 0 : xslot + 1;
-          }
-        }
-      }
-      grid_barrier(p, epoch, tid, abort_s);
-      continue;
-    }
+    // ---- the epilogue straight out of tensor memory.  First what needs nothing from the phase before, while the other CTAs
+    // arrive: old residual values are at least one barrier old.
+    const bool has_ss = g.epi == EPI_RESID_H || g.epi == EPI_STORE_H;
+    const bool sw = g.epi == EPI_SWIGLU_ACT;
+    // thread <-> weight row: quarter = warp index mod 4 (the tensor-memory lanes this warp may read),
+    // m tile = worker index / 4 (SWIGLU: the first four workers read both accumulators)
+    const int quarter = warp & 3, mi = sw ? 0 : (cw >> 2);
+    const int rloc = s.m64 ? (lane < 16 ? quarter * 16 + lane : 1 << 20) : quarter * 32 + lane;   // row inside the m tile
+    const bool active_warp = s.rows > 0 && (sw ? cw < 4 : mi < s.mtiles);
+    const int rslab = mi * s.box_rows + rloc;                   // row inside the slab
+    const bool valid = active_warp && rloc < s.box_rows && rslab < s.rows;
+    const int vrow = s.seg * g.Nseg + s.r0 + rslab;             // output column
 
-    // ---- workers: wait for the accumulator, then the epilogue straight out of tensor memory
+    // Epilogue items: (pass row, 32 rows of the slab) for a warp, dealt to all eight workers in turn.  K-split pair: CTA j of
+    // the pair finishes the pass rows j, j + 2, ...
+    const bool pair = s.ks > 1 && s.rows > 0;
+    const int t0 = pair ? s.kj : 0, tstep = pair ? 2 : 1, mine = pair ? (Tg + 1 - s.kj) >> 1 : Tg;
+    const int nseg32 = (s.rows + 31) >> 5, nitem = mine * nseg32;
+    const int col0 = s.seg * g.Nseg + s.r0;                     // output column of slab row 0
+    // the next norm's gain and old residual values of the first items, fetched while the products run
+    const __nv_bfloat16 *const gain = has_ss ? gain_after(p, kind, layer) : nullptr;
+    float hold[4], gn[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int wi = cw + kNumCWarps * k, tq = wi / max(1, nseg32), r = (wi - tq * nseg32) * 32 + lane;
+      const bool in = has_ss && wi < nitem && r < s.rows;
+      hold[k] = in && g.epi == EPI_RESID_H ? __ldcg(p.h + (size_t)(t0 + tq * tstep) * p.d + col0 + r) : 0.f;
+      gn[k] = in && gain ? __bfloat162float(gain[col0 + r]) : 1.f;
+    }
+    // the attention phase that follows: cache pages of the warp's pieces of this CTA's first item ...
+    int at_kfirst = 0, at_hh = -1;
+    if (kind == PH_QKV && TP <= 16 && !PROMPT && cta < rows->nitems) {   // (more rows: the epilogue needs the area)
+      int sq = 0;
+      while (cta >= rows->s_item0[sq + 1]) ++sq;
+      const int nsp = rows->s_nsp[sq], chunk = rows->s_chunk[sq], rel = cta - rows->s_item0[sq], hh = rel / nsp;
+      const int kbeg = (rel - hh * nsp) * chunk, kend = min(rows->s_pos0[sq] + rows->s_rows[sq], kbeg + chunk);
+      at_kfirst = kbeg + 16 * cw;
+      attn_pages(sq, at_kfirst, kend, 0);
+      if (at_kfirst < kend) at_hh = hh;
+    }
+    if (arrived) phase_await();
     const bool stamper = cta == 0 && ctid == 0;
     stamp(p, ph, 0, stamper);
     // 1/rms per row of h for phases whose input was h * gain (partials summed in CTA order)
@@ -1624,44 +1712,6 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
       }
     }
     stamp(p, ph, 1, stamper);
-    const bool has_ss = g.epi == EPI_RESID_H || g.epi == EPI_STORE_H;
-    const bool sw = g.epi == EPI_SWIGLU_ACT;
-    // thread <-> weight row: quarter = warp index mod 4 (the tensor-memory lanes this warp may read),
-    // m tile = worker index / 4 (SWIGLU: the first four workers read both accumulators)
-    const int quarter = warp & 3, mi = sw ? 0 : (cw >> 2);
-    const int rloc = s.m64 ? (lane < 16 ? quarter * 16 + lane : 1 << 20) : quarter * 32 + lane;   // row inside the m tile
-    const bool active_warp = s.rows > 0 && (sw ? cw < 4 : mi < s.mtiles);
-    const int rslab = mi * s.box_rows + rloc;                   // row inside the slab
-    const bool valid = active_warp && rloc < s.box_rows && rslab < s.rows;
-    const int vrow = s.seg * g.Nseg + s.r0 + rslab;             // output column
-
-    // Epilogue items: (pass row, 32 rows of the slab) for a warp, dealt to all eight workers in turn.  K-split pair: CTA j of
-    // the pair finishes the pass rows j, j + 2, ...
-    const bool pair = s.ks > 1 && s.rows > 0;
-    const int t0 = pair ? s.kj : 0, tstep = pair ? 2 : 1, mine = pair ? (Tg + 1 - s.kj) >> 1 : Tg;
-    const int nseg32 = (s.rows + 31) >> 5, nitem = mine * nseg32;
-    const int col0 = s.seg * g.Nseg + s.r0;                     // output column of slab row 0
-    // the next norm's gain and old residual values of the first items, fetched while the products run
-    const __nv_bfloat16 *const gain = has_ss ? gain_after(p, kind, layer) : nullptr;
-    float hold[4], gn[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const int wi = cw + kNumCWarps * k, tq = wi / max(1, nseg32), r = (wi - tq * nseg32) * 32 + lane;
-      const bool in = has_ss && wi < nitem && r < s.rows;
-      hold[k] = in && g.epi == EPI_RESID_H ? __ldcg(p.h + (size_t)(t0 + tq * tstep) * p.d + col0 + r) : 0.f;
-      gn[k] = in && gain ? __bfloat162float(gain[col0 + r]) : 1.f;
-    }
-    // the attention phase that follows: cache pages of the warp's pieces of this CTA's first item ...
-    int at_kfirst = 0, at_hh = -1;
-    if (kind == PH_QKV && TP <= 16 && !PROMPT && cta < rows->nitems) {   // (more rows: the epilogue needs the area)
-      int sq = 0;
-      while (cta >= rows->s_item0[sq + 1]) ++sq;
-      const int nsp = rows->s_nsp[sq], chunk = rows->s_chunk[sq], rel = cta - rows->s_item0[sq], hh = rel / nsp;
-      const int kbeg = (rel - hh * nsp) * chunk, kend = min(rows->s_pos0[sq] + rows->s_rows[sq], kbeg + chunk);
-      at_kfirst = kbeg + 16 * cw;
-      attn_pages(sq, at_kfirst, kend, 0);
-      if (at_kfirst < kend) at_hh = hh;
-    }
     // accumulators of section q of K and this warp's m tile from taddr + (q & 1) place on, its sums from `sums` on
     const uint32_t cols = acc_cols((uint32_t)TP), place = (uint32_t)s.mtiles * cols;
     const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)mi * cols;
@@ -1822,9 +1872,13 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
       }
     }
     stamp(p, ph, 3, stamper);
-    grid_barrier(p, epoch, tid, abort_s);
+    phase_arrive();
+    arrived = true;
 
-    if (g.epi == EPI_ARGMAX_LM && (cta == 0 || p.mode == 1)) {   // (every CTA needs the token of the next draft step)
+    if (g.epi != EPI_ARGMAX_LM) continue;
+    phase_await();
+    arrived = false;
+    if (cta == 0 || p.mode == 1) {   // (every CTA needs the token of the next draft step)
       // greedy choice per row: the candidates of all CTAs merged (largest value, lowest index among equals, so
       // any merge order gives the same result).  Warp w takes rows 2w and 2w + 1 (of each 16), 16 lanes per row, each lane
       // the CTAs congruent to it mod 16 with all its loads in flight at once.
@@ -1881,7 +1935,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
   }
   // ---- accept (CTA 0; the rows' tokens past a sequence's first are its draft).  Row list and accepting in the pass instead of
   // launches before and after it: tiny model, a step of 4 drafts 235 -> 232 us, four sequences 287 -> 283 us.
-  if (!PROMPT && p.mode == 0 && p.accept && cta == 0 && !is_xprod) {
+  if (!PROMPT && p.mode == 0 && p.accept && cta == 0) {
     named_bar(3, kNumCWarps * 32);
     if (ctid < p.B) {
       int i = 0;
@@ -1895,8 +1949,8 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
   // ---- the next draft step: its rows, and with the stopping rule of Section 4 whether there is one.  Every CTA comes to
   // the same decision.
   if (p.mode == 1 && !PROMPT) {
-    named_bar(2, (kNumXWarps + kNumCWarps) * 32);
-    if (tid == kFirstWorker * 32) {
+    named_bar(3, kNumCWarps * 32);
+    if (ctid == 0) {
       const int made = step + 1;
       int n = rows->n[0];
       if (p.ddd_thr < 0.f && made >= n) {
@@ -1919,22 +1973,15 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
           }
       }
     }
-    named_bar(2, (kNumXWarps + kNumCWarps) * 32);
+    named_bar(6, kBarThreads);
     if (p.ddd_thr < 0.f) nstep = rows->n[0];
   }
-  }
-  if (!PROMPT && p.steps_out && cta == 0 && tid == 32) *p.steps_out = nstep - first_step;
-  // the last CTA to leave clears the barrier count for the next launch (all have passed the last barrier)
-  if (tid == 32 && atomicAdd(p.gbar + 16, 1u) == (unsigned)ncta - 1u) {
-    p.gbar[0] = 0;
-    p.gbar[16] = 0;
+  if (arrived) phase_await();   // (a prompt's pass of the draft head ends with its layer)
   }
   // let warp 2 free the tensor memory once every worker has made its last read
-  if (!is_xprod) {
-    await_copies(abort_s);
-    tc_fence_before();
-    named_bar(5, 32 + kNumCWarps * 32);
-  }
+  await_copies(abort_s);
+  tc_fence_before();
+  named_bar(5, 32 + kNumCWarps * 32);
 }
 
 // Self-test of the bounded waits: the same wait routines as the pass kernel, on a barrier nobody arrives at (mode 0:
@@ -1957,9 +2004,15 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_wait_selftest(unsigned *gba
       await_copies(&abort_flag);
       result[0] = 1;
     }
-  } else if (warp == 1 || warp >= kFirstWorker) {   // the threads that take part in the pass kernel's grid barrier
-    grid_barrier_body(gbar, cnt, nullptr, 2u, tid, &abort_flag, limit);   // one CTA arrives, two are awaited
+  } else if (warp == 1) {   // as in the pass kernel: warp 1 stands for the CTA
+    named_bar(2, kBarThreads);
+    if (tid == 32) grid_wait(gbar, cnt, 2u * gridDim.x, &abort_flag, limit);   // one CTA arrives, two are awaited
+    __syncwarp();
+    named_arrive(4, kBarThreads);
     if (tid == 32) result[1] = 1;
+  } else if (warp >= kFirstWorker) {
+    phase_arrive();
+    phase_await();
   }
 }
 
