@@ -85,7 +85,7 @@ static_assert(kAttnBytes <= kXBytes, "the attention scratch must not reach the a
 constexpr int kScratchBytes = kXBytes + kRedBytes;
 constexpr int kPassSmemBytes = 1024 + kRingBytes + kMiscBytes + kScratchBytes;   // 1 KB to align the ring
 static_assert(kPassSmemBytes <= 227 * 1024, "shared memory budget");
-constexpr int kSsStride = 256;   // CTAs at most
+constexpr int kSsStride = 256;   // CTAs, or 64-column pieces of a row, at most
 constexpr int kStatTimeout = 4;
 constexpr unsigned kSpinLimit = 1u << 22;
 
@@ -145,7 +145,7 @@ struct PassParams {
   __nv_bfloat16 *at;              // K = d    attention output
   __nv_bfloat16 *ac;              // K = F    SwiGLU output
   __nv_bfloat16 *fc;              // K = 2d   draft-head input [e ; f]
-  float *ss_part;              // [rows][kSsStride] partial sums of squares of h by CTA
+  float *ss_part;              // [rows][kSsStride] partial sums of squares of h, see Slab::nss
   float *feat; int cap;        // target features by position [seq][cap][d]
   float *dfeat; int nmax;      // draft features [seq][nmax][d]
   // attention
@@ -401,6 +401,15 @@ __device__ __forceinline__ void xstore(__nv_bfloat16 *tiles, int TP, int t, int 
   tiles[o + TP * 64] = lo;   // row TP + t: same (row & 7)
 }
 
+// two neighbouring columns, k even
+__device__ __forceinline__ void xstore2(__nv_bfloat16 *tiles, int TP, int t, int k, float x, float y) {
+  __nv_bfloat162 hi, lo;
+  split_bf16(x, hi.x, lo.x);
+  split_bf16(y, hi.y, lo.y);
+  const size_t o = xtile(TP, t, k);
+  *reinterpret_cast<__nv_bfloat162 *>(tiles + o) = hi;
+  *reinterpret_cast<__nv_bfloat162 *>(tiles + o + TP * 64) = lo;
+}
 __device__ __forceinline__ void xstore4(__nv_bfloat16 *tiles, int TP, int t, int k, float4 v) {   // k a multiple of 4
   __nv_bfloat16 hi[4], lo[4];
   split_bf16(v.x, hi[0], lo[0]); split_bf16(v.y, hi[1], lo[1]); split_bf16(v.z, hi[2], lo[2]); split_bf16(v.w, hi[3], lo[3]);
@@ -510,6 +519,8 @@ struct Slab {
   int rot;          // ... which it walks from c0 + rot, around the end
   int per, nsec;    // chunks per section of K (in the order of the walk), sections
   int group;        // index of the slab (= group of ks CTAs)
+  int segs, nss;    // pieces of 64 columns (from an even one on) that cover any slab, and those of all slabs: a phase that leaves
+                    // sums of squares leaves one per pass row and piece
 };
 __host__ __device__ __forceinline__ int slab_rpc(int Nseg, int nseg, int ncta) {
   const int cps = ncta / nseg;
@@ -556,6 +567,8 @@ __device__ __forceinline__ Slab make_slab(const GemmDesc &g, int cta, int ncta) 
   s.r0 = li * rpc;
   s.rows = (s.seg < g.nseg) ? max(0, min(g.Nseg, s.r0 + rpc) - s.r0) : 0;
   if (s.c1 <= s.c0) s.rows = 0;
+  s.segs = ((rpc + 2) / 2 + 31) / 32;
+  s.nss = (g.Nseg + rpc - 1) / rpc * s.segs;
   s.box_rows = slab_box_rows(rpc, sw);
   s.mtiles = sw ? 2 : ((rpc + 127) / 128);
   if (!sw && s.rows <= s.box_rows) s.mtiles = 1;  // a short last slab may not reach the second tile
@@ -1643,21 +1656,42 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
     const bool valid = active_warp && rloc < s.box_rows && rslab < s.rows;
     const int vrow = s.seg * g.Nseg + s.r0 + rslab;             // output column
 
-    // Epilogue items: (pass row, 32 rows of the slab) for a warp, dealt to all eight workers in turn.  K-split pair: CTA j of
-    // the pair finishes the pass rows j, j + 2, ...
+    // K-split pair: CTA j of the pair finishes the pass rows j, j + 2, ...  Two neighbouring output columns go to a thread, an even
+    // one and the next; `odd` = 1 where the slab starts on an odd column.
     const bool pair = s.ks > 1 && s.rows > 0;
-    const int t0 = pair ? s.kj : 0, tstep = pair ? 2 : 1, mine = pair ? (Tg + 1 - s.kj) >> 1 : Tg;
-    const int nseg32 = (s.rows + 31) >> 5, nitem = mine * nseg32;
+    const int t0 = pair ? s.kj : 0, tstep = pair ? 2 : 1, mine = s.rows > 0 ? (pair ? (Tg + 1 - s.kj) >> 1 : Tg) : 0;
     const int col0 = s.seg * g.Nseg + s.r0;                     // output column of slab row 0
-    // the next norm's gain and old residual values of the first items, fetched while the products run
+    const int odd = s.r0 & 1;
+    // QKV, SwiGLU: (pass row, column pair) over all 256 threads.  Residual rows: a warp takes 64 columns of one pass row (an item),
+    // whose sum of squares it leaves.  (With one column per thread, 32 columns of a row per warp and step, a step was a chain of
+    // 400 to 700 clocks, two to four of them a phase, and the rows' sums went through shared memory.  Verify: 7B 5 rows 2738 -> 2708
+    // us, 11 rows 2918 -> 2840, 18 rows of three sequences 2975 -> 2875; middle model 18 rows 853 -> 814.)
+    const int pairs = (odd + s.rows + 1) >> 1, nflat = s.rows > 0 ? Tg * pairs : 0;
+    const unsigned per_pair = ((1u << 22) + (unsigned)pairs - 1u) / (unsigned)max(1, pairs);   // e / pairs = e per_pair >> 22: e < 48 pairs, pairs <= 129
+    const int segs = s.segs, nitem = mine * segs;
+    // the next norm's gain and old residual values of the first items
     const __nv_bfloat16 *const gain = has_ss ? gain_after(p, kind, layer) : nullptr;
-    float hold[4], gn[4];
+    constexpr int kAhead = 2;
+    float2 hold[kAhead], gn[kAhead];
+    auto item_old = [&](int wi, float2 &h, float2 &gv) {
+      const int tq = wi / segs, r = (wi - tq * segs) * 64 + 2 * lane - odd;
+      const float *hp = p.h + (size_t)(t0 + tq * tstep) * p.d + col0 + r;
+      h = make_float2(0.f, 0.f);
+      gv = make_float2(1.f, 1.f);
+      if (wi >= nitem) return;
+      const bool in0 = r >= 0 && r < s.rows, in1 = r + 1 < s.rows;
+      if (g.epi == EPI_RESID_H) {
+        if (in0) h.x = __ldcg(hp);
+        if (in1) h.y = __ldcg(hp + 1);
+      }
+      if (gain) {
+        if (in0) gv.x = __bfloat162float(gain[col0 + r]);
+        if (in1) gv.y = __bfloat162float(gain[col0 + r + 1]);
+      }
+    };
+    if (has_ss) {
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const int wi = cw + kNumCWarps * k, tq = wi / max(1, nseg32), r = (wi - tq * nseg32) * 32 + lane;
-      const bool in = has_ss && wi < nitem && r < s.rows;
-      hold[k] = in && g.epi == EPI_RESID_H ? __ldcg(p.h + (size_t)(t0 + tq * tstep) * p.d + col0 + r) : 0.f;
-      gn[k] = in && gain ? __bfloat162float(gain[col0 + r]) : 1.f;
+      for (int k = 0; k < kAhead; ++k) item_old(cw + kNumCWarps * k, hold[k], gn[k]);
     }
     // the attention phase that follows: cache pages of the warp's pieces of this CTA's first item ...
     int at_kfirst = 0, at_hh = -1;
@@ -1673,15 +1707,18 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
     if (arrived) phase_await();
     const bool stamper = cta == 0 && ctid == 0;
     stamp(p, ph, 0, stamper);
-    // 1/rms per row of h for phases whose input was h * gain (partials summed in CTA order)
+    // 1/rms per row of h for phases whose input was h * gain (partials summed in a fixed order)
     if (g.scale_inv_rms) {
-      for (int r = 2 * cw; r < T; r += 2 * kNumCWarps) {   // two rows per warp and step; lanes stride over the CTAs (at most 256), all loads in flight, fixed shuffle tree
+      // partials of a row: left by the phase that wrote h
+      const int nss = kind == PH_GATEUP ? gemms[PH_O - PH_FC].s.nss
+                      : kind == PH_LM || layer > 0 ? gemms[PH_DOWN - PH_FC].s.nss : p.mode == 0 ? ncta : gemms[0].s.nss;
+      for (int r = 2 * cw; r < T; r += 2 * kNumCWarps) {   // two rows per warp and step; lanes stride over the partials (at most 256), all loads in flight, fixed shuffle tree
         float v0[8], v1[8];
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
           const int i = lane + 32 * k;
-          v0[k] = i < ncta ? __ldcg(p.ss_part + r * kSsStride + i) : 0.f;
-          v1[k] = i < ncta && r + 1 < T ? __ldcg(p.ss_part + (r + 1) * kSsStride + i) : 0.f;
+          v0[k] = i < nss ? __ldcg(p.ss_part + r * kSsStride + i) : 0.f;
+          v1[k] = i < nss && r + 1 < T ? __ldcg(p.ss_part + (r + 1) * kSsStride + i) : 0.f;
         }
         float s0 = 0.f, s1 = 0.f;
 #pragma unroll
@@ -1789,33 +1826,51 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
     }
     if (pair) ++kuses;
     const int epi = g.epi;
-    if (epi != EPI_ARGMAX_LM) {
+    if (has_ss) {
       named_bar(3, kNumCWarps * 32);
 #pragma unroll 1
       for (int wi = cw, k = 0; wi < nitem; wi += kNumCWarps, ++k) {
-        const int tq = wi / nseg32, sg = wi - tq * nseg32, r = sg * 32 + lane, t = t0 + tq * tstep;
-        const bool in = r < s.rows;
-        const int col = col0 + r;
-        const float sc = g.scale_inv_rms ? inv_rms[t] : 1.f;
-        const float y = in ? ys[t * 256 + r] * sc : 0.f;
-        if (epi == EPI_STORE_QKV) {
-          if (in) p.qkv[(size_t)t * 3 * p.d + col] = y;
-        } else if (sw) {
-          if (in) xstore(p.ac, TP, t, col, (y / (1.f + __expf(-y))) * (ys[t * 256 + 128 + r] * sc));
+        const int tq = wi / segs, sg = wi - tq * segs, r = sg * 64 + 2 * lane - odd, t = t0 + tq * tstep;
+        const bool in0 = r >= 0 && r < s.rows, in1 = r + 1 < s.rows;
+        float2 hn = k == 0 ? hold[0] : hold[1], gv = k == 0 ? gn[0] : gn[1];
+        if (k >= kAhead) item_old(wi, hn, gv);   // (more items than were fetched ahead)
+        const float *y = ys + t * 256 + r;
+        hn.x = in0 ? hn.x + y[0] : 0.f;
+        hn.y = in1 ? hn.y + y[1] : 0.f;
+        float *hp = p.h + (size_t)t * p.d + col0 + r;
+        if (in0 && in1) {
+          *reinterpret_cast<float2 *>(hp) = hn;
+          xstore2(p.xa, TP, t, col0 + r, hn.x * gv.x, hn.y * gv.y);
+        } else if (in0) {
+          hp[0] = hn.x;
+          xstore(p.xa, TP, t, col0 + r, hn.x * gv.x);
+        } else if (in1) {
+          hp[1] = hn.y;
+          xstore(p.xa, TP, t, col0 + r + 1, hn.y * gv.y);
+        }
+        const float q = warp_sum(hn.x * hn.x + hn.y * hn.y);
+        if (lane == 0) p.ss_part[t * kSsStride + s.group * segs + sg] = q;
+      }
+    } else if (epi != EPI_ARGMAX_LM) {
+      named_bar(3, kNumCWarps * 32);
+#pragma unroll 1
+      for (int e = ctid; e < nflat; e += kNumCWarps * 32) {
+        const int t = (int)(((unsigned)e * per_pair) >> 22), r = 2 * (e - t * pairs) - odd;
+        const bool in0 = r >= 0, in1 = r + 1 < s.rows;
+        const float sc = inv_rms[t];
+        const float *y = ys + t * 256 + r;
+        float2 v = make_float2(in0 ? y[0] * sc : 0.f, in1 ? y[1] * sc : 0.f);
+        if (sw) {
+          v.x = (v.x / (1.f + __expf(-v.x))) * (in0 ? y[128] * sc : 0.f);
+          v.y = (v.y / (1.f + __expf(-v.y))) * (in1 ? y[129] * sc : 0.f);
+          if (in0 && in1) xstore2(p.ac, TP, t, col0 + r, v.x, v.y);
+          else if (in0) xstore(p.ac, TP, t, col0 + r, v.x);
+          else xstore(p.ac, TP, t, col0 + r + 1, v.y);
         } else {
-          float hn = k == 0 ? hold[0] : k == 1 ? hold[1] : k == 2 ? hold[2] : hold[3];
-          float gv = k == 0 ? gn[0] : k == 1 ? gn[1] : k == 2 ? gn[2] : gn[3];
-          if (k >= 4) {   // (more items than were fetched ahead)
-            hn = in && epi == EPI_RESID_H ? __ldcg(p.h + (size_t)t * p.d + col) : 0.f;
-            gv = in && gain ? __bfloat162float(gain[col]) : 1.f;
-          }
-          hn += y;
-          if (in) {
-            p.h[(size_t)t * p.d + col] = hn;
-            xstore(p.xa, TP, t, col, hn * gv);
-          }
-          const float q = warp_sum(in ? hn * hn : 0.f);
-          if (lane == 0) ssw[t * 8 + sg] = q;
+          float *o = p.qkv + (size_t)t * 3 * p.d + col0 + r;
+          if (in0 && in1) *reinterpret_cast<float2 *>(o) = v;
+          else if (in0) o[0] = v.x;
+          else o[1] = v.y;
         }
       }
     } else {
@@ -1848,16 +1903,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
         }
       }
     }
-    if (has_ss) {
-      // sum of squares per pass row over this CTA's columns, in column order (the rows the pair's other CTA finishes: 0)
-      named_bar(3, kNumCWarps * 32);
-      if (ctid < Tg) {
-        float r = 0.f;
-        if (!pair || (ctid & 1) == s.kj)
-          for (int j = 0; j < nseg32; ++j) r += ssw[ctid * 8 + j];
-        p.ss_part[ctid * kSsStride + cta] = r;
-      }
-    } else if (epi == EPI_ARGMAX_LM) {
+    if (epi == EPI_ARGMAX_LM) {
       named_bar(3, kNumCWarps * 32);
       if (ctid < Tg) {
         Top2 b = topw[ctid];
