@@ -127,6 +127,30 @@ def test_small_models_on_part_of_the_chip(vocab):
         e.close()
 
 
+@pytest.mark.parametrize("d,heads,ffn,batch", [(192, 3, 144, 2), (1088, 17, 400, 2), (4672, 73, 128, 1)])
+def test_slabs_of_odd_widths(d, heads, ffn, batch):
+    """Slabs that start on odd columns, thread blocks without a slab, pieces of 64 columns that a slab fills in part or that
+    spill into a second piece (64 rows a pair of thread blocks at the largest width), K outside whole chunks."""
+    import oracle
+    from paper_2412_18910_b200 import Engine
+    sh = si.scaled(si.SHAPES["tiny"], n_layers=1, d_model=d, n_heads=heads, head_dim=64, d_ffn=ffn, vocab=272)
+    w = si.make_weights(sh)
+    m = oracle.Model(sh, w)
+    e = Engine(sh, w, max_batch=batch, kv_capacity=128)
+    try:
+        seqs = []
+        for b in range(batch):
+            prompt = si.uniform_ids(11 + b, "odd%d" % b, 7 + 13 * b, 272)
+            seq = m.new_seq(128)
+            assert seq.prefill(prompt) == e.prefill(b, prompt)
+            seqs.append(seq)
+        res = lockstep.run_lockstep(e, seqs, 4)
+        assert not res["failures"], res["failures"]
+        assert e.ada_get_counters()["status"] == 0
+    finally:
+        e.close()
+
+
 @pytest.mark.parametrize("batch", [1, 3, 6])
 def test_drafts_do_not_depend_on_batch_mates(batch):
     """A sequence's drafts and draft features bit for bit beside short and beside long sequences (three sequences: every step in
