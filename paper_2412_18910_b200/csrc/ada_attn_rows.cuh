@@ -39,7 +39,6 @@ __global__ void __launch_bounds__(128) k_attn_rows(const Pass *pass, const float
   static_assert(HD == 64 || HD == 128, "head width");
   constexpr int page_size = kPageSize;
   pdl_launch_dependents();
-  pdl_wait();                  // queries and the new cache rows come from the kernel before this one
   constexpr int CH = HD / 8;   // 16-byte chunks per row
   constexpr int RG = 8;        // query rows per group
   // grid.z = sequences x nrg: CTA (b, rgi) takes the row groups rgi, rgi + nrg, ... of sequence b
@@ -47,11 +46,13 @@ __global__ void __launch_bounds__(128) k_attn_rows(const Pass *pass, const float
   const int rgi = blockIdx.z - b * nrg;
   const int4 si = pass->seq_info[b];   // (first row, rows, split size, first position) in one load
   const int row0 = si.x, R = si.y, pos0 = si.w;
-  if (R <= 0) return;
   const int nkeys = pos0 + R;
   const int chunk = attn_rows_chunk(si.z, cap);
   const int kbeg = split * chunk, kend = min(nkeys, kbeg + chunk);
-  if (kbeg >= nkeys) return;
+  if (rgi * RG >= R || kbeg >= nkeys) {
+    pdl_wait();
+    return;
+  }
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int d = H * HD;
 
@@ -96,10 +97,15 @@ __global__ void __launch_bounds__(128) k_attn_rows(const Pass *pass, const float
       bulk_g2s_hint(kst, kpool + off, (unsigned)(kAttnHalf * HD * 2), &bars[h & 1], l2_policy_evict_first());
       bulk_g2s_hint(kst + kAttnHalf * HD, vpool + off, (unsigned)(kAttnHalf * HD * 2), &bars[h & 1], l2_policy_evict_first());
     };
-    {   // both buffers are free: the first two halves fly under the staging of q
+    {   // Both buffers are free: the first two halves fly under the staging of q, and those without new rows already while the
+        // kernel before this one finishes, which makes the queries and the new cache rows.
       const int p0 = __shfl_sync(0xffffffffu, pages, 0), p1 = __shfl_sync(0xffffffffu, pages, 1);
-      if (lane == 0 && valid(0)) issue(0, p0);
-      if (lane == 0 && valid(1)) issue(1, p1);
+      const bool old0 = key0_of(0) + kAttnHalf <= pos0, old1 = key0_of(1) + kAttnHalf <= pos0;
+      if (lane == 0 && valid(0) && old0) issue(0, p0);
+      if (lane == 0 && valid(1) && old1) issue(1, p1);
+      if (rg == rgi * RG) pdl_wait();
+      if (lane == 0 && valid(0) && !old0) issue(0, p0);
+      if (lane == 0 && valid(1) && !old1) issue(1, p1);
     }
     {   // the group's query rows as (hi, lo) halves; rows past nr are zero: hi of row r in tile row r, lo in row r + 8
       constexpr int PER = RG * HD / 4 / 128;

@@ -343,10 +343,12 @@ struct ReduceHArgs {
 __global__ void __launch_bounds__(256) k_reduce_h(const ReduceHArgs a) {
   __shared__ float sh[32];
   pdl_launch_dependents();
-  pdl_wait();
   const int t = blockIdx.y, seg = blockIdx.x;
-  if (t >= a.pass->T) return;
   const int col = seg * 1024 + threadIdx.x * 4;
+  const bool live = t < a.pass->T;
+  const uint2 gg = a.gain && col < a.d ? *reinterpret_cast<const uint2 *>(a.gain + col) : make_uint2(0u, 0u);
+  pdl_wait();
+  if (!live) return;
   float ss = 0.f;
   if (col < a.d) {
     float4 y = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -363,7 +365,6 @@ __global__ void __launch_bounds__(256) k_reduce_h(const ReduceHArgs a) {
     *hp = hv;
     ss = (hv.x * hv.x + hv.y * hv.y) + (hv.z * hv.z + hv.w * hv.w);
     if (a.gain) {
-      const uint2 gg = *reinterpret_cast<const uint2 *>(a.gain + col);
       const __nv_bfloat162 g01 = *reinterpret_cast<const __nv_bfloat162 *>(&gg.x), g23 = *reinterpret_cast<const __nv_bfloat162 *>(&gg.y);
       const float x[4] = {hv.x * __bfloat162float(g01.x), hv.y * __bfloat162float(g01.y), hv.z * __bfloat162float(g23.x),
                           hv.w * __bfloat162float(g23.y)};
@@ -399,13 +400,17 @@ struct ReduceQkvArgs {
 };
 __global__ void __launch_bounds__(256) k_reduce_qkv(const ReduceQkvArgs a) {
   pdl_launch_dependents();
-  pdl_wait();
   const int t = blockIdx.y;
-  if (t >= a.pass->T) return;
   const int d = a.H * a.hd, half = a.hd >> 1;
   const int idx = blockIdx.x * 256 + threadIdx.x;
-  if (idx >= a.H * half) return;
   const int hh = idx / half, i = idx - hh * half, o = hh * a.hd + i;
+  // what the row list and the tables hold, before the wait: three lookups one behind the other
+  const bool live = t < a.pass->T && idx < a.H * half;
+  const int pos = live ? a.pass->row_pos[t] : 0, b = live ? a.pass->row_seq[t] : 0;
+  const float2 cs = live ? a.rope[(size_t)pos * half + i] : make_float2(1.f, 0.f);
+  const int page = live ? a.page_table[b * a.pages_per_seq + pos / kPageSize] : 0, slot = pos % kPageSize;
+  pdl_wait();
+  if (!live) return;
   float v[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};   // q_i, q_i+half, k_i, k_i+half, v_i, v_i+half
   for (int sp = 0; sp < a.S; ++sp) {
     const float *pp = a.part + ((size_t)sp * a.part_rows + t) * (3 * d);
@@ -416,11 +421,8 @@ __global__ void __launch_bounds__(256) k_reduce_qkv(const ReduceQkvArgs a) {
   const float inv = inv_rms_of(a.ss_part, t, d, a.eps);
 #pragma unroll
   for (int j = 0; j < 6; ++j) v[j] *= inv;
-  const int pos = a.pass->row_pos[t], b = a.pass->row_seq[t];
-  const float2 cs = a.rope[(size_t)pos * half + i];
   a.qout[(size_t)t * d + o] = (v[0] * cs.x - v[1] * cs.y) * a.qscale;
   a.qout[(size_t)t * d + o + half] = (v[1] * cs.x + v[0] * cs.y) * a.qscale;
-  const int page = a.page_table[b * a.pages_per_seq + pos / kPageSize], slot = pos % kPageSize;
   const size_t base = (((size_t)page * a.L + a.layer) * a.H + hh) * kPageSize * a.hd + (size_t)slot * a.hd;
   const int sw = slot & 7;
   a.kpool[base + ((((i >> 3) ^ sw) << 3) | (i & 7))] = kv_store(v[2] * cs.x - v[3] * cs.y);
@@ -439,9 +441,9 @@ struct ReduceSwigluArgs {
 };
 __global__ void __launch_bounds__(256) k_reduce_swiglu(const ReduceSwigluArgs a) {
   pdl_launch_dependents();
-  pdl_wait();
   const int T = a.pass->T;
   const int c4 = a.F >> 2;
+  pdl_wait();
   for (int idx = blockIdx.x * 256 + threadIdx.x; idx < T * c4; idx += gridDim.x * 256) {
     const int t = idx / c4, col = (idx - t * c4) << 2;
     float4 y = make_float4(0.f, 0.f, 0.f, 0.f), u = y;
