@@ -103,6 +103,33 @@ def test_step_ends_as_its_parts_do_when_sequences_fill_up():
             e.close()
 
 
+@pytest.mark.parametrize("batch", [5, 6, 8])
+def test_catch_up_rows_of_more_than_one_pass(tiny, batch):
+    """Drafts after nine tokens were committed in every sequence: 45, 54 and 72 catch-up rows, which the draft head takes in one
+    pass of up to 48 rows or in two (of five sequences and the others)."""
+    import oracle
+    from paper_2412_18910_b200 import Engine
+    sh, w, _, m = tiny
+    e = Engine(sh, w, max_batch=batch, kv_capacity=512)
+    try:
+        seqs, prompts, streams = [], [], []
+        for b in range(batch):
+            prompts.append(si.uniform_ids(23 + b, "catch%d" % b, 30 + 29 * b, sh.vocab))
+            streams.append(oracle.decode(m, prompts[b], 40, n_policy=0)["tokens"])
+            seqs.append(m.new_seq(512))
+            assert seqs[b].prefill(prompts[b]) == e.prefill(b, prompts[b])
+        e.ada_force_n([8] * batch)
+        res = lockstep.run_lockstep(e, seqs, 2, n_forced=8, forced_stream=streams, prompts=prompts)
+        assert not res["failures"], res["failures"]
+        assert all(seq.counters()["n_waste"] == 0 for seq in seqs)
+        e.ada_force_draft(None)
+        res = lockstep.run_lockstep(e, seqs, 2, n_forced=8)     # the heads' own drafts on those cache rows
+        assert not res["failures"], res["failures"]
+        assert e.ada_get_counters()["status"] == 0
+    finally:
+        e.close()
+
+
 @pytest.mark.parametrize("vocab", [4096, 5120, 9216, 9728])
 def test_small_models_on_part_of_the_chip(vocab):
     """Widths around the 64 thread blocks that the smallest models run on, between them and all of the chip, and on either
