@@ -1000,7 +1000,8 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
       uint32_t sphase = 0;     // per place of the accumulators the parity of its next release in this phase
       for (int v = 0;
            v < npasses || (p.ddd_thr < 0.f && v < (int)__reduce_max_sync(0xffffffffu, (unsigned)await_length(step_bar, decisions, rows, p.cnt, abort_s)));
-           ++v, xslot = 0)
+           ++v, xslot = 0) {
+      unsigned tp = 0;         // padded rows of the pass
       for (int ph = 0; ph < nphase; ++ph) {
         int layer;
         const int kind = phase_kind(p, ph, layer);
@@ -1010,8 +1011,10 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
         const Slab s = make_slab(g, cta, ncta);
         const int K = g.K;
         if (s.rows == 0) continue;
-        // (the rows of the pass are known once its first activations have landed)
-        mbar_wait(&xfull[xslot], (xphase >> xslot) & 1u, p.cnt, abort_s);
+        if (tp == 0) {   // (the rows of the pass are known once its first activations have landed)
+          mbar_wait(&xfull[xslot], (xphase >> xslot) & 1u, p.cnt, abort_s);
+          tp = __reduce_max_sync(0xffffffffu, (unsigned)*reinterpret_cast<const volatile int *>(&rows->TP));
+        }
         // A phase's products.  The padded row count is a constant in each form: box strides and the instruction descriptor
         // then need no registers that the tensor-core instructions could not take (with a row count read from memory gate/up
         // of 5 rows took 44.5 us, with one put into a uniform register by a reduction 33.5, as a constant 31.1).
@@ -1099,13 +1102,16 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
             }
             --left;
             const uint64_t bdesc0 = umma_desc(xbuf_u + (uint32_t)(xslot * xbuf_bytes(TP)));
-            mbar_wait(&xfull[xslot], (xphase >> xslot) & 1u, p.cnt, abort_s);
 #pragma unroll
             for (int q = 0; q < kxb / KB * MT; ++q) {
               const int mi = q % MT, b0 = q / MT * KB;
               const uint32_t off = cur.take(bytes);
               const unsigned slot = (cur.n - 1) % kSlots;
               mbar_wait(&full[slot], ((cur.n - 1) / kSlots) & 1u, p.cnt, abort_s);
+              // The activations last: a phase's first weights are there long before them, and all that leads to the products is done
+              // when they land (the row count, too, is asked for once a pass).  Draft of four + verify, waiting for them first ->
+              // so: small model 145 + 66.5 -> 139 + 64.5 us, middle model 331 + 717 -> 323 + 703, 7B 583 + 2663 -> 576 + 2628.
+              if (q == 0) mbar_wait(&xfull[xslot], (xphase >> xslot) & 1u, p.cnt, abort_s);
               tc_fence_after();
               if (elect_one()) {
                 const uint64_t ad = umma_desc(ring_u + off);
@@ -1135,7 +1141,6 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
             else whole_chunks(rows_const, integral_constant<int, 2>{}, integral_constant<int, 2>{});
           }
         };
-        const unsigned tp = __reduce_max_sync(0xffffffffu, (unsigned)*reinterpret_cast<const volatile int *>(&rows->TP));
         auto dispatch = [&](auto &&form) {
           if (tp == 8) form(std::integral_constant<uint32_t, 8>{});
           else if (tp == 16) form(std::integral_constant<uint32_t, 16>{});
@@ -1149,6 +1154,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
         if (elect_one()) umma_commit(accfull);
         __syncwarp();
         sphase = sections_done(sphase, s.nsec);
+      }
       }
     }
     __syncwarp();
