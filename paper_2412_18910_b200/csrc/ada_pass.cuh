@@ -40,6 +40,7 @@
 #pragma once
 #include <type_traits>
 
+#include "ada_areas.h"
 #include "ada_kernels.cuh"
 #include "ada_ring.h"
 
@@ -75,7 +76,7 @@ constexpr int kRedBytes = (kPassRowsMax / 8) * 128 * 16;
 constexpr int kMiscBytes = 6144;                 // mbarriers and small per-CTA arrays
 // attention scratch lives where the activation buffers and the reduction buffer are (both idle
 // during the attention phase); the ring is NOT reused: the producer keeps filling it meanwhile
-constexpr int kAttnLoopBytes = 4 * 16 * 128 * 2 + 8 * 2 * 16 * 128 * 2;   // q hi, q lo, new k, v rows; per warp 16 keys and 16 values
+constexpr int kAttnLoopBytes = kKeysAt + kNumCWarps * kKeysWarpBytes;   // q hi, q lo, new k, v rows; per warp 16 keys and 16 values
 constexpr int kPassMaxSplits = 32;                // cache splits of a sequence at most (its split size is at least capacity / 32)
 constexpr int kPartRow = 136;   // floats per row of a warp's partial result: 128 sums, m, l, padded so that a half-warp's fragment stores (4 rows x 4 column pairs) fall into 32 different banks
 constexpr int kAttnPartBytes = 8 * 16 * kPartRow * 4;   // per-warp partial results
@@ -1255,8 +1256,11 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
   unsigned acc_phase = 0;   // GEMM phases of this CTA whose accumulator has been awaited
   unsigned attn_uses = 0;           // completed phases of this warp's two attention barriers
   // Keys and values of a worker warp: 16-key pieces cw, cw + 8, ... of an item's split, one bulk copy each into the warp's
-  // own two buffers (a piece is contiguous in its cache page).  No warp waits for another inside an item.
-  __nv_bfloat16 *const wst = reinterpret_cast<__nv_bfloat16 *>(xbuf) + 4 * 16 * 128 + cw * 2 * 16 * 128;
+  // own two buffers (a piece is contiguous in its cache page).  No warp waits for another inside an item.  The buffers lie over the
+  // epilogues' sums of pass rows 16 and up (ada_areas.h): where there are such rows a warp's first pieces are requested behind
+  // a barrier of the workers, else in the QKV phase.  (Behind that barrier but before the other CTAs' release, against behind the
+  // release: verify of 7B 18 rows 2760 -> 2742 us, 22 rows at context 1900 3435 -> 3418; middle model 18 rows 788 -> 784.)
+  __nv_bfloat16 *const wst = reinterpret_cast<__nv_bfloat16 *>(xbuf + kKeysAt + cw * kKeysWarpBytes);
   int pages = 0;                    // cache pages of the warp's pieces 32 i + lane of the current item
   auto attn_pages = [&](int sq, int kfirst, int kend, int i0) {   // (fetched 32 at a time: no copy waits for a table lookup)
     const int k0 = kfirst + 128 * (i0 + lane);
@@ -1383,9 +1387,9 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
           const int prow = rows->s_part0[sq] + hh * nsp * R;                          // first row of the head's partial results
           const int kbeg = split * chunk, kend = min(nkeys, kbeg + chunk);
           const int kfirst = kbeg + 16 * cw;
-          if (item != cta || TP > 16 || PROMPT) {   // (up to 16 rows the first item's pieces were requested in the QKV phase)
-            if (item != cta) named_bar(3, kNumCWarps * 32);   // the previous item's merge has read the shared areas
+          if (item != cta || !keys_clear_of_sums(TP) || PROMPT) {   // (else the pieces were requested in the QKV phase)
             attn_pages(sq, kfirst, kend, 0);
+            named_bar(3, kNumCWarps * 32);   // every warp has read what lay there: the QKV phase's sums, or the item before
             const int pg = __shfl_sync(0xffffffffu, pages, 0);
             if (lane == 0 && kfirst < kend) {
               attn_issue(0, kfirst, hh, layer, false, pg);
@@ -1723,7 +1727,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
     }
     // the attention phase that follows: cache pages of the warp's pieces of this CTA's first item ...
     int at_kfirst = 0, at_hh = -1;
-    if (kind == PH_QKV && TP <= 16 && !PROMPT && cta < rows->nitems) {   // (more rows: the epilogue needs the area)
+    if (kind == PH_QKV && keys_clear_of_sums(TP) && !PROMPT && cta < rows->nitems) {   // (more rows: the epilogue needs the area)
       int sq = 0;
       while (cta >= rows->s_item0[sq + 1]) ++sq;
       const int nsp = rows->s_nsp[sq], chunk = rows->s_chunk[sq], rel = cta - rows->s_item0[sq], hh = rel / nsp;
@@ -1808,6 +1812,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
     // half, whoever is faster.  (With plain stores and a releasing arrive the exchange took 1.7 to 2.4 us, most of it the
     // release; one CTA fetching all rows of the other and finishing them alone was no better.)
     // Per layer, 5 rows: 7B O 10.7 -> 8.6, down 19.6 -> 18.2 us; middle model 7.6 -> 6.4 and 11.4 -> 10.2 us.
+    static_assert(kSumsRowBytes == 256 * sizeof(float), "rows of sums");
     float *const ys = reinterpret_cast<float *>(xbuf);    // [rows][256] accumulator values; SwiGLU: 128 gate, 128 up columns
     const bool sends = pair && cw < 4;
     if (sends && ctid == 0) mbar_expect_tx(kbar, (unsigned)(128 * 16 * (TP >> 3)));

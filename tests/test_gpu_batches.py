@@ -206,3 +206,45 @@ def test_drafts_do_not_depend_on_batch_mates(batch):
     for mate_len, n in ((20, sh.n_max), (450, sh.n_max), (450, 3)):
         t, f = draft(batch, mate_len, n)
         assert torch.equal(t, tokens[:n]) and torch.equal(f, feats[:n]), (mate_len, n)
+
+
+@pytest.mark.parametrize("lengths", [[8, 7], [8, 8], [5, 5, 5], [8, 8, 5], [8, 8, 8], [8, 8, 8, 8, 2], [8, 8, 8, 8, 8]])
+def test_verified_rows_do_not_depend_on_batch_mates(lengths):
+    """Logits, features and cache rows of verify passes of 17 to 45 rows, heads 128 wide, bit for bit as each sequence alone has
+    them: 16 rows at most, whose first keys are requested in the QKV phase; those of more rows wait until the sums that lie in the
+    same shared memory are read.  Several cache splits and more than one piece of keys a warp; two layers, so that the cache
+    rows of the first are read behind the second's sums; a second pass reads the cache rows that the first left."""
+    from paper_2412_18910_b200 import Engine
+    sh = si.scaled(si.SHAPES["tiny"], d_model=512, n_heads=4, head_dim=128, d_ffn=1376)
+    w = si.make_weights(sh)
+    prompts = [si.uniform_ids(41 + b, "rows%d" % b, 700 - 130 * b, sh.vocab) for b in range(len(lengths))]
+    drafts = torch.from_numpy(np.stack([si.uniform_ids(51 + b, "draft%d" % b, 2 * sh.n_max, sh.vocab) for b in range(len(lengths))]))
+
+    def verify(members):
+        e = Engine(sh, w, max_batch=len(members), kv_capacity=1024)
+        try:
+            for i, b in enumerate(members):
+                e.prefill(i, prompts[b])
+            out = []
+            for it in range(2):
+                e.d_n.copy_(torch.tensor([lengths[b] for b in members], dtype=torch.int32))
+                e.d_draft.copy_(drafts[members, it * sh.n_max: (it + 1) * sh.n_max])
+                logits = torch.zeros(e.B, sh.n_max + 1, sh.vocab, device=e.dev)
+                e.ada_verify(e.d_draft, e.d_n, e.d_target, logits)
+                feat = e.ada_debug_buffer(0, torch.float32, (e.B, 1024, sh.d_model))
+                pos = [len(prompts[b]) + it for b in members]
+                out.append([(logits[i, : lengths[b] + 1].clone(), feat[i, pos[i]: pos[i] + lengths[b] + 1].clone())
+                            for i, b in enumerate(members)])
+                for i, b in enumerate(members):     # one token on, the same whatever was drafted
+                    e.ada_force_commit(i, drafts[b, it: it + 1].to(e.dev).int(), 1)
+            assert e.ada_get_counters()["status"] == 0
+            return out
+        finally:
+            e.close()
+
+    together = verify(list(range(len(lengths))))
+    for b in range(len(lengths)):
+        alone = verify([b])
+        for it in range(2):
+            for x, y in zip(together[it][b], alone[it][0]):
+                assert torch.equal(x, y), (b, it)
