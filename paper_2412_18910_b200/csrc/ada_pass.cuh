@@ -86,7 +86,13 @@ static_assert(kAttnBytes <= kXBytes, "the attention scratch must not reach the a
 constexpr int kScratchBytes = kXBytes + kRedBytes;
 constexpr int kPassSmemBytes = 1024 + kRingBytes + kMiscBytes + kScratchBytes;   // 1 KB to align the ring
 static_assert(kPassSmemBytes <= 227 * 1024, "shared memory budget");
-constexpr int kSsStride = 256;   // CTAs, or 64-column pieces of a row, at most
+constexpr int kSsStride = 256;   // CTAs at most; pairs of CTAs, three partials each (ss_slots)
+// Partial sums of squares that a slab leaves per pass row: of its columns in groups of 32, the first two groups' sum and, where a
+// slab has more than 64 columns, the third and the fourth, which are added to it one after the other.  A row's sum is made in the
+// same order whatever phase or pass leaves it: another order moves the last bit of the row's scale, and with it 16-bit cache
+// elements.  (Against trees over 64 columns and one partial for each: 7B verify of 5 rows 2659 -> 2671 us, 18 rows 2840 -> 2854,
+// middle model 18 rows 785 -> 789.)
+__host__ __device__ constexpr int ss_slots(int segs) { return segs > 1 ? 3 : 1; }
 constexpr int kStatTimeout = 4;
 constexpr unsigned kSpinLimit = 1u << 22;
 
@@ -148,7 +154,7 @@ struct PassParams {
   __nv_bfloat16 *at;              // K = d    attention output
   __nv_bfloat16 *ac;              // K = F    SwiGLU output
   __nv_bfloat16 *fc;              // K = 2d   draft-head input [e ; f]
-  float *ss_part;              // [rows][kSsStride] partial sums of squares of h, see Slab::nss
+  float *ss_part;              // [rows][kSsStride] partial sums of squares of h, see ss_slots
   float *feat; int cap;        // target features by position [seq][cap][d]
   float *dfeat; int nmax;      // draft features [seq][nmax][d]
   // attention
@@ -522,8 +528,8 @@ struct Slab {
   int rot;          // ... which it walks from c0 + rot, around the end
   int per, nsec;    // chunks per section of K (in the order of the walk), sections
   int group;        // index of the slab (= group of ks CTAs)
-  int segs, nss;    // pieces of 64 columns (from an even one on) that cover any slab, and those of all slabs: a phase that leaves
-                    // sums of squares leaves one per pass row and piece
+  int segs, slabs;  // pieces of 64 columns that cover any slab (one or two), and slabs: a phase that leaves sums of squares leaves
+                    // one per pass row and slab, of slabs of two pieces three (ss_slots)
 };
 __host__ __device__ __forceinline__ int slab_rpc(int Nseg, int nseg, int ncta) {
   const int cps = ncta / nseg;
@@ -570,8 +576,8 @@ __device__ __forceinline__ Slab make_slab(const GemmDesc &g, int cta, int ncta) 
   s.r0 = li * rpc;
   s.rows = (s.seg < g.nseg) ? max(0, min(g.Nseg, s.r0 + rpc) - s.r0) : 0;
   if (s.c1 <= s.c0) s.rows = 0;
-  s.segs = ((rpc + 2) / 2 + 31) / 32;
-  s.nss = (g.Nseg + rpc - 1) / rpc * s.segs;
+  s.segs = (rpc + 63) / 64;
+  s.slabs = (g.Nseg + rpc - 1) / rpc;
   s.box_rows = slab_box_rows(rpc, sw);
   s.mtiles = sw ? 2 : ((rpc + 127) / 128);
   if (!sw && s.rows <= s.box_rows) s.mtiles = 1;  // a short last slab may not reach the second tile
@@ -1688,16 +1694,17 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
     const bool valid = active_warp && rloc < s.box_rows && rslab < s.rows;
     const int vrow = s.seg * g.Nseg + s.r0 + rslab;             // output column
 
-    // K-split pair: CTA j of the pair finishes the pass rows j, j + 2, ...  Two neighbouring output columns go to a thread, an even
-    // one and the next; `odd` = 1 where the slab starts on an odd column.
+    // K-split pair: CTA j of the pair finishes the pass rows j, j + 2, ...  Two neighbouring output columns go to a thread;
+    // `odd` = 1 where the slab starts on an odd column.
     const bool pair = s.ks > 1 && s.rows > 0;
     const int t0 = pair ? s.kj : 0, tstep = pair ? 2 : 1, mine = s.rows > 0 ? (pair ? (Tg + 1 - s.kj) >> 1 : Tg) : 0;
     const int col0 = s.seg * g.Nseg + s.r0;                     // output column of slab row 0
     const int odd = s.r0 & 1;
-    // QKV, SwiGLU: (pass row, column pair) over all 256 threads.  Residual rows: a warp takes 64 columns of one pass row (an item),
-    // whose sum of squares it leaves.  (With one column per thread, 32 columns of a row per warp and step, a step was a chain of
-    // 400 to 700 clocks, two to four of them a phase, and the rows' sums went through shared memory.  Verify: 7B 5 rows 2738 -> 2708
-    // us, 11 rows 2918 -> 2840, 18 rows of three sequences 2975 -> 2875; middle model 18 rows 853 -> 814.)
+    // QKV, SwiGLU: (pass row, even column and the next) over all 256 threads.  Residual rows: a warp takes 64 columns of one pass
+    // row (an item), counted from the slab's first one, and leaves their sums of squares.  (With one column per thread, 32 columns of
+    // a row per warp and step, a step was a chain of 400 to 700 clocks, two to four of them a phase, and the rows' sums went through
+    // shared memory.  Verify: 7B 5 rows 2738 -> 2708 us, 11 rows 2918 -> 2840, 18 rows of three sequences 2975 -> 2875; middle model
+    // 18 rows 853 -> 814.)
     const int pairs = (odd + s.rows + 1) >> 1, nflat = s.rows > 0 ? Tg * pairs : 0;
     const unsigned per_pair = ((1u << 22) + (unsigned)pairs - 1u) / (unsigned)max(1, pairs);   // e / pairs = e per_pair >> 22: e < 48 pairs, pairs <= 129
     const int segs = s.segs, nitem = mine * segs;
@@ -1706,12 +1713,12 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
     constexpr int kAhead = 2;
     float2 hold[kAhead], gn[kAhead];
     auto item_old = [&](int wi, float2 &h, float2 &gv) {
-      const int tq = wi / segs, r = (wi - tq * segs) * 64 + 2 * lane - odd;
+      const int tq = wi / segs, r = (wi - tq * segs) * 64 + 2 * lane;
       const float *hp = p.h + (size_t)(t0 + tq * tstep) * p.d + col0 + r;
       h = make_float2(0.f, 0.f);
       gv = make_float2(1.f, 1.f);
       if (wi >= nitem) return;
-      const bool in0 = r >= 0 && r < s.rows, in1 = r + 1 < s.rows;
+      const bool in0 = r < s.rows, in1 = r + 1 < s.rows;
       if (g.epi == EPI_RESID_H) {
         if (in0) h.x = __ldcg(hp);
         if (in1) h.y = __ldcg(hp + 1);
@@ -1739,18 +1746,32 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
     if (arrived) phase_await();
     const bool stamper = cta == 0 && ctid == 0;
     stamp(p, ph, 0, stamper);
-    // 1/rms per row of h for phases whose input was h * gain (partials summed in a fixed order)
+    // 1/rms per row of h for phases whose input was h * gain (partials summed in CTA order)
     if (g.scale_inv_rms) {
-      // partials of a row: left by the phase that wrote h
-      const int nss = kind == PH_GATEUP ? gemms[PH_O - PH_FC].s.nss
-                      : kind == PH_LM || layer > 0 ? gemms[PH_DOWN - PH_FC].s.nss : p.mode == 0 ? ncta : gemms[0].s.nss;
-      for (int r = 2 * cw; r < T; r += 2 * kNumCWarps) {   // two rows per warp and step; lanes stride over the partials (at most 256), all loads in flight, fixed shuffle tree
+      // partials of a row: left by the phase that wrote h, by the CTA of a pair that finishes the row (the embedding: by all CTAs)
+      const int from = kind == PH_GATEUP ? PH_O : kind == PH_LM || layer > 0 ? PH_DOWN : p.mode == 0 ? PH_EMBED : PH_FC;
+      const bool emb = from == PH_EMBED;
+      const Slab &w = gemms[emb ? 0 : from - PH_FC].s;
+      const int sh = !emb && w.ks > 1, slots = emb ? 1 : ss_slots(w.segs), n = (emb ? ncta : w.slabs) << sh;
+      for (int r = 2 * cw; r < T; r += 2 * kNumCWarps) {   // two rows per warp and step; lanes stride over the CTAs (at most 256), all loads in flight, fixed shuffle tree
         float v0[8], v1[8];
+        const int n0 = ((lane ^ r) & sh) ? 0 : n, n1 = r + 1 >= T || ((lane ^ (r + 1)) & sh) ? 0 : n;   // (CTA j of a pair: rows j, j + 2, ...)
+        const float *q = p.ss_part + r * kSsStride + (lane >> sh) * slots;
+        const int inc = (32 >> sh) * slots;
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
-          const int i = lane + 32 * k;
-          v0[k] = i < nss ? __ldcg(p.ss_part + r * kSsStride + i) : 0.f;
-          v1[k] = i < nss && r + 1 < T ? __ldcg(p.ss_part + (r + 1) * kSsStride + i) : 0.f;
+          v0[k] = lane + 32 * k < n0 ? __ldcg(q + k * inc) : 0.f;
+          v1[k] = lane + 32 * k < n1 ? __ldcg(q + k * inc + kSsStride) : 0.f;
+        }
+        for (int j = 1; j < slots; ++j) {
+          float u0[8], u1[8];
+#pragma unroll
+          for (int k = 0; k < 8; ++k) {
+            u0[k] = lane + 32 * k < n0 ? __ldcg(q + k * inc + j) : 0.f;
+            u1[k] = lane + 32 * k < n1 ? __ldcg(q + k * inc + j + kSsStride) : 0.f;
+          }
+#pragma unroll
+          for (int k = 0; k < 8; ++k) { v0[k] += u0[k]; v1[k] += u1[k]; }
         }
         float s0 = 0.f, s1 = 0.f;
 #pragma unroll
@@ -1863,26 +1884,43 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
       named_bar(3, kNumCWarps * 32);
 #pragma unroll 1
       for (int wi = cw, k = 0; wi < nitem; wi += kNumCWarps, ++k) {
-        const int tq = wi / segs, sg = wi - tq * segs, r = sg * 64 + 2 * lane - odd, t = t0 + tq * tstep;
-        const bool in0 = r >= 0 && r < s.rows, in1 = r + 1 < s.rows;
+        const int tq = wi / segs, sg = wi - tq * segs, r = sg * 64 + 2 * lane, t = t0 + tq * tstep;
+        const bool in0 = r < s.rows, in1 = r + 1 < s.rows;
         float2 hn = k == 0 ? hold[0] : hold[1], gv = k == 0 ? gn[0] : gn[1];
         if (k >= kAhead) item_old(wi, hn, gv);   // (more items than were fetched ahead)
         const float *y = ys + t * 256 + r;
         hn.x = in0 ? hn.x + y[0] : 0.f;
         hn.y = in1 ? hn.y + y[1] : 0.f;
         float *hp = p.h + (size_t)t * p.d + col0 + r;
-        if (in0 && in1) {
+        if (in1 && !odd) {
           *reinterpret_cast<float2 *>(hp) = hn;
           xstore2(p.xa, TP, t, col0 + r, hn.x * gv.x, hn.y * gv.y);
-        } else if (in0) {
-          hp[0] = hn.x;
-          xstore(p.xa, TP, t, col0 + r, hn.x * gv.x);
-        } else if (in1) {
-          hp[1] = hn.y;
-          xstore(p.xa, TP, t, col0 + r + 1, hn.y * gv.y);
+        } else {
+          if (in0) {
+            hp[0] = hn.x;
+            xstore(p.xa, TP, t, col0 + r, hn.x * gv.x);
+          }
+          if (in1) {
+            hp[1] = hn.y;
+            xstore(p.xa, TP, t, col0 + r + 1, hn.y * gv.y);
+          }
         }
-        const float q = warp_sum(hn.x * hn.x + hn.y * hn.y);
-        if (lane == 0) p.ss_part[t * kSsStride + s.group * segs + sg] = q;
+        // squares: each half of the piece as a tree over its 32 columns, the halves of a slab one after the other (those of a second
+        // piece are left apart; ss_slots)
+        float q = __fmul_rn(hn.x, hn.x), q1 = __fmul_rn(hn.y, hn.y);
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) {
+          q += __shfl_xor_sync(0xffffffffu, q, o);
+          q1 += __shfl_xor_sync(0xffffffffu, q1, o);
+        }
+        q += q1;
+        float *ss = p.ss_part + t * kSsStride + s.group * ss_slots(segs);
+        if (sg == 0) {
+          q += __shfl_xor_sync(0xffffffffu, q, 16);
+          if (lane == 0) ss[0] = q;
+        } else if ((lane & 15) == 0) {
+          ss[1 + (lane >> 4)] = q;
+        }
       }
     } else if (epi != EPI_ARGMAX_LM) {
       named_bar(3, kNumCWarps * 32);

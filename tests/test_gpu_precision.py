@@ -10,6 +10,7 @@ The 64-bit reference reads the library's own 16-bit cache, so that no rounding o
 """
 import math
 
+import numpy as np
 import pytest
 import torch
 
@@ -137,3 +138,63 @@ def test_decode_routes(model, measure, lens):
         assert e.ada_get_counters()["status"] == 0
     finally:
         e.close()
+
+
+def _tree(v):
+    """The sum of 32 values as a warp's exchanges make it: pairs 16 apart, then 8, 4, 2, 1."""
+    for o in (16, 8, 4, 2, 1):
+        v = v + v[..., np.arange(32) ^ o]
+    return v[..., 0]
+
+
+def _pass_row_sum(sq, row, width, ctas, pairs):
+    """A row's sum of squares as passes of up to 48 rows form it: per thread block that finishes the row (of a pair that splits K
+    each second row) its columns in groups of 32, the groups in order; the thread blocks 32 apart in order, then a tree."""
+    c = np.zeros(256, dtype=np.float32)
+    for s in range(-(-len(sq) // width)):
+        cols = sq[s * width: (s + 1) * width]
+        cols = np.concatenate([cols, np.zeros(-len(cols) % 32, dtype=np.float32)]).reshape(-1, 32)
+        r = np.float32(0)
+        for g in _tree(cols):
+            r = r + g
+        c[2 * s + row % 2 if pairs else s] = r
+    assert -(-len(sq) // width) * (2 if pairs else 1) <= ctas
+    lanes = np.zeros(32, dtype=np.float32)
+    for k in range(8):
+        lanes = lanes + c[32 * k: 32 * k + 32]
+    return _tree(lanes)
+
+
+@pytest.mark.parametrize("d,ffn,width,pairs", [(256, 128, 4, False), (768, 688, 11, True), (1024, 688, 14, True), (1536, 688, 21, True),
+                                               (4096, 688, 56, True), (4800, 688, 65, True), (5120, 688, 70, True), (8192, 688, 111, True)])
+def test_order_of_a_rows_sum_of_squares(d, ffn, width, pairs):
+    """Its last bit moves a row's scale, and with it 16-bit cache elements: the first rows of a short prompt see few keys, and 7B
+    features move by 2e-4 of their size with another order.  All layers hand the embedding on, so the final norm's input and every
+    square are known; where it holds 1 the features are the row's scale itself."""
+    from paper_2412_18910_b200 import Engine
+    tiny = si.SHAPES["tiny"]
+    hd = 128 if d > 5120 else 64
+    sh = si.scaled(tiny, d_model=d, n_heads=d // hd, head_dim=hd, d_ffn=ffn, n_layers=1)
+    size = {tiny.d_model: d, 2 * tiny.d_model: 2 * d, tiny.d_ffn: ffn}
+
+    def zeros(a):
+        return [zeros(x) for x in a] if isinstance(a, list) else np.zeros([size.get(n, n) for n in a.shape], dtype=np.uint16)
+
+    w = {k: zeros(v[:1] if isinstance(v, list) else v) for k, v in si.make_weights(tiny).items()}
+    w["final_norm"][:] = 0x3F80
+    w["embed"] = si.normal_bf16(5, "order", (sh.vocab, d))
+    w["embed"][:, 0] = 0x3F80
+    ids = si.uniform_ids(7, "order", 48, sh.vocab)
+    e = Engine(sh, w, kv_capacity=512)
+    try:
+        e.prefill(0, ids)
+        got = e.ada_debug_buffer(0, torch.float32, (1, 512, d))[0, :48, 0].clone()
+    finally:
+        e.close()
+    h = si.bf16_bits_to_f32(w["embed"][ids])
+    widest = max(sh.vocab, ffn, 3 * d) * d * 2
+    ctas = min(torch.cuda.get_device_properties(0).multi_processor_count, max(64, widest >> 15)) & ~1
+    assert width == -(-d // (ctas // 2 if pairs else ctas))     # (the width of a thread block's columns at this size)
+    s = np.array([_pass_row_sum(h[t] * h[t], t, width, ctas, pairs) for t in range(48)])
+    want = torch.rsqrt(torch.from_numpy(s / np.float32(d) + np.float32(sh.rms_eps)).to(e.dev))
+    assert torch.equal(got, want), int((got != want).sum())
