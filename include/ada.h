@@ -230,7 +230,7 @@ int ada_get_profile(ada_ctx *ctx, double out[8]);
  * all device memory, code running while another allocator holds the whole GPU, or a latency-bound
  * path where an allocation would stall the device.  Its only scratch, the predictor's hidden
  * activations, lives in a fixed array inside the library image: ADA_STATIC_MAX_HIDDEN floats
- * (16 KiB, and 4 KiB of counts) on every GPU that loads the library, until the process exits.
+ * (16 KiB) on every GPU that loads the library, until the process exits.
  *   z = W2 ReLU(W1 [e ; f] + b1) + b2,  n = argmax(z) + 1 (lowest index among equals)
  * d_w1 [hidden][2*d_model], d_b1 [hidden], d_w2 [n_max][hidden], d_b2 [n_max], d_embed_row [d_model]
  * are bf16; d_feature [d_model] fp32; outputs d_n (one int32) and d_z ([n_max] fp32, optional).
@@ -241,8 +241,7 @@ int ada_get_profile(ada_ctx *ctx, double out[8]);
  * The first call on each device looks up the array's device address (that device must be current);
  * make that first call before any stream capture begins.  All calls on a device share the array,
  * which keeps the previous call's contents (nothing in it needs clearing: each call overwrites
- * what it reads); calls that overlap on the GPU race on it, so order them on one stream: they leave
- * wrong results or none, and the calls after them are right again. */
+ * what it reads); calls that overlap on the GPU race on it, so order them on one stream. */
 #define ADA_STATIC_MAX_HIDDEN 4096
 int ada_ldlp_eval_static(const void *d_w1, const void *d_b1, const void *d_w2, const void *d_b2,
                          const void *d_embed_row, const float *d_feature, int32_t d_model, int32_t hidden,

@@ -9,7 +9,7 @@
 // until the process exits.
 //
 // The array is shared by all calls on a device and keeps what the last call wrote.  Nothing in it has
-// to start at zero: a call overwrites every entry it later reads (the counts beside it do, see g_ldlp_done).  Two calls that overlap on the
+// to start at zero: a call overwrites every entry it later reads.  Two calls that overlap on the
 // GPU (different streams, or threads racing on one device) use the same array and corrupt each
 // other; callers must order them.
 #include <cuda_bf16.h>
@@ -31,48 +31,36 @@ std::atomic<float *> g_scratch_addr[kMaxDevices];   // (zero-initialised; thread
 using ada::kLdlpThreads;
 using ada::kLdlpUnits;
 
-// Blocks that have left their hidden activations, by the number of blocks of a call: a count wraps to zero with the call's last
-// block, and it is whole again even after calls that overlapped, for those that share it add as much each.
-static __device__ unsigned g_ldlp_done[(ADA_STATIC_MAX_HIDDEN + ada::kLdlpUnits - 1) / ada::kLdlpUnits];
-
-// One launch: hidden = ReLU(W1 [e ; f] + b1), four units a block; the block that comes last takes z = W2 hidden + b2, a warp per
-// output, and n = argmax + 1, lowest index among equals.  Bound by the latency of its chain (launch, W1 from HBM, count, hidden
-// from level 2), not by its bytes.  7B widths, calls back to back: 30.7 us with one warp and element-wise loads per hidden unit,
-// 9.1 us with a second launch for the outputs behind this one, 7.5 us so.  Launched with programmatic serialization: the blocks
-// are in place, waiting, when the kernel before them ends (nothing is read or written before that).
+// hidden = ReLU(W1 [e ; f] + b1); the kernel after this one may start its own loads meanwhile.  Launched plainly: the call
+// is ordered behind all that was enqueued before it.  7B widths, whole call: 30.7 us with one warp and element-wise loads per
+// hidden unit; now 8.2 us back to back with the weights in level 2, 13.3 us for one call with them in HBM.  (One launch whose last
+// block takes the outputs: 10.3 and 14.3 us.  With programmatic serialization 7.8 and 14.3, but behind a kernel of the caller's
+// that was itself launched so and ends without waiting, that would start before the kernels in front of it have completed.)
 template <bool VEC>
-__global__ void __launch_bounds__(kLdlpThreads) k_static_predict(const __nv_bfloat16 *w1, const __nv_bfloat16 *b1,
-                                                                 const __nv_bfloat16 *w2, const __nv_bfloat16 *b2,
-                                                                 const __nv_bfloat16 *e, const float *f, int d, int hid, int nmax,
-                                                                 float *hidden, int *n_out, float *z_out) {
-  constexpr int kWarps = kLdlpThreads / 32;
-  __shared__ float zs[ADA_MAX_NMAX];
-  __shared__ int last_s;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+__global__ void __launch_bounds__(kLdlpThreads) k_static_hidden(const __nv_bfloat16 *w1, const __nv_bfloat16 *b1,
+                                                                const __nv_bfloat16 *e, const float *f, int d, int hid,
+                                                                float *hidden) {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  ada::ldlp_hidden_block<VEC>(w1, b1, e, f, d, hid, blockIdx.x * kLdlpUnits, hidden);
+}
+
+// z = W2 hidden + b2, one warp per output; n = argmax + 1, lowest index among equals.  Launched with programmatic
+// serialization behind the kernel above: the weights are requested before it waits for the hidden activations.
+template <bool VEC>
+__global__ void __launch_bounds__(32 * ADA_MAX_NMAX) k_static_out(const float *hidden, const __nv_bfloat16 *w2,
+                                                                  const __nv_bfloat16 *b2, int hid, int nmax, int *n_out,
+                                                                  float *z_out) {
+  __shared__ float zs[ADA_MAX_NMAX];
+  const int c = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  ada::LdlpRow row;
+  const __nv_bfloat16 *w = w2 + (size_t)c * hid;
+  ada::ldlp_out_ahead<VEC>(w, hid, row);
+  const float bias = __bfloat162float(b2[c]);
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  if (blockIdx.x == 0)   // the last block finds W2 in level 2
-    for (int i = threadIdx.x * 64; i < nmax * hid; i += kLdlpThreads * 64) asm volatile("prefetch.global.L2 [%0];" ::"l"(w2 + i));
-  ada::ldlp_hidden_block<VEC>(w1, b1, e, f, d, hid, blockIdx.x * kLdlpUnits, hidden);   // (its first threads store)
-  if (warp == 0) {
-    __syncwarp();
-    if (lane == 0) {
-      unsigned old;
-      asm volatile("atom.acq_rel.gpu.global.inc.u32 %0, [%1], %2;" : "=r"(old) : "l"(g_ldlp_done + (gridDim.x - 1)), "r"(gridDim.x - 1) : "memory");
-      last_s = old == gridDim.x - 1;
-    }
-  }
-  __syncthreads();
-  if (!last_s) return;
-  for (int c = warp; c < nmax; c += kWarps) {
-    ada::LdlpRow row;
-    const __nv_bfloat16 *w = w2 + (size_t)c * hid;
-    ada::ldlp_out_ahead<VEC>(w, hid, row);
-    const float z = ada::ldlp_out_dot<VEC>(w, hidden, hid, row) + __bfloat162float(b2[c]);
-    if (lane == 0) {
-      zs[c] = z;
-      if (z_out) z_out[c] = z;
-    }
+  const float z = ada::ldlp_out_dot<VEC>(w, hidden, hid, row) + bias;
+  if (lane == 0) {
+    zs[c] = z;
+    if (z_out) z_out[c] = z;
   }
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -87,13 +75,14 @@ __global__ void __launch_bounds__(kLdlpThreads) k_static_predict(const __nv_bflo
 template <bool VEC>
 cudaError_t launch(const __nv_bfloat16 *w1, const __nv_bfloat16 *b1, const __nv_bfloat16 *w2, const __nv_bfloat16 *b2,
                    const __nv_bfloat16 *e, const float *f, int d, int hid, int nmax, int *n, float *z, float *hidden, cudaStream_t st) {
+  k_static_hidden<VEC><<<(hid + kLdlpUnits - 1) / kLdlpUnits, kLdlpThreads, 0, st>>>(w1, b1, e, f, d, hid, hidden);
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((hid + kLdlpUnits - 1) / kLdlpUnits); cfg.blockDim = dim3(kLdlpThreads); cfg.stream = st;
+  cfg.gridDim = dim3(1); cfg.blockDim = dim3(32 * nmax); cfg.stream = st;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at; cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_static_predict<VEC>, w1, b1, w2, b2, e, f, d, hid, nmax, hidden, n, z);
+  return cudaLaunchKernelEx(&cfg, k_static_out<VEC>, (const float *)hidden, w2, b2, hid, nmax, n, z);
 }
 
 }  // namespace
