@@ -67,7 +67,7 @@ struct ada_ctx {
   int host_force_n[ADA_MAX_BATCH];
   size_t part_floats;
   // persistent pass kernel: device copies of the layer pointer tables and its scratch
-  int pass_ok, n_sm;   // it can run here: drafts go through it
+  int pass_ok, n_sm;   // it can run here: draft steps of one row per sequence go through it
   int use_pass;        // so do all decode passes (see pass_takes)
   // tensor-core GEMM of the multi-row path (passes of up to 88 rows): tensor maps of every weight matrix and of
   // the activation planes, found by base pointer
@@ -685,9 +685,9 @@ double pass_weight_bytes(const ada_ctx *x, int mode, int prompt) {
 
 // One persistent launch: mode 0, a target pass (embedding, layers, final norm -> features, LM head -> target choices) over
 // the rows of x->pass (at most kPassRowsMax); mode 1, the draft head's steps (fc on [e ; f], its layer, LM head ->
-// draft tokens) up to the longest draft length on the device.
+// draft tokens) from step0 to the longest draft length on the device.
 // prompt: the rows are a short prompt of one sequence (mode 0: the choice after its last row only; mode 1: no LM head).
-void run_pass(ada_ctx *x, int mode, float *logits, int *tok_out, float2 *top_out, const int *forced, int prompt = 0,
+void run_pass(ada_ctx *x, int mode, int step0, float *logits, int *tok_out, float2 *top_out, const int *forced, int prompt = 0,
               int only_seq = -1, int accept = 0) {
   const ada_config &c = x->c;
   PassParams p;
@@ -701,7 +701,7 @@ void run_pass(ada_ctx *x, int mode, float *logits, int *tok_out, float2 *top_out
   p.cache_layers = p.n_layers;
   p.d = c.d_model; p.H = c.n_heads; p.hd = c.head_dim; p.F = c.d_ffn; p.V = c.vocab; p.eps = c.rms_eps;
   p.embed = x->embed; p.final_norm = x->final_norm;
-  p.mode = mode; p.prompt = prompt; p.st = x->st; p.B = x->B; p.tok = x->tok; p.tok_stride = x->seq_stride;
+  p.mode = mode; p.prompt = prompt; p.step0 = step0; p.st = x->st; p.B = x->B; p.tok = x->tok; p.tok_stride = x->seq_stride;
   p.draft = x->draft; p.only_seq = only_seq; p.accept = accept; p.acc_out = x->out_acc; p.emit_out = x->out_emit; p.nemit_out = x->out_nemit;
   p.ddd_thr = mode == 1 && x->B == 1 && !prompt ? c.ddd_threshold : 0.f;   // (packed start positions: full-length drafts)
   p.h = x->h; p.qkv = x->qkv; p.ss_part = x->ss_part;
@@ -757,25 +757,28 @@ void enqueue_ldlp(ada_ctx *x, int *d_n) {
 
 void enqueue_draft(ada_ctx *x) {
   const ada_config &c = x->c;
-  // The steps are one persistent launch and follow each other on the device, as many as the longest draft asks for; the first one
-  // takes several passes where its catch-up rows (up to n_max + 1 of every sequence) are more than a pass holds.  Step by step
-  // through the multi-row path, which models remain on whose slabs the kernel does not hold, a batch pays 17 launches a step, needed
-  // or not: 8 sequences on the 7B shape 225 us a step that ran and 50 us one that did not, small model 70 and 37 us.  (With
-  // only its first step there, five steps: 1131 us on the 7B shape, now 1104; middle model 589 -> 579.)
-  if (x->pass_ok) {
-    run_pass(x, 1, nullptr, x->draft, x->dtop, x->force_draft);
-    return;
+  // The steps are one persistent launch and follow each other on the device, as many as the longest draft asks for; the first
+  // step of a batch whose catch-up rows (up to n_max + 1 of every sequence) a persistent pass may not hold takes the multi-row
+  // path.  Step by step through the multi-row path a batch paid 17 launches a step, needed or not: 8 sequences on the 7B
+  // shape 225 us a step that ran and 50 us one that did not, small model 70 and 37 us.  (The first step in the persistent kernel
+  // too, in passes of whole sequences, as its rows are known on the device only: five steps of 8 sequences with a row each 1131 ->
+  // 1104 us on the 7B shape, but one step behind 88 rows, two passes, 268 -> 415; in one pass, 5 sequences of 16 layers of 2048, a
+  // row each at context 100 133 -> 112, nine rows each at context 1850 160 -> 179.)
+  int step = 0;
+  if (!x->use_pass) {
+    const int multi = x->pass_ok ? 1 : c.n_max;
+    for (; step < multi; ++step) {
+      LAUNCH(x, k_rows_draft, 1, 32, 0, x->pass, x->st, x->tok, x->seq_stride, x->draft, c.n_max, x->B, step, x->TM, x->cnt);
+      draft_rows(x, step, true);
+    }
   }
-  for (int step = 0; step < c.n_max; ++step) {
-    LAUNCH(x, k_rows_draft, 1, 32, 0, x->pass, x->st, x->tok, x->seq_stride, x->draft, c.n_max, x->B, step, x->TM, x->cnt);
-    draft_rows(x, step, true);
-  }
+  if (step < c.n_max) run_pass(x, 1, step, nullptr, x->draft, x->dtop, x->force_draft);
 }
 
 void enqueue_verify(ada_ctx *x, int only_seq, float *d_logits, bool accept = false) {
   const ada_config &c = x->c;
   if (x->use_pass) {
-    run_pass(x, 0, d_logits, x->target, x->vtop, nullptr, 0, only_seq, accept ? 1 : 0);
+    run_pass(x, 0, 0, d_logits, x->target, x->vtop, nullptr, 0, only_seq, accept ? 1 : 0);
     return;
   }
   LAUNCH(x, k_rows_verify, 1, 32, 0, x->pass, x->st, x->tok, x->seq_stride, c.kv_capacity, x->draft, c.n_max, x->B, only_seq);
@@ -862,10 +865,10 @@ void enqueue_prompt(ada_ctx *x, int seq, int m, int chunk) {
   x->prompt_seq = seq;
   if (m <= kPassRowsMax && x->pass_ok) {   // few rows: a persistent pass each for the target and the draft head
     LAUNCH(x, k_rows_chunk, 1, 256, 0, x->pass, x->tok, c.kv_capacity, seq, 0, m, 0, x->B, chunk);
-    run_pass(x, 0, nullptr, x->chunk_tok, x->vtop + x->B * (c.n_max + 1), nullptr, 1);
+    run_pass(x, 0, 0, nullptr, x->chunk_tok, x->vtop + x->B * (c.n_max + 1), nullptr, 1);
     if (m > 1) {
       LAUNCH(x, k_rows_chunk, 1, 256, 0, x->pass, x->tok, c.kv_capacity, seq, 0, m - 1, 1, x->B, chunk);
-      run_pass(x, 1, nullptr, nullptr, nullptr, nullptr, 1);
+      run_pass(x, 1, 0, nullptr, nullptr, nullptr, nullptr, 1);
     }
     x->prompt_seq = -1;
     return;

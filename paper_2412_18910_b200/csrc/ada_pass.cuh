@@ -120,9 +120,6 @@ struct PassRows {
   // draft steps: per sequence its draft length, pending position, first catch-up position, split size and newest draft token
   int n[kMaxBatch], j[kMaxBatch], p0[kMaxBatch], chunk[kMaxBatch], cur[kMaxBatch];
   float lp, cum;                        // log-probability of the newest token, of the draft (stopping rule)
-  // Catch-up rows (step 0) that one pass does not hold go through several, whole sequences each: how many more than one, the pass
-  // of a sequence, the padded rows of each pass.  (A row's result does not depend on the rows beside it.)
-  int extra, part[kMaxBatch], part_TP[4];
 };
 enum { MAP_WQ = 0, MAP_WK, MAP_WV, MAP_WO, MAP_WG, MAP_WU, MAP_WD };
 
@@ -137,9 +134,10 @@ struct PassParams {
   int d, H, hd, F, V;
   float eps;
   const __nv_bfloat16 *embed, *final_norm;
-  int mode;                    // 0 target pass over the pending tokens and drafts, 1 draft-head steps 0 .. (longest draft length) - 1
+  int mode;                    // 0 target pass over the pending tokens and drafts, 1 draft-head steps step0 .. (longest draft length) - 1
   int prompt;                  // 1: the rows of `pass` are a short prompt of one sequence (mode 0: greedy choice after the last
                                // row; mode 1: the draft head over its rows, no LM head)
+  int step0;                   // draft: first step of this launch (0: catch-up rows of the one sequence)
   SeqState *st; int B;         // lengths and draft lengths of the sequences
   int *tok; int tok_stride;    // committed tokens, and positions between two sequences in tok and feat
   const int *draft;            // target pass: draft tokens [seq][nmax]
@@ -677,14 +675,13 @@ __device__ __noinline__ int await_length(uint64_t *step_bar, unsigned &decisions
   return *reinterpret_cast<const volatile int *>(&rows->n[0]);
 }
 
-// Rows of pass v of the draft head (Eq. 2; one thread).  Step 0 (passes 0 .. extra): the catch-up rows p = p0 .. j - 1 of the
-// sequences, row p pairs the target feature of p with the embedding of token p + 1, a sequence's last row feeds the LM head.  Step
-// s >= 1 (pass extra + s): one row per sequence with n > s at position j + s - 1, its token the newest draft token.
-__device__ __noinline__ void draft_rows_of_pass(PassRows *r, const PassParams &p, int v) {
-  const int step = max(0, v - r->extra);
+// Rows of draft step `step` (Eq. 2; one thread).  Step 0: the catch-up rows p = p0 .. j - 1 of every sequence, row p pairs
+// the target feature of p with the embedding of token p + 1, a sequence's last row feeds the LM head.  Step s >= 1: one row per
+// sequence with n > s at position j + s - 1, its token the newest draft token.
+__device__ __noinline__ void draft_rows_of_step(PassRows *r, const PassParams &p, int step) {
   int T = 0, ns = 0;
   for (int b = 0; b < p.B; ++b) {
-    if (r->n[b] <= step || (v <= r->extra && r->part[b] != v)) continue;
+    if (r->n[b] <= step) continue;
     const int first = step == 0 ? r->p0[b] : r->j[b] + step - 1, R = step == 0 ? r->j[b] - first : 1;
     r->s_b[ns] = b; r->s_row0[ns] = T; r->s_rows[ns] = R; r->s_pos0[ns] = first; r->s_chunk[ns] = r->chunk[b];
     for (int i = 0; i < R; ++i, ++T) {
@@ -739,12 +736,14 @@ __device__ __noinline__ void verify_rows(PassRows *r, const PassParams &p, bool 
   }
 }
 
-// First catch-up position of a sequence that takes part in the draft steps, -1 for one that does not: no draft asked for, or more rows behind than a pass holds of a sequence.  One that is up
+// First catch-up position of a sequence that takes part in the draft steps of this launch (0 if the launch has no catch-up
+// step), -1 for one that does not: no draft asked for, or more rows behind than a pass holds of a sequence.  One that is up
 // to date (a second draft from the same state, e.g. after a label pass) computes the row of position j - 1 again -- same
 // inputs, same cache row -- because its output yields the first draft token.
 __device__ __forceinline__ int draft_first(const PassParams &p, const SeqState &q) {
   const int j = q.len - 1;
-  if (q.n <= 0 || j < 1) return -1;
+  if (q.n <= p.step0 || j < 1) return -1;
+  if (p.step0 > 0) return 0;
   const int p0 = q.dlen == j ? j - 1 : q.dlen;
   return j - p0 < 1 || j - p0 > p.nmax + 1 || q.stale ? -1 : p0;
 }
@@ -795,39 +794,34 @@ template <bool PROMPT>
 __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant__ PassParams p) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int cta = blockIdx.x, ncta = gridDim.x;
-  // Passes of the launch: the target's one, or the draft head's for the steps up to the longest draft length (with the stopping
-  // rule the length grows while the kernel runs, see `step_bar`), `extra` more where step 0 takes several.  Every thread reads the
-  // states here; CTA 0 changes them after the first grid barrier only.
-  int npass = 0, extra = 0;
+  // Steps of the launch: the target's one pass, or the draft steps step0 .. the longest draft length (with the stopping
+  // rule the length grows while the kernel runs, see `step_bar`).  Every thread reads the states here; CTA 0 changes them
+  // after the first grid barrier only.
+  int nstep = 0;
   if (PROMPT) {
-    npass = p.pass->T > 0 ? 1 : 0;
+    nstep = p.pass->T > 0 ? 1 : 0;
   } else if (p.mode == 0) {
     for (int b = 0; b < p.B; ++b) {
       const int len = p.st[b].len, n = p.st[b].n;
-      if ((p.only_seq < 0 || b == p.only_seq) && len >= 1 && len + n + 1 <= p.cap) npass = 1;
+      if ((p.only_seq < 0 || b == p.only_seq) && len >= 1 && len + n + 1 <= p.cap) nstep = 1;
     }
     // no sequence takes part: nothing to verify, and accepting reports just that
-    if (!npass && p.accept && cta == 0 && tid < p.B)
+    if (!nstep && p.accept && cta == 0 && tid < p.B)
       accept_sequence(p.st, p.tok, p.cap, p.tok_stride, nullptr, nullptr, p.nmax, tid, p.cnt, nullptr, 0, p.acc_out, p.emit_out,
                       p.nemit_out, nullptr);
   } else {
-    int T = 0;
     for (int b = 0; b < p.B; ++b) {
       const SeqState q = p.st[b];
-      const int p0 = draft_first(p, q);
-      if (p0 < 0) {
-        if (q.n > 0 && q.len > 1 && cta == 0 && tid == 0) { p.st[b].n = 0; atomicOr(&p.cnt->status, kStatStale); }
+      if (draft_first(p, q) < 0) {
+        if (q.n > p.step0 && q.len > 1 && cta == 0 && tid == 0) { p.st[b].n = 0; atomicOr(&p.cnt->status, kStatStale); }
         continue;
       }
-      npass = max(npass, q.n);
-      const int R = q.len - 1 - p0;
-      if (T + R > kPassRowsMax) { T = 0; ++extra; }
-      T += R;
+      nstep = max(nstep, q.n);
     }
-    npass += extra;
   }
-  if (!PROMPT && p.steps_out && npass == 0 && cta == 0 && tid == 0) *p.steps_out = 0;
-  if (npass == 0) return;
+  const int first_step = p.mode == 0 || PROMPT ? 0 : p.step0;
+  if (!PROMPT && p.steps_out && nstep <= first_step && cta == 0 && tid == 0) *p.steps_out = 0;
+  if (nstep <= first_step) return;
 
   extern __shared__ __align__(128) unsigned char pass_smem[];
   // swizzled TMA boxes need 1024-byte aligned bases
@@ -897,21 +891,10 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
         rows->j[lane] = q.len - 1;
         rows->p0[lane] = p0;
         rows->chunk[lane] = max(32, q.chunk);
+        rows->cur[lane] = first_step > 0 ? __ldcg(p.tok_out + lane * p.nmax + first_step - 1) : 0;
       }
       __syncwarp();
-      if (lane == 0) {
-        int T = 0, v = 0;
-        for (int b = 0; b < p.B; ++b) {
-          if (rows->n[b] <= 0) continue;
-          const int R = rows->j[b] - rows->p0[b];
-          if (T + R > kPassRowsMax) { T = 0; ++v; }
-          T += R;
-          rows->part[b] = v;
-          rows->part_TP[v] = (T + 7) & ~7;
-        }
-        rows->extra = v;
-        draft_rows_of_pass(rows, p, 0);
-      }
+      if (lane == 0) draft_rows_of_step(rows, p, first_step);
     }
   }
   tc_fence_before();
@@ -936,9 +919,9 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
     RingRetire rr;   // both producers place and retire every stage of the schedule (see ada_ring.h)
     rr.init();
     const uint64_t pol_w = l2_policy_evict_first();   // weights are read once per pass
-    const int TP0 = *reinterpret_cast<const volatile int *>(&rows->TP);   // (the rows of the first pass)
+    const int TP0 = *reinterpret_cast<const volatile int *>(&rows->TP);
     unsigned decisions = 0;
-    for (int v = 0; v < npass || (p.ddd_thr < 0.f && v < await_length(step_bar, decisions, rows, p.cnt, abort_s)); ++v)
+    for (int step = first_step; step < nstep || (p.ddd_thr < 0.f && step < await_length(step_bar, decisions, rows, p.cnt, abort_s)); ++step)
     for (int ph = 0; ph < nphase && !*abort_s; ++ph) {
       int layer;
       const int kind = phase_kind(p, ph, layer);
@@ -954,8 +937,8 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
       map1 += map_base(p, kind, layer);
       const unsigned long long m0 = reinterpret_cast<unsigned long long>(p.maps + map0);
       const unsigned long long m1 = reinterpret_cast<unsigned long long>(p.maps + map1);
-      // (a stage holds no more boxes than an activation buffer of the pass; the steps after the first have one row per sequence)
-      const int region = s.region, kb = min(s.kb, xbuf_boxes(v > extra ? 8 : v > 0 ? rows->part_TP[v] : TP0)), mtiles = s.mtiles, K = g.K, c0 = s.c0, c1 = s.c1;
+      // (a stage holds no more boxes than an activation buffer of the step; the steps after the first have one row per sequence)
+      const int region = s.region, kb = min(s.kb, xbuf_boxes(step == first_step ? TP0 : 8)), mtiles = s.mtiles, K = g.K, c0 = s.c0, c1 = s.c1;
       int c = c0 + s.rot;
       const unsigned tx_box = (unsigned)(s.box_rows * 128);
       for (int i = c0; i < c1; ++i, c = c + 1 == c1 ? c0 : c + 1) {
@@ -1002,13 +985,13 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
       // depend on is therefore worked out from the launch's parameters, or passes through a warp reduction, whose result the
       // compiler knows to be uniform; with a slab description or a step count read from memory each product took 80 cycles
       // to issue instead of 45, and the loops were bound by it (7B, 5 rows: QKV 22 400 of its 28 800 cycles).
-      const int npasses = (int)__reduce_max_sync(0xffffffffu, (unsigned)npass);
+      const int nsteps = (int)__reduce_max_sync(0xffffffffu, (unsigned)nstep);
       unsigned decisions = 0;
       uint32_t sphase = 0;     // per place of the accumulators the parity of its next release in this phase
-      for (int v = 0;
-           v < npasses || (p.ddd_thr < 0.f && v < (int)__reduce_max_sync(0xffffffffu, (unsigned)await_length(step_bar, decisions, rows, p.cnt, abort_s)));
-           ++v, xslot = 0) {
-      unsigned tp = 0;         // padded rows of the pass
+      for (int step = first_step;
+           step < nsteps || (p.ddd_thr < 0.f && step < (int)__reduce_max_sync(0xffffffffu, (unsigned)await_length(step_bar, decisions, rows, p.cnt, abort_s)));
+           ++step, xslot = 0) {
+      unsigned tp = 0;         // padded rows of the step
       for (int ph = 0; ph < nphase; ++ph) {
         int layer;
         const int kind = phase_kind(p, ph, layer);
@@ -1018,7 +1001,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
         const Slab s = make_slab(g, cta, ncta);
         const int K = g.K;
         if (s.rows == 0) continue;
-        if (tp == 0) {   // (the rows of the pass are known once its first activations have landed)
+        if (tp == 0) {   // (the rows of the step are known once its first activations have landed)
           mbar_wait(&xfull[xslot], (xphase >> xslot) & 1u, p.cnt, abort_s);
           tp = __reduce_max_sync(0xffffffffu, (unsigned)*reinterpret_cast<const volatile int *>(&rows->TP));
         }
@@ -1183,11 +1166,11 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
     const uint64_t pol_x = l2_policy_evict_last();   // (every CTA reads the same input tiles)
     uint32_t xused = 0, xphase = 0;                  // buffers used before, parity of their next release
     unsigned target = 0, epoch = 0;
-    for (int v = 0; v < npass; ++v) {
+    for (int step = first_step; step < nstep; ++step) {
       const int TP = *reinterpret_cast<const volatile int *>(&rows->TP);
-      const int kxb = xbuf_boxes(TP), nx = xbuf_count(TP);    // boxes per buffer, buffers (of this pass)
+      const int kxb = xbuf_boxes(TP), nx = xbuf_count(TP);    // boxes per buffer, buffers (of this step)
       const unsigned xbytes = (unsigned)xbuf_bytes(TP);
-      int xslot = 0;   // (all buffers are free between passes)
+      int xslot = 0;   // (all buffers are free between steps)
       const __nv_bfloat16 *src = nullptr;
       int beg = 0, end = 0, b = 0, parts = 0;        // boxes of this CTA's part of K, the next one, copies to make
       for (int ph = 0; ph < nphase; ++ph) {
@@ -1240,13 +1223,13 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
           }
         }
       }
-      if (p.mode == 1 && !PROMPT) {   // the next pass's rows, and whether there is one
+      if (p.mode == 1 && !PROMPT) {   // the next step's rows, and whether there is one
         named_bar(6, kBarThreads);
-        if (p.ddd_thr < 0.f) npass = *reinterpret_cast<const volatile int *>(&rows->n[0]);
+        if (p.ddd_thr < 0.f) nstep = *reinterpret_cast<const volatile int *>(&rows->n[0]);
       }
     }
     if (lane == 0) {
-      if (!PROMPT && p.steps_out && cta == 0) *p.steps_out = npass;
+      if (!PROMPT && p.steps_out && cta == 0) *p.steps_out = nstep - first_step;
       // the last CTA to leave clears the barrier count for the next launch (all have passed the last barrier)
       if (atomicAdd(p.gbar + 16, 1u) == (unsigned)ncta - 1u) {
         p.gbar[0] = 0;
@@ -1285,8 +1268,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
   unsigned kuses = 0;               // completed phases of the K-split pair barrier
   uint32_t sphase = 0;              // per place of the accumulators the parity of its next section of this phase
 
-  for (int v = 0; v < npass; ++v) {
-  const int step = max(0, v - extra);   // draft step
+  for (int step = first_step; step < nstep; ++step) {
   const int T = rows->T, lmT = rows->lmT, TP = rows->TP;
   bool arrived = false;             // at a grid barrier whose release has not been awaited
   for (int ph = 0; ph < nphase; ++ph) {
@@ -1809,7 +1791,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
     const int t_end = sw ? 2 * TP : TP;                  // (SwiGLU: the gate rows, then the up rows)
     if (s.nsec > 1 && s.rows > 0) sphase = add_sections(secfull, secempty, sphase, s.nsec, active_warp ? t_end : 0, TP, taddr, place, sums, p.cnt, abort_s);
     // (the cache rows of the draft steps before this one, under the products)
-    if (kind == PH_QKV && v > 0 && lane == 0) fence_global_copies();
+    if (kind == PH_QKV && step > first_step && lane == 0) fence_global_copies();
     if (s.rows > 0) {
       mbar_wait(accfull, acc_phase & 1u, p.cnt, abort_s);
       ++acc_phase;
@@ -2068,7 +2050,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
   if (p.mode == 1 && !PROMPT) {
     named_bar(3, kNumCWarps * 32);
     if (ctid == 0) {
-      const int made = v + 1;               // passes (with the stopping rule: steps)
+      const int made = step + 1;
       int n = rows->n[0];
       if (p.ddd_thr < 0.f && made >= n) {
         // the running log-probability takes the new token's; at the predicted length and still at or above the
@@ -2081,17 +2063,17 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
       } else if (p.ddd_thr < 0.f) {
         rows->cum = (step == 0 ? 0.f : rows->cum) + rows->lp;
       }
-      if (p.ddd_thr < 0.f ? made < n : made < npass) draft_rows_of_pass(rows, p, made);
+      if (p.ddd_thr < 0.f ? made < n : made < nstep) draft_rows_of_step(rows, p, made);
       else if (cta == 0) {   // the draft is complete
         for (int b = 0; b < p.B; ++b)
-          if (rows->n[b] > 0) {
+          if (rows->n[b] > 0 && p.step0 == 0) {
             p.st[b].dlen = rows->j[b];
             if (p.ddd_thr < 0.f) p.st[b].n = n;
           }
       }
     }
     named_bar(6, kBarThreads);
-    if (p.ddd_thr < 0.f) npass = rows->n[0];
+    if (p.ddd_thr < 0.f) nstep = rows->n[0];
   }
   if (arrived) phase_await();   // (a prompt's pass of the draft head ends with its layer)
   }

@@ -105,8 +105,8 @@ def test_step_ends_as_its_parts_do_when_sequences_fill_up():
 
 @pytest.mark.parametrize("batch", [5, 6, 8])
 def test_catch_up_rows_of_more_than_one_pass(tiny, batch):
-    """Drafts after nine tokens were committed in every sequence: 45, 54 and 72 catch-up rows, which the draft head takes in one
-    pass of up to 48 rows or in two (of five sequences and the others)."""
+    """Drafts after nine tokens were committed in every sequence: 45, 54 and 72 catch-up rows, which the draft head takes in a
+    persistent pass of up to 48 rows or on the multi-row path."""
     import oracle
     from paper_2412_18910_b200 import Engine
     sh, w, _, m = tiny
