@@ -830,14 +830,14 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
   uint64_t *bars = reinterpret_cast<uint64_t *>(smem + kRingBytes);
   uint64_t *full = bars, *empty = bars + kSlots, *xfull = bars + 2 * kSlots, *xempty = bars + 2 * kSlots + kXBufs;
   float *inv_rms = reinterpret_cast<float *>(bars + 2 * kSlots + 2 * kXBufs + 8 + 2 * kNumCWarps);   // [rows] (after the single barriers)
-  float *ssw = inv_rms + kPassRowsMax;                                             // [rows][8] (log-probabilities: [8][16])
-  int *flag_s = reinterpret_cast<int *>(ssw + 8 * kPassRowsMax);
+  float *lps = inv_rms + kPassRowsMax;                                             // [8][16] sums of exponentials, for log-probabilities (one sequence)
+  int *flag_s = reinterpret_cast<int *>(lps + kNumCWarps * 16);
   volatile int *abort_s = flag_s + 1;
   unsigned char *xbuf = smem + kRingBytes + kMiscBytes;
   float *red = reinterpret_cast<float *>(xbuf + kXBytes);   // [rows / 8][128 threads][4 rows] sums of the K-split pair's other CTA
   Top2 *topw = reinterpret_cast<Top2 *>(red);   // [8][rows] (LM head, which has no pairs)
   static_assert(8 * kPassRowsMax * sizeof(Top2) <= kRedBytes, "room for the warps' candidates");
-  static_assert((2 * kSlots + 2 * kXBufs + 8 + 2 * kNumCWarps) * 8 + 9 * kPassRowsMax * 4 + 16 + 4 * kFlight * 4 + sizeof(PassRows) + 8 + kPhaseGemms * sizeof(PhaseGemm) <= kMiscBytes, "misc area");
+  static_assert((2 * kSlots + 2 * kXBufs + 8 + 2 * kNumCWarps) * 8 + (kPassRowsMax + kNumCWarps * 16) * 4 + 16 + 4 * kFlight * 4 + sizeof(PassRows) + 8 + kPhaseGemms * sizeof(PhaseGemm) <= kMiscBytes, "misc area");
 
   uint64_t *accfull = xempty + kXBufs;                     // accumulator of the phase complete
   uint64_t *attn_bar = accfull + 1;                        // attention: per worker warp, its 16 keys and its 16 values have landed
@@ -1806,8 +1806,8 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
     }
     stamp(p, ph, 2, stamper);
     // The sums go through shared memory (the activation buffers are idle once the accumulator is complete), by pass row and
-    // slab row, so that all eight warps take part however few rows the slab has: a warp finishes 32 columns of one pass row
-    // per step.  (Each thread walking the pass rows of its own weight row took 0.18 us a row.)
+    // slab row, so that all eight warps take part however few rows the slab has (see nflat and nitem above).  (Each thread walking
+    // the pass rows of its own weight row took 0.18 us a row.)
     //
     // K-split pair = the two CTAs of a cluster (same slab, same thread <-> row mapping): each finishes half of the pass rows
     // (CTA j of the pair rows j, j + 2, ...).  A thread sends its sums of the other rows into the peer's shared memory, to an
@@ -1948,7 +1948,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
           // for the log-probability of the chosen token: sum of exp(logit - warp maximum), and the logit of a
           // forced token where one is given
           const float e = warp_sum(valid ? __expf(y - b.v1) : 0.f);
-          if (lane == 0) ssw[cw * 16 + t] = e;
+          if (lane == 0) lps[cw * 16 + t] = e;
           if (valid && p.forced) {
             const int slot_out = g.lm_rows ? rows->lm_out[t] : rows->out[t];
             if (p.forced[slot_out] == vrow) p.tok_logit[slot_out] = y;
@@ -1965,7 +1965,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
         if (p.lp_out)
           for (int w = 0; w < kNumCWarps; ++w) {
             const float mw = topw[w * kPassRowsMax + ctid].v1;
-            if (mw > -INFINITY) se += ssw[w * 16 + ctid] * __expf(mw - b.v1);
+            if (mw > -INFINITY) se += lps[w * 16 + ctid] * __expf(mw - b.v1);
           }
         p.amax[(size_t)cta * kPassRowsMax + ctid] = make_float4(b.v1, __int_as_float(b.i1), b.v2, se);
       }

@@ -130,6 +130,34 @@ def test_catch_up_rows_of_more_than_one_pass(tiny, batch):
         e.close()
 
 
+@pytest.mark.parametrize("batch,wider", [(1, dict(vocab=40960)), (6, dict(vocab=40960)), (2, dict(d_ffn=19200))])
+def test_models_that_the_persistent_pass_does_not_hold(batch, wider):
+    """Vocabularies above 37 888 and d_ffn above 18 944 (256 and 128 columns for each of 148 thread blocks): prompts, every draft step
+    and verify passes on the multi-row path."""
+    import oracle
+    from paper_2412_18910_b200 import Engine
+    sh = si.scaled(si.SHAPES["tiny"], **wider)
+    w = si.make_weights(sh)
+    m = oracle.Model(sh, w)
+    e = Engine(sh, w, max_batch=batch, kv_capacity=256)
+    try:
+        seqs = []
+        for b in range(batch):
+            prompt = si.uniform_ids(81 + b, "wide%d" % b, 9 + 31 * b, sh.vocab)
+            seq = m.new_seq(256)
+            assert seq.prefill(prompt) == e.prefill(b, prompt)
+            seqs.append(seq)
+        e.ada_force_n([8] * batch)
+        res = lockstep.run_lockstep(e, seqs, 2, n_forced=8)
+        assert not res["failures"], res["failures"]
+        e.ada_force_n(None)
+        res = lockstep.run_lockstep(e, seqs, 3)
+        assert not res["failures"], res["failures"]
+        assert e.ada_get_counters()["status"] == 0
+    finally:
+        e.close()
+
+
 @pytest.mark.parametrize("vocab", [4096, 5120, 9216, 9728])
 def test_small_models_on_part_of_the_chip(vocab):
     """Widths around the 64 thread blocks that the smallest models run on, between them and all of the chip, and on either
@@ -154,10 +182,10 @@ def test_small_models_on_part_of_the_chip(vocab):
         e.close()
 
 
-@pytest.mark.parametrize("d,heads,ffn,batch", [(192, 3, 144, 2), (1088, 17, 400, 2), (4672, 73, 128, 1)])
+@pytest.mark.parametrize("d,heads,ffn,batch", [(192, 3, 144, 2), (1088, 17, 400, 2), (4672, 73, 128, 1), (4800, 75, 128, 1)])
 def test_slabs_of_odd_widths(d, heads, ffn, batch):
-    """Slabs that start on odd columns, thread blocks without a slab, pieces of 64 columns that a slab fills in part or that
-    spill into a second piece (64 rows a pair of thread blocks at the largest width), K outside whole chunks."""
+    """Slabs that start on odd columns, thread blocks without a slab, pieces of 64 columns that a slab fills in part, wholly, or
+    with a column in a second piece (64 and 65 columns a pair of thread blocks at the largest widths), K outside whole chunks."""
     import oracle
     from paper_2412_18910_b200 import Engine
     sh = si.scaled(si.SHAPES["tiny"], n_layers=1, d_model=d, n_heads=heads, head_dim=64, d_ffn=ffn, vocab=272)
