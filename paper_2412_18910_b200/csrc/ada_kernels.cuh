@@ -88,7 +88,8 @@ __device__ __forceinline__ float kv_hi(uint32_t pair) { return __half2float(__us
 // the row list (Pass, page table): the chain of a pass begins with a kernel that is launched plainly after the one that makes the
 // list and lets none start before it has completed, and the list is rewritten only after the chain.  (A kernel's lookups one behind
 // the other, 0.4 to 1 us of its 3, then go on while the one before it finishes, and so do the first copies of old cache rows.  Verify
-// of eight sequences: 16 layers of 2048 1229 -> 1122 us, 7B 4880 -> 4835 us.)
+// of eight sequences: 16 layers of 2048 1242 -> 1134 us, 7B 4531 and 4530.  Prompts of 49 and 64 rows: 16 layers of 2048 1227 -> 1138
+// and 1250 -> 1165 us, 13B 7168 -> 7038 and 7236 -> 7254, 7B 4125 -> 4167 and 4261 -> 4262.)
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
