@@ -15,6 +15,7 @@
 
 #include "ada_kernels.cuh"
 #include "ada_pass.cuh"
+#include "ada_small.cuh"
 #include "ada_gemm_tc.cuh"
 #include "ada_gemm_pair.cuh"
 #include "ada_attn_rows.cuh"
@@ -69,6 +70,8 @@ struct ada_ctx {
   // persistent pass kernel: device copies of the layer pointer tables and its scratch
   int pass_ok, n_sm;   // it can run here: draft steps of one row per sequence go through it
   int use_pass;        // so do all decode passes (see pass_takes)
+  int small;           // they run on a cluster of 16 CTAs per sequence instead (see small_takes)
+  SmallShape small_shape;
   // tensor-core GEMM of the multi-row path (passes of up to 88 rows): tensor maps of every weight matrix and of
   // the activation planes, found by base pointer
   TensorMap128 *d_tcmaps;
@@ -687,8 +690,8 @@ double pass_weight_bytes(const ada_ctx *x, int mode, int prompt) {
 // the rows of x->pass (at most kPassRowsMax); mode 1, the draft head's steps (fc on [e ; f], its layer, LM head ->
 // draft tokens) from step0 to the longest draft length on the device.
 // prompt: the rows are a short prompt of one sequence (mode 0: the choice after its last row only; mode 1: no LM head).
-void run_pass(ada_ctx *x, int mode, int step0, float *logits, int *tok_out, float2 *top_out, const int *forced, int prompt = 0,
-              int only_seq = -1, int accept = 0) {
+PassParams pass_params(ada_ctx *x, int mode, int step0, float *logits, int *tok_out, float2 *top_out, const int *forced, int prompt = 0,
+                       int only_seq = -1, int accept = 0) {
   const ada_config &c = x->c;
   PassParams p;
   memset(&p, 0, sizeof(p));
@@ -715,6 +718,11 @@ void run_pass(ada_ctx *x, int mode, int step0, float *logits, int *tok_out, floa
   p.gbar = x->gbar; p.cnt = x->cnt;
   p.lp_out = p.ddd_thr < 0.f ? x->dlp : nullptr; p.tok_logit = x->dfl;
   p.phase_ns = (x->prof && mode == 0) ? x->phase_ns : nullptr;
+  return p;
+}
+void run_pass(ada_ctx *x, int mode, int step0, float *logits, int *tok_out, float2 *top_out, const int *forced, int prompt = 0,
+              int only_seq = -1, int accept = 0) {
+  PassParams p = pass_params(x, mode, step0, logits, tok_out, top_out, forced, prompt, only_seq, accept);
   // a launch of draft steps streams the head once per step that runs: the kernel leaves their number in the record's place
   const bool steps = mode == 1 && !prompt;
   if (x->prof && steps && x->ev_used + 2 <= (int)x->ev_pool.size()) p.steps_out = x->prof_steps + x->ev_used / 2;
@@ -734,6 +742,29 @@ void run_pass(ada_ctx *x, int mode, int step0, float *logits, int *tok_out, floa
     lc.attrs = at; lc.numAttrs = noncoop ? 1 : 2;
     if (prompt) cudaLaunchKernelEx(&lc, k_pass<true>, p);
     else cudaLaunchKernelEx(&lc, k_pass<false>, p);
+    x->launches++;
+  });
+}
+
+// All draft steps (mode 1), or the verify pass (mode 0), of a small model: a cluster of 16 thread blocks per sequence.
+typedef void (*SmallKernel)(const PassParams, const SmallShape);
+SmallKernel small_kernel(int mode) { return mode ? k_small<true> : k_small<false>; }
+void run_small(ada_ctx *x, int mode, PassParams &p) {
+  const bool steps = mode == 1 && x->prof && x->ev_used + 2 <= (int)x->ev_pool.size();
+  if (steps) {   // profiles: the kernel leaves the number of steps in the record's place
+    p.steps_out = x->prof_steps + x->ev_used / 2;
+    cudaMemsetAsync(p.steps_out, 0, sizeof(int), x->stream);
+  }
+  timed(x, mode == 1 ? kProfDraft : 0, pass_weight_bytes(x, mode, 0), [&] {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(kSmCtas * p.B); cfg.blockDim = dim3(kSmThreads); cfg.dynamicSmemBytes = x->small_shape.total; cfg.stream = x->stream;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = kSmCtas; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = x->pdl;
+    cfg.attrs = at; cfg.numAttrs = 2;
+    cudaLaunchKernelEx(&cfg, small_kernel(mode), p, x->small_shape);
     x->launches++;
   });
 }
@@ -764,6 +795,10 @@ void enqueue_draft(ada_ctx *x) {
   // too, in passes of whole sequences, as its rows are known on the device only: five steps of 8 sequences with a row each 1131 ->
   // 1104 us on the 7B shape, but one step behind 88 rows, two passes, 268 -> 415; in one pass, 5 sequences of 16 layers of 2048, a
   // row each at context 100 133 -> 112, nine rows each at context 1850 160 -> 179.)
+  if (x->small) {
+    PassParams p = pass_params(x, 1, 0, nullptr, x->draft, x->dtop, x->force_draft);
+    return run_small(x, 1, p);
+  }
   int step = 0;
   if (!x->use_pass) {
     const int multi = x->pass_ok ? 1 : c.n_max;
@@ -777,6 +812,10 @@ void enqueue_draft(ada_ctx *x) {
 
 void enqueue_verify(ada_ctx *x, int only_seq, float *d_logits, bool accept = false) {
   const ada_config &c = x->c;
+  if (x->small) {
+    PassParams p = pass_params(x, 0, 0, d_logits, x->target, x->vtop, nullptr, 0, only_seq, accept ? 1 : 0);
+    return run_small(x, 0, p);
+  }
   if (x->use_pass) {
     run_pass(x, 0, 0, d_logits, x->target, x->vtop, nullptr, 0, only_seq, accept ? 1 : 0);
     return;
@@ -797,7 +836,35 @@ void enqueue_verify(ada_ctx *x, int only_seq, float *d_logits, bool accept = fal
 // 1.58, 2.02 / 1.73 ms, 5 sequences 1.35 / 1.47, 1.72 / 1.61, 2.34 / 1.85; 8 layers of 4096 with 32 heads, 6 sequences 1.17 / 1.34, 1.37 /
 // 1.42, 2.33 / 1.96 (before batches took this kernel: 1.88); 8 layers of 2048 with 16 heads, 8 sequences 0.67 / 0.80, 0.83 / 0.88, 1.17 / 1.04.
 bool pass_takes(const ada_ctx *x, int B) {
-  return x->pass_ok && B * (x->c.n_max + 1) <= kPassRowsMax && B * x->c.n_heads <= 128;
+  return x->small || (x->pass_ok && B * (x->c.n_max + 1) <= kPassRowsMax && B * x->c.n_heads <= 128);
+}
+
+// Whether decode passes run on one cluster of 16 thread blocks per sequence (ada_small.cuh): models whose layer and a share of the LM head
+// fit the cluster's shared memory and registers.  Where they do it is the faster one throughout, but for large vocabularies
+// (kSmVocabMax): draft of four + verify, k_pass -> cluster, context 480 146 + 69 -> 59 + 48 us, 3900 183 + 87 -> 93 + 65, eight sequences 188
+// + 119 -> 100 + 81, d_model 128 130 + 60 -> 51 + 38.
+int small_takes(ada_ctx *x) {
+  const ada_config &c = x->c;
+  SmallShape &z = x->small_shape;
+  if (!small_shape(c.n_layers, c.d_model, c.n_heads, c.head_dim, c.d_ffn, c.vocab, c.n_max, x->pages_per_seq, z)) return 0;
+  z.w_fc = x->eagle_fc; z.w_lm = x->lm_head;
+  for (int mode = 0; mode < 2; ++mode) {
+    const SmallKernel kernel = small_kernel(mode);
+    int clusters = 0;
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = dim3(kSmCtas); lc.blockDim = dim3(kSmThreads); lc.dynamicSmemBytes = z.total;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = kSmCtas; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    lc.attrs = at; lc.numAttrs = 1;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmSmemMax) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&clusters, kernel, &lc) != cudaSuccess || clusters < 1) {
+      cudaGetLastError();
+      return 0;
+    }
+  }
+  return 1;
 }
 
 // Labels of start positions j0 .. j0 + count - 1 of a sequence in packed passes: up to eight start positions at a time are
@@ -1001,7 +1068,7 @@ extern "C" int ada_init(ada_ctx **out, const ada_config *cfg, const ada_weights 
   if (e == cudaSuccess) e = cudaMemsetAsync(x->x2hi, 0, sizeof(bf16) * (size_t)x->prompt_rows * x->ldx2, x->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(x->x2lo, 0, sizeof(bf16) * (size_t)x->prompt_rows * x->ldx2, x->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(x->stream);  // host vectors go out of scope
-  x->use_pass = x->pass_ok = 0;
+  x->use_pass = x->pass_ok = x->small = 0;
   if (e == cudaSuccess) {
     int dev = 0, sms = 0, per_sm = 0;
     e = cudaGetDevice(&dev);
@@ -1034,6 +1101,7 @@ extern "C" int ada_init(ada_ctx **out, const ada_config *cfg, const ada_weights 
     }
     if (e == cudaSuccess && per_sm >= 1 && sms <= 256 && fits && max_clusters >= grid / 2) {
       x->pass_ok = 1;
+      x->small = small_takes(x);
       x->use_pass = pass_takes(x, cfg->max_batch);
       x->n_sm = grid;
       std::vector<LayerPtrs> lp(cfg->n_layers);
