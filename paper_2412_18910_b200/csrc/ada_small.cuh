@@ -10,8 +10,9 @@
 // on the way; 24 clocks one behind the other).  What is left is a chain of dependent instructions, some eight clocks each, so the
 // kernel does as little as it can between an exchange and the next: one copy per reader (a warp's copies are issued lane by lane, 100
 // clocks each), gains and rotary factors in shared memory beforehand, a body of its own for draft steps of one row.
-// Draft of four + verify of five rows, 2 layers of 256, vocabulary 4096, context 100: k_pass 134 + 62 us, here 55 + 46; seven sequences
-// 188 + 117 -> 57 + 46; verify with 8 layers 173 -> 120.
+// Draft of four + verify of five rows, 2 layers of 256, vocabulary 4096, context 100: k_pass 134 + 62 us, here 50 + 42 (55 + 46 with candidates
+// merged by five exchanges of three words and a thread walking all of its partial sums of attention); seven sequences 188 + 117 -> 57 +
+// 46; verify with 8 layers 173 -> 120.
 //
 // Weights depend on no phase.  A layer's lie in shared memory (bulk copies as they are in memory, 118 KB a CTA at these sizes; those of the
 // next layer's phase follow when the phase's products are done), draft steps keep them; the first 4096 rows of the LM head, 128 KB
@@ -189,6 +190,21 @@ __device__ __forceinline__ void sts_f2(uint32_t a, float x, float y) {
 }
 __device__ __forceinline__ void sts_f(uint32_t a, float x) { asm volatile("st.shared.f32 [%0], %1;" ::"r"(a), "f"(x) : "memory"); }
 __device__ __forceinline__ void sts_h(uint32_t a, unsigned short x) { asm volatile("st.shared.u16 [%0], %1;" ::"r"(a), "h"(x) : "memory"); }
+// The best of 32 candidates and the largest value among the others, as top2_merge gives them: the largest value, of equal ones the one
+// of the lowest index.  (Integers in the order of the values; three reductions of the warp instead of five exchanges of three words.)
+__device__ __forceinline__ int small_key(float v) {
+  const int k = __float_as_int(v + 0.f);   // (-0 counts as 0)
+  return k ^ ((k >> 31) & 0x7fffffff);
+}
+__device__ __forceinline__ float small_unkey(int k) { return __int_as_float(k ^ ((k >> 31) & 0x7fffffff)); }
+__device__ __forceinline__ Top2 small_best(Top2 c) {
+  const int k = small_key(c.v1), best = __reduce_max_sync(0xffffffffu, k);
+  Top2 r;
+  r.i1 = __reduce_min_sync(0xffffffffu, k == best ? c.i1 : 0x7fffffff);
+  r.v1 = small_unkey(best);
+  r.v2 = small_unkey(__reduce_max_sync(0xffffffffu, small_key(k == best && c.i1 == r.i1 ? c.v2 : c.v1)));
+  return r;
+}
 // Accepting is rare and serial: out of line.
 __device__ __noinline__ void small_accept(const PassParams &p, int b, const int *draft, const int *target) {
   accept_sequence(p.st, p.tok, p.cap, p.tok_stride, draft, target, p.nmax, b, p.cnt, nullptr, 0, p.acc_out, p.emit_out, p.nemit_out, nullptr);
@@ -536,35 +552,43 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(const __grid_constant__
         }
         __syncthreads();
         next_send();
-        // merge of n (at most 8) partial sums, `step` bytes apart: (m, l) at ml, four channels at o; in their order
-        auto merge8 = [&](uint32_t ml, uint32_t o, int step, int n, float4 &y, float &M, float &L) {
-          float2 v[kSmWarps];
+        // Adds up to N partial sums, `step` bytes apart, to those so far, in order: (m, l) at ml, four channels at o.  (One a lane, merged by
+        // exchanges, took three times as long for five rows.)
+        auto merge = [&](auto slots, uint32_t ml, uint32_t o, int step, int n, float4 &y, float &M, float &L) {
+          constexpr int N = decltype(slots)::value;
+          float2 v[N];
+          float4 ov[N];
 #pragma unroll
-          for (int k = 0; k < kSmWarps; ++k) v[k] = k < n ? lds_f2(ml + k * step) : make_float2(-INFINITY, 0.f);
+          for (int k = 0; k < N; ++k) {
+            v[k] = make_float2(-INFINITY, 0.f);
+            ov[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (k < n) { v[k] = lds_f2(ml + k * step); ov[k] = lds_f4(o + k * step); }
+          }
           const float M0 = M;
 #pragma unroll
-          for (int k = 0; k < kSmWarps; ++k) M = fmaxf(M, v[k].x);
+          for (int k = 0; k < N; ++k) M = fmaxf(M, v[k].x);
           const float base = M > -INFINITY ? M : 0.f, f0 = __expf(M0 - base);
           L *= f0;
           y.x *= f0; y.y *= f0; y.z *= f0; y.w *= f0;
 #pragma unroll
-          for (int k = 0; k < kSmWarps; ++k)
-            if (k < n) {
-              const float4 ov = lds_f4(o + k * step);
-              const float f = __expf(v[k].x - base);
-              L += v[k].y * f;
-              y.x += ov.x * f; y.y += ov.y * f; y.z += ov.z * f; y.w += ov.w * f;
-            }
+          for (int k = 0; k < N; ++k) {
+            const float f = __expf(v[k].x - base);
+            L += v[k].y * f;
+            y.x += ov[k].x * f; y.y += ov[k].y * f; y.z += ov[k].z * f; y.w += ov[k].w * f;
+          }
         };
         if (has_head) {
           // over the warps, four channels of a row per thread
+          const int nw = min(mine, kSmWarps);
 #pragma unroll 1
           for (int e = tid; e < T * (HD / 4); e += kSmThreads) {
             const int r = e / (HD / 4), c = (e & (HD / 4 - 1)) * 4;
             const uint32_t pr = scratch + r * PS * 4;
             float M = -INFINITY, L = 0.f;
             float4 y = make_float4(0.f, 0.f, 0.f, 0.f);
-            merge8(pr + HD * 4, pr + c * 4, T * PS * 4, min(mine, kSmWarps), y, M, L);
+#pragma unroll 1
+            for (int k = 0; k < nw; k += 4)
+              merge(std::integral_constant<int, 4>{}, pr + k * T * PS * 4 + HD * 4, pr + k * T * PS * 4 + c * 4, T * PS * 4, nw - k, y, M, L);
             sts_f4(send + (r * HD + c) * 4, y);
             if (c == 0) sts_f2(send + part_o + r * 8, M, L);
           }
@@ -574,23 +598,22 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(const __grid_constant__
         if (has_head) copy_to_all(z.ac + rank * part, part, SMX_A);
         wait(SMX_A);
         // over the CTAs of each head, by every CTA for itself: O's input
-        auto merge = [&](int r, int c) {
-          const int h = 4 * c / HD, ch = 4 * c & (HD - 1);
-          const uint32_t src = sm0 + z.ac + h * z.ns * part;
+        auto merge_head = [&](int r, int c) {
+          const uint32_t src = sm0 + z.ac + 4 * c / HD * z.ns * part, ch = (r * HD + (4 * c & (HD - 1))) * 4;
           float M = -INFINITY, L = 0.f;
           float4 y = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 1
-          for (int k = 0; k < z.ns; k += kSmWarps)
-            merge8(src + k * part + part_o + 8 * r, src + k * part + (r * HD + ch) * 4, part, min(z.ns - k, kSmWarps), y, M, L);
+          for (int k = 0; k < z.ns; k += 4)
+            merge(std::integral_constant<int, 4>{}, src + k * part + part_o + 8 * r, src + k * part + ch, part, z.ns - k, y, M, L);
           const float inv = 1.f / L;
           sts4(sm0 + z.e + ((c >> 1) * 2 * TS + (c & 1) * TS + r) * 16, small_split4(y.x * inv, y.y * inv, y.z * inv, y.w * inv));
         };
         if (ONE) {
-          if (tid < d4) merge(0, tid);
+          if (tid < d4) merge_head(0, tid);
         } else {
 #pragma unroll 1
           for (int r = r4, c = c4; r < T;) {
-            merge(r, c);
+            merge_head(r, c);
             r += dr4; c += dc4;
             if (c >= d4) { c -= d4; ++r; }
           }
@@ -823,8 +846,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(const __grid_constant__
             c.v1 = y; c.i1 = v0;
           }
           const float y = c.v1;
-#pragma unroll
-          for (int o = 16; o > 0; o >>= 1) c = top2_shfl_xor(c, o);
+          c = small_best(c);
           float s = 0.f;
           if (lps) s = warp_sum(own ? __expf(y - c.v1) : 0.f);   // sum of exp(logit - maximum)
           if (lane == 0) {
@@ -848,7 +870,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(const __grid_constant__
     }
     __syncthreads();
     next_send();
-    // candidates of the warps, then of the CTAs: a row to a warp, 16 lanes
+    // candidates of the warps, then of the CTAs: a row to a warp, a candidate to a lane
     const bool takes = DRAFT || rank == 0;
 #pragma unroll 1
     for (int stage = 0; stage < (takes ? 2 : 1); ++stage) {
@@ -858,25 +880,22 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(const __grid_constant__
         Top2 c;
         c.v1 = c.v2 = -INFINITY; c.i1 = 0x7fffffff;
         float cs = 0.f, fl = -INFINITY;
-        if (stage == 0) {
-          if ((lane & 15) < kSmWarps) { c = topw[(lane & 15) * kSmRowsMax + r]; cs = sew[(lane & 15) * kSmRowsMax + r]; }
-          if (lps) fl = flog[r];
-        } else {
-          const uint32_t cp = sm0 + z.cand + (lane & 15) * 32 * Tg + r * 32;
-          const float4 v = lds_f4(cp);
-          c.v1 = v.x; c.i1 = __float_as_int(v.y); c.v2 = v.z; cs = v.w;
-          fl = lds_f(cp + 16);
+        if (lane < (stage == 0 ? kSmWarps : kSmCtas)) {
+          if (stage == 0) {
+            c = topw[lane * kSmRowsMax + r];
+            if (lps) { cs = sew[lane * kSmRowsMax + r]; fl = flog[r]; }
+          } else {
+            const uint32_t cp = sm0 + z.cand + lane * 32 * Tg + r * 32;
+            const float4 v = lds_f4(cp);
+            c.v1 = v.x; c.i1 = __float_as_int(v.y); c.v2 = v.z; cs = v.w;
+            if (lps) fl = lds_f(cp + 16);
+          }
         }
         const float own = c.v1;
-#pragma unroll
-        for (int o = 8; o > 0; o >>= 1) c = top2_shfl_xor(c, o);
+        c = small_best(c);
         if (lps) {
-          cs = own > -INFINITY ? cs * __expf(own - c.v1) : 0.f;
-#pragma unroll
-          for (int o = 8; o > 0; o >>= 1) {
-            cs += __shfl_xor_sync(0xffffffffu, cs, o);
-            fl = fmaxf(fl, __shfl_xor_sync(0xffffffffu, fl, o));
-          }
+          cs = warp_sum(own > -INFINITY ? cs * __expf(own - c.v1) : 0.f);
+          fl = warp_max(fl);
         }
         if (stage == 0) {
           if (lane == 0) {
@@ -949,11 +968,12 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(const __grid_constant__
 #pragma unroll 1
     while (more) more = run_pass(std::true_type{});
   }
-  for (int k = 0; k < SM_LM; ++k) wait_weights(k);   // no copy may outlive the CTA
-  // no CTA leaves while copies into its memory, or out of it, are under way: all that were sent have been awaited by their readers
-  await_copies(abort_s);
-  __syncthreads();
-  cluster_sync_all();                                // (and all have read the state)
+  // ================================================================ the sequence's state
+  // (a pass has exchanged results with every CTA of the cluster, so all of them have read the state; without one they meet first)
+  if (nstep == 0) {
+    for (int k = 0; k < SM_LM; ++k) wait_weights(k);   // no copy may outlive the CTA
+    cluster_sync_all();
+  }
   if (rank == 0 && tid == 0) {
     SeqState *const st = p.st + b;
     if (DRAFT) {
@@ -968,6 +988,10 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(const __grid_constant__
       if (p.accept) small_accept(p, b, nstep > 0 ? tok_s + 1 : nullptr, nstep > 0 ? choice_s : nullptr);
     }
   }
+  // no CTA leaves while copies into its memory, or out of it, are under way: all that were sent have been awaited by their readers
+  await_copies(abort_s);
+  __syncthreads();
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;\n barrier.cluster.wait.aligned;" ::: "memory");   // (nothing is published here)
 }
 
 }  // namespace ada
