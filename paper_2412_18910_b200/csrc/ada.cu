@@ -92,6 +92,7 @@ struct ada_ctx {
   float *lb_feat;
   float2 *lb_top;
   float4 *amax2;
+  int *cut_flags;                     // tiles of prompt GEMMs that several pairs share (zero between launches)
   unsigned *gbar;
   unsigned long long *phase_ns;
   int *prof_steps;
@@ -247,12 +248,14 @@ size_t part_need_tc(int epi, int nseg, int Nseg, int K) {
 // boxes, 2048 4.54e-6 -> 4.48e-6 with 4 (4.89e-6 with 8), 1024 1.99e-6 -> 2.01e-6 and 256 2.64e-7 -> 2.58e-7 with 2 (2.76e-7 with 4).  With
 // 8 boxes the middle model's 333 tokens took 1.97 ms (2.09 with 4, 2.52 with 2), 2001 tokens of 7B 50.9 (52.2 with 4, 60.4 with 2).
 int pair_chunk(int K) { return K < 2048 ? 2 : 4; }
-struct PairPlan { int nb, token_tiles, S; };
+struct PairPlan { int nb, token_tiles, S, whole; };
 constexpr int kPairs = 74;
 constexpr int kPairSplitRows = 2048;    // S x rows of the partial sums at most (scratch is sized for it)
-PairPlan plan_pair(int T, int weight_tiles, int N, int K, bool may_split, size_t split_rows) {
-  PairPlan best{128, (T + 255) / 256, 1};
-  double best_us = 1e30;
+// whole: tiles dealt whole, from the first on; fewer than there are: the rest in equal runs.  scratch: floats for sums that cross pairs.
+PairPlan plan_pair(int T, int weight_tiles, int N, int K, bool may_split, size_t split_rows, int chunk, size_t scratch) {
+  PairPlan best{128, (T + 255) / 256, 1, (T + 255) / 256 * weight_tiles};
+  PairPlan cut = best;
+  double best_us = 1e30, cut_us = 1e30;
   const int kboxes = (K + 63) / 64;
   for (int nb = 32; nb <= 128; nb += 32) {
     const int tt = (T + 2 * nb - 1) / (2 * nb);
@@ -261,10 +264,25 @@ PairPlan plan_pair(int T, int weight_tiles, int N, int K, bool may_split, size_t
       const double clk_box = fmax(8.0 * nb, (16384.0 + 256.0 * nb) / 48.0);
       double us = waves * ((double)((kboxes + S - 1) / S) * clk_box / 1900.0 + 2.0);
       us = fmax(us, 2.0 * N * (double)K / 6.4e6) + (S > 1 ? 8.0 * S * (double)T * N / 4.0e6 : 0.0);
-      if (us < best_us) { best_us = us; best = PairPlan{nb, tt, S}; }
+      if (us < best_us) { best_us = us; best = PairPlan{nb, tt, S, items}; }
+    }
+    // All whole waves but one, the rest cut into runs of accumulators as long for every pair.  The cut tiles' sums are put at 10 us at nb
+    // = 128, and the cut has to come out below 0.92 of the time (weights of several token tiles come from HBM more than once).  GEMMs
+    // that may be split along K only at the widest tiles and with one for every pair at least: more cuts a tile, or narrower tiles,
+    // cost more than an idle part of a wave (13B down of 640 rows 160 -> 188 us).  Four layers and the head, prompts of 130, 205, 256, 333,
+    // 512 and 1000 tokens, whole tiles -> so: 7B 1119, 1285, 1317, 1660, 2015 -> 1012, 1182, 1210, 1620, 1975 us (1000: not cut), 13B
+    // 1414, 1625, 1658, 2306, 2875, 5790 -> 1348, 1568, 1608, 2306, 2840, 5430.
+    const int kruns = (kboxes + chunk - 1) / chunk, items = tt * weight_tiles;
+    const size_t sums = (may_split ? (size_t)T * N : 0) + (size_t)kPairs * 2 * 128 * 2 * nb;
+    if (sums <= scratch && items * kruns >= kPairs && (!may_split || (nb == 128 && items >= kPairs))) {
+      const double clk_box = fmax(8.0 * nb, (16384.0 + 256.0 * nb) / 48.0);
+      const int waves = std::max(0, items / kPairs - 1), rest = items - waves * kPairs;
+      double us = waves * (kboxes * clk_box / 1900.0 + 2.0) + (double)((rest * kruns + kPairs - 1) / kPairs) * chunk * clk_box / 1900.0 + 2.0 + 10.0 * nb / 128.0;
+      us = fmax(us, 2.0 * N * (double)K / 6.4e6);
+      if (us < cut_us) { cut_us = us; cut = PairPlan{nb, tt, 1, waves * kPairs}; }
     }
   }
-  return best;
+  return cut_us < 0.92 * best_us ? cut : best;
 }
 
 // Rows of a prompt chunk (and of the row scratch) that an engine asks for; ada_init takes the most, down to 128, that the
@@ -358,7 +376,8 @@ size_t carve(ada_ctx *x, const ada_config *c, int rows, char *base) {
   x->fc = w.take<bf16>(((2 * d + 63) / 64) * (kPassRowsMax * 128));
   x->ss_part = w.take<float>(kSsStride * kPassRowsMax);
   x->attn_cnt = w.take<int>(kMaxBatch * H);
-  x->amax2 = w.take<float4>(256 * kPassRowsMax);
+  x->amax2 = w.take<float4>(kPassCtasMax * kPassRowsMax);
+  x->cut_flags = w.take<int>(2 * kPairs * 8);
   x->gbar = w.take<unsigned>(64);
   x->phase_ns = w.take<unsigned long long>(512 + 4 * 512);
   x->prof_steps = w.take<int>(kProfRecords);
@@ -393,6 +412,10 @@ void reduce_h(ada_ctx *x, int S, int part_rows, const Reduce &r) {
   launch_pdl(x, k_reduce_h, dim3((d + 1023) / 1024, x->TM), 256, 0, a);
 }
 
+void (*const kPairKernels[3][2])(const GemmPairArgs) = {{k_gemm_pair<PAIR_PART, false>, k_gemm_pair<PAIR_PART, true>},
+                                                        {k_gemm_pair<PAIR_QKV, false>, k_gemm_pair<PAIR_QKV, true>},
+                                                        {k_gemm_pair<PAIR_SWIGLU, false>, k_gemm_pair<PAIR_SWIGLU, true>}};
+
 // A GEMM of a prompt pass (x->TM rows of one sequence) and what follows it.
 bool gemm_prompt(ada_ctx *x, int epi, const bf16 *W0, const bf16 *W1, const bf16 *W2, int nseg, int Nseg, int K,
                  const bf16 *Xhi, const bf16 *Xlo, const Reduce &r) {
@@ -403,8 +426,9 @@ bool gemm_prompt(ada_ctx *x, int epi, const bf16 *W0, const bf16 *W1, const bf16
   const int kind = sw ? PAIR_SWIGLU : r.kind == Reduce::QKV_ROPE ? PAIR_QKV : PAIR_PART;
   t.nseg = nseg; t.Nseg = Nseg; t.K = K; t.T = x->TM; t.chunk = pair_chunk(K);
   t.weight_tiles = sw ? (Nseg + 127) / 128 : nseg * ((Nseg + 255) / 256);
-  const PairPlan plan = plan_pair(x->TM, t.weight_tiles, sw ? 2 * Nseg : nseg * Nseg, K, kind == PAIR_PART, x->part_floats / c.d_model);
-  t.nb = plan.nb; t.token_tiles = plan.token_tiles; t.S = plan.S;
+  const PairPlan plan = plan_pair(x->TM, t.weight_tiles, sw ? 2 * Nseg : nseg * Nseg, K, kind == PAIR_PART, x->part_floats / c.d_model, t.chunk, x->part_floats);
+  t.nb = plan.nb; t.token_tiles = plan.token_tiles; t.S = plan.S; t.whole = plan.whole;
+  t.cut = x->gemm_part + (kind == PAIR_PART ? (size_t)x->TM * Nseg : 0); t.cut_flags = x->cut_flags;
   const bf16 *Ws[3] = {W0, W1, W2};
   for (int i = 0; i < 3; ++i)
     if (Ws[i] && !(t.wmap[i] = find_map(x, sw ? x->pairmap_of : x->tcmap_of, Ws[i]))) return no_map(x);
@@ -420,10 +444,8 @@ bool gemm_prompt(ada_ctx *x, int epi, const bf16 *W0, const bf16 *W1, const bf16
   t.pass = x->pass; t.cnts = x->cnt;
   const int items = t.token_tiles * t.weight_tiles * t.S;
   timed(x, 0, 2.0 * (double)Nseg * (double)K * (epi == EPI_SWIGLU ? 2 : nseg), [&] {
-    const int pairs = items < kPairs ? items : kPairs;
-    if (kind == PAIR_QKV) launch_pair(x, k_gemm_pair<PAIR_QKV>, pairs, kPairThreads, kPairSmemBytes, t);
-    else if (kind == PAIR_SWIGLU) launch_pair(x, k_gemm_pair<PAIR_SWIGLU>, pairs, kPairThreads, kPairSmemBytes, t);
-    else launch_pair(x, k_gemm_pair<PAIR_PART>, pairs, kPairThreads, kPairSmemBytes, t);
+    const int pairs = items < kPairs && t.whole == items ? items : kPairs;
+    launch_pair(x, kPairKernels[kind][t.whole < items], pairs, kPairThreads, kPairSmemBytes, t);
     if (kind == PAIR_PART) reduce_h(x, t.S, t.part_rows, r);
   });
   return true;
@@ -1057,6 +1079,7 @@ extern "C" int ada_init(ada_ctx **out, const ada_config *cfg, const ada_weights 
     if (e == cudaSuccess) e = cudaMemsetAsync(x->dv, 0, pool, x->stream);
   }
   if (e == cudaSuccess) e = cudaMemsetAsync(x->cnt, 0, sizeof(Counters), x->stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(x->cut_flags, 0, sizeof(int) * 2 * kPairs * 8, x->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(x->pass, 0, sizeof(Pass), x->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(x->tok, 0, sizeof(int) * (size_t)x->B * cap, x->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(x->draft, 0, sizeof(int) * x->B * cfg->n_max, x->stream);
@@ -1099,7 +1122,7 @@ extern "C" int ada_init(ada_ctx **out, const ada_config *cfg, const ada_weights 
       lc.attrs = at; lc.numAttrs = 1;
       if (cudaOccupancyMaxActiveClusters(&max_clusters, k_pass<false>, &lc) != cudaSuccess) { max_clusters = 0; cudaGetLastError(); }
     }
-    if (e == cudaSuccess && per_sm >= 1 && sms <= 256 && fits && max_clusters >= grid / 2) {
+    if (e == cudaSuccess && per_sm >= 1 && sms <= kPassCtasMax && fits && max_clusters >= grid / 2) {
       x->pass_ok = 1;
       x->small = small_takes(x);
       x->use_pass = pass_takes(x, cfg->max_batch);
@@ -1132,7 +1155,7 @@ extern "C" int ada_init(ada_ctx **out, const ada_config *cfg, const ada_weights 
     auto pair_smem = [&](void (*k)(const GemmPairArgs)) {
       if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kPairSmemBytes);
     };
-    pair_smem(k_gemm_pair<PAIR_PART>); pair_smem(k_gemm_pair<PAIR_QKV>); pair_smem(k_gemm_pair<PAIR_SWIGLU>);
+    for (auto &k : kPairKernels) { pair_smem(k[0]); pair_smem(k[1]); }
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(k_gemm_tc<kTcRowsMax>, cudaFuncAttributeMaxDynamicSharedMemorySize, TcShape<kTcRowsMax>::kSmemBytes);
     std::vector<TensorMap128> maps;

@@ -11,6 +11,14 @@
 // products of the next (persistent grid, one pair per two SMs, tiles dealt in a fixed order with the token tiles of a
 // weight tile side by side so that its weights cross HBM once).
 //
+// Where the last tiles would leave most pairs idle (86 gate/up tiles of 256 rows on 74 pairs take the time of 148), the tiles
+// from `whole` on are cut: every pair gets a run of as many accumulators, which may begin and end inside a tile.  A tile's first boxes
+// are the end of a pair's run, its last ones the beginning of another's (or whole runs between): those leave their fp32 sums in memory,
+// and the pair that has the first boxes adds them up in order and finishes the tile.  By then they have long been there: all runs begin
+// together.  7B, level 2 cold: gate/up of 205 rows 106 -> 81 us, of 512 159 -> 146, QKV of 205 63 -> 58; 13B QKV of 1024 258 -> 239, down 255
+// -> 206.  With token tiles side by side no longer, weights cross HBM more than once (13B QKV of 512 168 -> 323 MB; kept in level 2
+// instead of passing through it they were slower, 129 -> 134 us).
+//
 //   warp 0      producer, one thread per CTA: weight box and plane boxes of its half of the tile into a ring of stages;
 //               the bytes of both CTAs are counted on the leader's (even CTA's) barrier
 //   warp 1      leader only: one elected thread issues the products and commits to both CTAs' barriers
@@ -51,6 +59,9 @@ struct GemmPairArgs {
   int nb;                                  // prompt rows per CTA and tile: 32, 64, 96 or 128
   int token_tiles, weight_tiles, S;        // S: K splits (PART only)
   int chunk;                               // 64-k boxes per accumulator
+  int whole;                               // tiles (and splits) dealt whole; the rest (S = 1) in equal runs to all pairs
+  float *cut; int *cut_flags;              // ... sums of a tile's cut-off parts [CTA][prompt row][128 weight rows]; per CTA and epilogue warp
+                                           // 1 when they are there (zero between launches)
   float *part; int part_rows;              // PART: [S][part_rows][Nseg]
   // QKV and SWIGLU
   const float *ss_part; float eps; int d;
@@ -128,7 +139,8 @@ __device__ __forceinline__ float silu(float x) {
   return x > 88.f ? x : x < -80.f ? x * 0.f : z;
 }
 
-template <int EPI>
+// CUT: with tiles that pairs share (a kernel of its own: as a branch of one it cost the others 1.6 us a launch).
+template <int EPI, bool CUT>
 __global__ void __launch_bounds__(kPairThreads, 1) k_gemm_pair(const GemmPairArgs a) {
   pdl_launch_dependents();
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -153,6 +165,30 @@ __global__ void __launch_bounds__(kPairThreads, 1) k_gemm_pair(const GemmPairArg
   const int kboxes = (a.K + 63) >> 6;
   const int items = a.token_tiles * a.weight_tiles * a.S;
   const int tiles_per_seg = sw ? a.weight_tiles : a.weight_tiles / a.nseg;
+  // The pair's work, a tile and a range of its boxes at a time: whole tiles (or K splits) dealt in turn, then, of the tiles from `whole`
+  // on, a run of accumulators as long as every other pair's, which may start and end inside a tile.
+  const int kruns = CUT ? (kboxes + a.chunk - 1) / a.chunk : 0, whole = CUT ? a.whole : items;
+  auto run_begin = [&](int p) { return p * ((items - whole) * kruns) / npairs; };
+  struct Work { int item, kb0, kb1, next, run, end; };
+  auto first_work = [&](Work &w) {
+    w.next = pair;
+    if (CUT) { w.run = run_begin(pair); w.end = run_begin(pair + 1); }
+  };
+  auto next_work = [&](Work &w) {
+    if (w.next < whole) {
+      w.item = w.next;
+      const int split = w.item / (a.token_tiles * a.weight_tiles);
+      w.kb0 = split * kboxes / a.S; w.kb1 = (split + 1) * kboxes / a.S;
+      w.next += npairs;
+      return true;
+    }
+    if (!CUT || w.run >= w.end) return false;
+    const int i = w.run / kruns, c0 = w.run - i * kruns, c1 = min(kruns, c0 + w.end - w.run);
+    w.item = whole + i;
+    w.kb0 = c0 * a.chunk; w.kb1 = min(kboxes, c1 * a.chunk);
+    w.run += c1 - c0;
+    return true;
+  };
 
   if (tid == 0) {
     *abort_s = 0;
@@ -168,15 +204,13 @@ __global__ void __launch_bounds__(kPairThreads, 1) k_gemm_pair(const GemmPairArg
   const uint32_t tmem_base = *tmem_slot;
 
   // item -> split, weight tile (segment and first row), token tile
-  auto decode = [&](int item, int &seg, int &tile, int &tok0, int &kb0, int &kb1, int &split) {
+  auto decode = [&](int item, int &seg, int &tile, int &tok0, int &split) {
     const int tt = item % a.token_tiles, rest = item / a.token_tiles;
     const int wt = rest % a.weight_tiles;
     split = rest / a.weight_tiles;
     seg = sw ? 0 : wt / tiles_per_seg;
     tile = sw ? wt : wt - seg * tiles_per_seg;
     tok0 = tt * N;
-    kb0 = split * kboxes / a.S;
-    kb1 = (split + 1) * kboxes / a.S;
   };
 
   // the epilogue warps hold a tile's sums: 256 x 224 + 128 x 56 registers = the 384 x 168 of the launch
@@ -188,9 +222,11 @@ __global__ void __launch_bounds__(kPairThreads, 1) k_gemm_pair(const GemmPairArg
     const unsigned tx = 2u * (unsigned)stage_bytes;   // both CTAs' boxes (rows past a matrix arrive as zeros)
     int slot = 0, it = 0;
     bool waited = false;
-    for (int item = pair; item < items; item += npairs) {
-      int seg, tile, tok0, kb0, kb1, split;
-      decode(item, seg, tile, tok0, kb0, kb1, split);
+    Work wk;
+    for (first_work(wk); next_work(wk);) {
+      int seg, tile, tok0, split;
+      decode(wk.item, seg, tile, tok0, split);
+      const int kb0 = wk.kb0, kb1 = wk.kb1;
       const TensorMap128 *m0 = sw ? a.wmap[0] : a.wmap[seg];
       const int row = sw ? tile * 128 + (int)rank * 64 : tile * 256 + (int)rank * 128;
       const int xrow = tok0 + (int)rank * a.nb;
@@ -238,9 +274,9 @@ __global__ void __launch_bounds__(kPairThreads, 1) k_gemm_pair(const GemmPairArg
     // 15.9 -> 14.9 ms a prompt; 333 rows, 16 layers of 2048: 2296 -> 2130 us)
     const uint32_t tb = __reduce_max_sync(0xffffffffu, tmem_base), sb = __reduce_max_sync(0xffffffffu, smem_u32(smem));
     int slot = 0, it = 0, n = 0;   // n: accumulators filled so far
-    for (int item = pair; item < items; item += npairs) {
-      int seg, tile, tok0, kb0, kb1, split;
-      decode(item, seg, tile, tok0, kb0, kb1, split);
+    Work wk;
+    for (first_work(wk); next_work(wk);) {
+      const int kb0 = wk.kb0, kb1 = wk.kb1;
       for (int kc = kb0; kc < kb1; kc += a.chunk, ++n) {
         const int buf = n & 1, kc1 = min(kb1, kc + a.chunk);
         if (n >= 2) mbar_wait_inline(&accempty[buf], ((unsigned)(n >> 1) & 1u) ^ 1u, a.cnts, abort_s);
@@ -301,9 +337,11 @@ __global__ void __launch_bounds__(kPairThreads, 1) k_gemm_pair(const GemmPairArg
         }
       }
     };
-    for (int item = pair; item < items; item += npairs) {
-      int seg, tile, tok0, kb0, kb1, split;
-      decode(item, seg, tile, tok0, kb0, kb1, split);
+    Work wk;
+    for (first_work(wk); next_work(wk);) {
+      int seg, tile, tok0, split;
+      decode(wk.item, seg, tile, tok0, split);
+      const int kb0 = wk.kb0, kb1 = wk.kb1;
       const int Tl = min(N, a.T - tok0);
       float sum[4][32];
 #pragma unroll
@@ -329,7 +367,53 @@ __global__ void __launch_bounds__(kPairThreads, 1) k_gemm_pair(const GemmPairArg
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive_peer(peer_addr(&accempty[buf], 0));
-        if (EPI != PAIR_PART && kc == kb0) row_info(tok0, Tl);   // (under the products of the chunks that follow)
+        if (EPI != PAIR_PART && kc == 0) row_info(tok0, Tl);   // (under the products of the chunks that follow)
+      }
+      if constexpr (CUT) {
+        // A tile cut by the runs' ends: the pair that has its first boxes, the last of its run, finishes it; the others, for which it is the
+        // first of theirs, leave their sums in memory.  A warp takes what the same warp of the other pairs left.
+        const size_t at = (size_t)(ch * a.nb) * 128 + quarter * 32 + lane;
+        const int ew = warp - 4;
+        if (kb0 > 0) {
+          float *o = a.cut + (size_t)blockIdx.x * N * 128 + at;
+#pragma unroll
+          for (int blk = 0; blk < 4; ++blk)
+            if (blk * 32 < a.nb) {
+#pragma unroll
+              for (int i = 0; i < 32; ++i) __stcg(o + (size_t)(blk * 32 + i) * 128, sum[blk][i]);
+            }
+          __syncwarp();
+          if (lane == 0) asm volatile("st.release.gpu.global.s32 [%0], 1;" ::"l"(a.cut_flags + blockIdx.x * 8 + ew) : "memory");
+          continue;
+        }
+        if (kb1 < kboxes) {
+          const int tile_end = (wk.item - whole + 1) * kruns;
+#pragma unroll 1
+          for (int p = pair + 1; run_begin(p) < tile_end; ++p) {
+            const int cta = 2 * p + (int)rank;
+            int *flag = a.cut_flags + cta * 8 + ew;
+            if (lane == 0) {
+              for (unsigned i = 0;; ++i) {
+                if (ld_acquire(reinterpret_cast<const unsigned *>(flag)) == 1u || *abort_s) break;
+                if (i > 64) __nanosleep(40);
+                if (i == kSpinLimit) { *abort_s = 1; atomicOr(&a.cnts->status, kStatTimeout); }
+              }
+            }
+            __syncwarp();
+            const float *q = a.cut + (size_t)cta * N * 128 + at;
+#pragma unroll
+            for (int blk = 0; blk < 4; ++blk)
+              if (blk * 32 < a.nb) {
+                float v[32];
+#pragma unroll
+                for (int i = 0; i < 32; ++i) v[i] = __ldcg(q + (size_t)(blk * 32 + i) * 128);
+#pragma unroll
+                for (int i = 0; i < 32; ++i) sum[blk][i] += v[i];
+              }
+            __syncwarp();
+            if (lane == 0) *flag = 0;
+          }
+        }
       }
       const int row = (sw ? tile * 128 + (int)rank * 64 : tile * 256 + (int)rank * 128) +
                       (sw ? (quarter & 1) * 32 + lane : quarter * 32 + lane);     // weight row inside its matrix

@@ -58,6 +58,7 @@ constexpr int kXBufs = 10;                       // activation buffers at most
 // takes four boxes up to 40 rows, two beyond; as many buffers as fit the area are in flight.  (A stage of weights has no more
 // boxes than a buffer, and stages are what the issuing thread's time goes into: 7B, 30 rows, 3500 us a pass with two boxes,
 // 3263 with four.)
+constexpr int kPassCtasMax = 160;                // CTAs at most
 constexpr int kPassRowsMax = 48;                 // rows of a pass at most
 constexpr int kXBytes = 80 * 1024;               // the buffers' area
 __host__ __device__ constexpr int xbuf_boxes(int TP) { return TP <= 40 ? 4 : 2; }

@@ -1,0 +1,44 @@
+"""Prompt GEMMs whose tiles are cut so that every pair of thread blocks gets as much: tiles in two and in more parts, of one and of
+several token tiles, partly filled ones, behind whole waves; and of a GEMM that leaves sums for a reduction.  Against 64-bit sums
+over the library's own cache, by the measure of the precision tests (the 128-row kernel's error); and bit for bit when repeated
+behind other lengths, whose sums lie in the same memory."""
+import pytest
+import torch
+
+import synth_inputs as si
+from tests import test_gpu_precision as prec
+
+pytestmark = pytest.mark.gpu
+
+CAP = 1088
+
+
+def _errors(sh, lengths, monkeypatch):
+    from paper_2412_18910_b200 import Engine
+    monkeypatch.setattr(prec, "CAP", CAP)
+    e = Engine(sh, si.make_weights(sh), kv_capacity=CAP)
+    try:
+        out = {}
+        for m in lengths + lengths[::-1]:
+            e.prefill(0, si.uniform_ids(29, "runs%d" % m, m, sh.vocab))
+            feat = e.ada_debug_buffer(0, torch.float32, (1, CAP, sh.d_model))[0, :m].clone()
+            if m in out:
+                assert torch.equal(feat, out[m][0]), m
+                continue
+            toks = e.ada_debug_buffer(2, torch.int32, (1, CAP))[0, :m]
+            out[m] = feat, prec._off(feat, prec._features(e, sh, 0, torch.arange(m, device=e.dev), toks))
+        assert e.ada_get_counters()["status"] == 0
+        return {m: x[1] for m, x in out.items()}
+    finally:
+        e.close()
+
+
+@pytest.mark.parametrize("shape,lengths", [
+    (dict(d_model=2048, n_heads=32, head_dim=64, d_ffn=11264), [129, 205, 256, 300, 517]),
+    (dict(d_model=5120, n_heads=40, head_dim=128, d_ffn=688), [205, 1000]),
+])
+def test_cut_tiles(shape, lengths, monkeypatch):
+    sh = si.scaled(si.SHAPES["tiny"], n_layers=1, vocab=272, **shape)
+    off = _errors(sh, [100] + lengths, monkeypatch)
+    for m in lengths:
+        assert off[m] < 1.05 * off[100], (m, off)
