@@ -113,6 +113,7 @@ __global__ void __launch_bounds__(kPaThreads, 1) k_attn_prompt(const AttnPromptA
   if (warp == 8) {
     // ------------------------------------------------------------- producer
     if (lane == 0) {
+#pragma unroll 1
       for (int t = 0; t < nmax; ++t) {
         const int s = t & 1;
         if (t >= 2) mbar_wait_inline(&empty[s], ((unsigned)(t >> 1) & 1u) ^ 1u, a.cnt, abort_s);
@@ -167,13 +168,13 @@ __global__ void __launch_bounds__(kPaThreads, 1) k_attn_prompt(const AttnPromptA
       }
       __syncwarp();
     };
-    for (int i = 0; i < 2; ++i)
-      if ((i ? n1 : n0) > 0) scores(i, 0);
-    for (int t = 0; t < nmax; ++t)
+#pragma unroll 1
+    for (int t = -1; t < nmax; ++t)
+#pragma unroll 1
       for (int i = 0; i < 2; ++i) {
         const int n = i ? n1 : n0;
         if (t >= n) continue;
-        values(i, t, i == 1 || t >= n1);
+        if (t >= 0) values(i, t, i == 1 || t >= n1);
         // (the softmax warps have read S of page t before they wrote its weights)
         if (t + 1 < n) scores(i, t + 1);
       }
@@ -269,8 +270,10 @@ __global__ void __launch_bounds__(kPaThreads, 1) k_attn_prompt(const AttnPromptA
           tmem_st8(tm + 96u + 8u * q4, pl);
         }
       };
-      for (int t = 0; t < n; ++t) {
+#pragma unroll 1
+      for (int t = 0;; ++t) {
         if (t > 0) add_o(t - 1);
+        if (t == n) break;
         mbar_wait_inline(&sfull[i], (unsigned)t & 1u, a.cnt, abort_s);
         tc_fence_after();
         const int key0 = t * kPageSize;
@@ -282,7 +285,6 @@ __global__ void __launch_bounds__(kPaThreads, 1) k_attn_prompt(const AttnPromptA
         __syncwarp();
         if (lane == 0) mbar_arrive(&pready[i]);
       }
-      add_o(n - 1);
       if (row < a.T) {
         const float inv = 1.f / l;
         __nv_bfloat16 *ph = a.xhi + (size_t)row * a.ldx + hh * HD, *pl = a.xlo + (size_t)row * a.ldx + hh * HD;
