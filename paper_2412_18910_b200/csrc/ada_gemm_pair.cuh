@@ -144,6 +144,13 @@ __device__ __forceinline__ float silu(float x) {
   return x > 88.f ? x : x < -80.f ? x * 0.f : z;
 }
 
+__device__ __forceinline__ uint4 pack8(const __nv_bfloat162 (&v)[4]) {
+  uint32_t u[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) u[k] = *reinterpret_cast<const uint32_t *>(&v[k]);
+  return make_uint4(u[0], u[1], u[2], u[3]);
+}
+
 // CUT: with tiles that pairs share (a kernel of its own: as a branch of one it cost the others 1.6 us a launch).
 template <int EPI, bool CUT>
 __global__ void __launch_bounds__(kPairThreads, 1) k_gemm_pair(const GemmPairArgs a) {
@@ -327,15 +334,15 @@ __global__ void __launch_bounds__(kPairThreads, 1) k_gemm_pair(const GemmPairArg
     pdl_wait();
     const int quarter = warp & 3, ch = (warp - 4) >> 2, etid = tid - 128;    // ch: which nb columns of the tile
     int n = 0;
-    // the lane that holds the other value of this thread's pair: gate / up are 64 lanes apart, rotary pairs hd / 2
+    // the other value of a pair: gate / up are 64 lanes apart, rotary pairs hd / 2
     const int dist = sw ? 2 : (a.hd == 128 ? 2 : 1);       // in warps
-    const bool low = (quarter & dist) == 0;
-    // exchange area of a warp: [16 prompt rows][32 weight rows], odd prompt rows with their halves swapped (an even and an odd
-    // lane then read from different banks)
-    const int par = lane & 1;
+    // Exchange area of a warp: [16 prompt rows][32 weight rows].  Thread gid of the four warps reads eight weight rows (w0, and those `dist`
+    // warps on) of prompt row gid / 8; the warps whose areas the same eight threads read have their groups of four swapped, so
+    // that the eight read from different banks.
     float *own_at = xch + (ch * 4 + quarter) * 16 * 32;
-    const float *low_at = xch + (ch * 4 + (low ? quarter : quarter ^ dist)) * 16 * 32 + ((lane ^ par) ^ (par << 4));
-    const float *high_at = xch + (ch * 4 + (low ? quarter ^ dist : quarter)) * 16 * 32 + ((lane ^ par) ^ (par << 4));
+    const int gid = etid & 127, wq = sw || a.hd == 128 ? (gid & 7) >> 2 : ((gid & 7) >> 2) * 2;
+    const float *low_at = xch + (ch * 4 + wq) * 16 * 32 + (gid >> 3) * 32 + 8 * (gid & 3), *high_at = low_at + dist * 16 * 32;
+    auto xch_swap = [](int q) { return ((q ^ (q >> 1)) & 1) << 2; };
     auto row_info = [&](int tok0, int Tl) {
       // per prompt row of the tile: 1/rms of its residual stream and, for keys and values, where its cache row starts
       for (int i = etid; i < Tl; i += 256) {
@@ -426,11 +433,9 @@ __global__ void __launch_bounds__(kPairThreads, 1) k_gemm_pair(const GemmPairArg
           }
         }
       }
-      const int row = (sw ? tile * 128 + (int)rank * 64 : tile * 256 + (int)rank * 128) +
-                      (sw ? (quarter & 1) * 32 + lane : quarter * 32 + lane);     // weight row inside its matrix
       if constexpr (EPI == PAIR_PART) {
         // By way of the warp's exchange area, 16 prompt rows at a time, so that a lane stores four weight rows of a prompt row at once.
-        const int row4 = row - lane + 4 * (lane & 7), rows = min(a.nb, Tl - ch * a.nb);
+        const int row4 = tile * 256 + (int)rank * 128 + quarter * 32 + 4 * (lane & 7), rows = min(a.nb, Tl - ch * a.nb);
         float *pp = a.part + ((size_t)split * a.part_rows + tok0 + ch * a.nb + (lane >> 3)) * a.Nseg + row4;
 #pragma unroll 1
         for (int b16 = 0; b16 * 16 < rows; ++b16) {
@@ -448,21 +453,21 @@ __global__ void __launch_bounds__(kPairThreads, 1) k_gemm_pair(const GemmPairArg
               __stcg(reinterpret_cast<float4 *>(pp), *reinterpret_cast<const float4 *>(own_at + k * 32 + 4 * lane));
         }
       } else {
-        // A thread finishes two neighbouring weight rows of every other prompt row (row by row the stores were of two bytes, and
-        // the warps' time went into them).  The low threads of a pair take prompt rows 0 .. 7 of a block of 16, the high
-        // threads the other eight.
-        const int half = a.hd >> 1, row2 = row - par;
-        const int hh = sw ? 0 : row2 / a.hd, il = sw ? 0 : (row2 - hh * a.hd) & (half - 1);   // head, index of the pair
+        // A thread finishes eight neighbouring weight rows (and the eight that they are paired with) of one of 16 prompt rows, so that what
+        // it stores are 16 bytes or more and a row's information is read once.  (Two
+        // weight rows of four prompt rows a thread: the tile of a CTA took 6.3 thousand clocks at nb = 64 for 3.9 now, SwiGLU, and 19 for 17 at nb
+        // = 128, queries; four layers of 2048 and 333 rows 677 -> 665 us, 7B 205 rows 1169 -> 1153.)
+        const int half = a.hd >> 1, gr = gid & 7, w0 = sw || a.hd == 128 ? 8 * gr : 64 * (gr >> 2) + 8 * (gr & 3);
+        const int row = (sw ? tile * 128 + (int)rank * 64 : tile * 256 + (int)rank * 128) + w0;   // first weight row inside its matrix
+        const int hh = sw ? 0 : row / a.hd, il = sw ? 0 : row - hh * a.hd;                         // head, index of the first pair
         const size_t head_off = (size_t)hh * kPageSize * a.hd;
-        const int k0 = (low ? 0 : 8) + par;
         named_bar(3, 256);   // the rows' information is complete
         float4 cs[4];        // rotary factors of the block, requested a block ahead
         auto rotary = [&](int tb) {
           if constexpr (!sw) {
+            const float4 *f = reinterpret_cast<const float4 *>(a.rope + (size_t)t_pos[min(tb + (gid >> 3), Tl - 1)] * half + il);
 #pragma unroll
-            for (int k = 0; k < 4; ++k)
-              cs[k] = seg < 2 ? __ldg(reinterpret_cast<const float4 *>(a.rope + (size_t)t_pos[min(tb + k0 + 2 * k, Tl - 1)] * half + il))
-                              : make_float4(1.f, 0.f, 1.f, 0.f);
+            for (int k = 0; k < 4; ++k) cs[k] = seg < 2 ? __ldg(f + k) : make_float4(1.f, 0.f, 1.f, 0.f);
           }
         };
         rotary(ch * a.nb);
@@ -471,58 +476,63 @@ __global__ void __launch_bounds__(kPairThreads, 1) k_gemm_pair(const GemmPairArg
         // tile against 14 for the next.
 #pragma unroll 1
         for (int b16 = 0; b16 * 16 < min(a.nb, Tl - ch * a.nb); ++b16) {     // (uniform over the four warps that exchange)
-          const int tb = ch * a.nb + b16 * 16;
+          const int tb = ch * a.nb + b16 * 16, i = tb + (gid >> 3);
           named_bar(1 + ch, 128);
 #pragma unroll
           for (int b = 0; b < 8; ++b)
             if (b == b16) {
 #pragma unroll
-              for (int k = 0; k < 16; ++k) own_at[k * 32 + (lane ^ ((k & 1) << 4))] = sum[b >> 1][(b & 1) * 16 + k];
+              for (int k = 0; k < 16; ++k) own_at[k * 32 + (lane ^ xch_swap(quarter))] = sum[b >> 1][(b & 1) * 16 + k];
             }
           named_bar(1 + ch, 128);
-          // all reads first, then the arithmetic and the stores (row by row every read waited behind the stores of the row
-          // before it, which might have been to the same place)
-          float2 x[4], y[4];        // (gate, up) or rows (i, i + hd / 2)
+          float x[8], y[8];        // (gate, up) or rows (i, i + hd / 2)
+          const float inv = t_inv[i];
 #pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            const float inv = t_inv[tb + k0 + 2 * k];
-            x[k] = *reinterpret_cast<const float2 *>(low_at + (k0 + 2 * k) * 32);
-            y[k] = *reinterpret_cast<const float2 *>(high_at + (k0 + 2 * k) * 32);
-            x[k].x *= inv; x[k].y *= inv; y[k].x *= inv; y[k].y *= inv;
+          for (int k = 0; k < 2; ++k) {
+            const float4 u = *reinterpret_cast<const float4 *>(low_at + ((4 * k) ^ xch_swap(wq))), v = *reinterpret_cast<const float4 *>(high_at + ((4 * k) ^ xch_swap(wq + dist)));
+            x[4 * k] = u.x * inv; x[4 * k + 1] = u.y * inv; x[4 * k + 2] = u.z * inv; x[4 * k + 3] = u.w * inv;
+            y[4 * k] = v.x * inv; y[4 * k + 1] = v.y * inv; y[4 * k + 2] = v.z * inv; y[4 * k + 3] = v.w * inv;
           }
           float4 c[4];
 #pragma unroll
           for (int k = 0; k < 4; ++k) c[k] = cs[k];
           if ((b16 + 1) * 16 < a.nb) rotary(tb + 16);
-          if (row2 >= a.Nseg) continue;
+          if (row >= a.Nseg || i >= Tl) continue;
+          if constexpr (sw) {
+            __nv_bfloat162 hi[4], lo[4];
 #pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            const int i = tb + k0 + 2 * k;
-            if (i >= Tl) continue;
-            if constexpr (sw) {
-              __nv_bfloat162 hi, lo;
-              split_bf16(silu(x[k].x) * y[k].x, hi.x, lo.x);
-              split_bf16(silu(x[k].y) * y[k].y, hi.y, lo.y);
-              const size_t o = (size_t)(tok0 + i) * a.ldo + row2;
-              *reinterpret_cast<__nv_bfloat162 *>(a.ohi + o) = hi;
-              *reinterpret_cast<__nv_bfloat162 *>(a.olo + o) = lo;
-            } else {
-              float2 v0, v1;   // (values: x and y as they are)
-              v0.x = x[k].x * c[k].x - y[k].x * c[k].y; v0.y = x[k].y * c[k].z - y[k].y * c[k].w;
-              v1.x = y[k].x * c[k].x + x[k].x * c[k].y; v1.y = y[k].y * c[k].z + x[k].y * c[k].w;
-              if (seg == 0) {
-                float *q = a.qout + (size_t)(tok0 + i) * a.d + hh * a.hd + il;
-                *reinterpret_cast<float2 *>(q) = make_float2(v0.x * a.qscale, v0.y * a.qscale);
-                *reinterpret_cast<float2 *>(q + half) = make_float2(v1.x * a.qscale, v1.y * a.qscale);
-              } else {
-                const int s7 = t_pos[i] & 7;
-                const int o0 = (((il >> 3) ^ s7) << 3) | (il & 7), o1 = ((((il + half) >> 3) ^ s7) << 3) | (il & 7);
-                __nv_bfloat16 *pool = (seg == 1 ? a.kpool : a.vpool) + t_base[i] + head_off;
-                __nv_bfloat162 w0, w1;
-                w0.x = kv_store(v0.x); w0.y = kv_store(v0.y); w1.x = kv_store(v1.x); w1.y = kv_store(v1.y);
-                *reinterpret_cast<__nv_bfloat162 *>(pool + o0) = w0;
-                *reinterpret_cast<__nv_bfloat162 *>(pool + o1) = w1;
+            for (int k = 0; k < 4; ++k) {
+              split_bf16(silu(x[2 * k]) * y[2 * k], hi[k].x, lo[k].x);
+              split_bf16(silu(x[2 * k + 1]) * y[2 * k + 1], hi[k].y, lo[k].y);
+            }
+            const size_t o = (size_t)(tok0 + i) * a.ldo + row;
+            *reinterpret_cast<uint4 *>(a.ohi + o) = pack8(hi);
+            *reinterpret_cast<uint4 *>(a.olo + o) = pack8(lo);
+          } else {
+            float v0[8], v1[8];   // (values: x and y as they are)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              v0[2 * k] = x[2 * k] * c[k].x - y[2 * k] * c[k].y; v0[2 * k + 1] = x[2 * k + 1] * c[k].z - y[2 * k + 1] * c[k].w;
+              v1[2 * k] = y[2 * k] * c[k].x + x[2 * k] * c[k].y; v1[2 * k + 1] = y[2 * k + 1] * c[k].z + x[2 * k + 1] * c[k].w;
+            }
+            if (seg == 0) {
+              float *q = a.qout + (size_t)(tok0 + i) * a.d + hh * a.hd + il;
+#pragma unroll
+              for (int k = 0; k < 8; k += 4) {
+                *reinterpret_cast<float4 *>(q + k) = make_float4(v0[k] * a.qscale, v0[k + 1] * a.qscale, v0[k + 2] * a.qscale, v0[k + 3] * a.qscale);
+                *reinterpret_cast<float4 *>(q + half + k) = make_float4(v1[k] * a.qscale, v1[k + 1] * a.qscale, v1[k + 2] * a.qscale, v1[k + 3] * a.qscale);
               }
+            } else {
+              const int s7 = t_pos[i] & 7;
+              __nv_bfloat16 *pool = (seg == 1 ? a.kpool : a.vpool) + t_base[i] + head_off;
+              __nv_bfloat162 p0[4], p1[4];
+#pragma unroll
+              for (int k = 0; k < 4; ++k) {
+                p0[k].x = kv_store(v0[2 * k]); p0[k].y = kv_store(v0[2 * k + 1]);
+                p1[k].x = kv_store(v1[2 * k]); p1[k].y = kv_store(v1[2 * k + 1]);
+              }
+              *reinterpret_cast<uint4 *>(pool + (((il >> 3) ^ s7) << 3)) = pack8(p0);
+              *reinterpret_cast<uint4 *>(pool + ((((il + half) >> 3) ^ s7) << 3)) = pack8(p1);
             }
           }
         }
