@@ -77,7 +77,7 @@ struct ada_ctx {
   TensorMap128 *d_tcmaps;
   int n_tcmaps;
   std::unordered_map<const void *, int> tcmap_of;
-  std::unordered_map<const void *, int> pairmap_of;   // prompt passes: gate and up in boxes of 64 rows, planes in boxes of 32, 64, 96, 128 rows (four maps)
+  std::unordered_map<const void *, int> pairmap_of;   // prompt passes: gate and up in boxes of 64 rows; planes (of all multi-row passes) in boxes of 8, 16, .. 128 rows (sixteen maps)
   LayerPtrs *d_layers, *d_eagle;
   TensorMap128 *d_maps;
   int n_maps;
@@ -368,7 +368,7 @@ size_t carve(ada_ctx *x, const ada_config *c, int rows, char *base) {
   x->d_eagle = w.take<LayerPtrs>(1);
   x->n_maps = (int)(7 * (L + 1) + 2);
   x->d_maps = w.take<TensorMap128>(x->n_maps);
-  x->n_tcmaps = (int)(9 * (L + 1) + 2 + 4 + 4 + 16);   // weights (gate and up twice), planes of decode passes, cache pools, planes of prompt passes
+  x->n_tcmaps = (int)(9 * (L + 1) + 2 + 4 + 4 * 16);   // weights (gate and up twice), cache pools, planes
   x->d_tcmaps = w.take<TensorMap128>(x->n_tcmaps);
   x->xa = w.take<bf16>(((d + 63) / 64) * (kPassRowsMax * 128));
   x->at = w.take<bf16>(((d + 63) / 64) * (kPassRowsMax * 128));
@@ -432,8 +432,8 @@ bool gemm_prompt(ada_ctx *x, int epi, const bf16 *W0, const bf16 *W1, const bf16
   const bf16 *Ws[3] = {W0, W1, W2};
   for (int i = 0; i < 3; ++i)
     if (Ws[i] && !(t.wmap[i] = find_map(x, sw ? x->pairmap_of : x->tcmap_of, Ws[i]))) return no_map(x);
-  t.xhi_map = find_map(x, x->pairmap_of, Xhi, plan.nb / 32 - 1);
-  t.xlo_map = find_map(x, x->pairmap_of, Xlo, plan.nb / 32 - 1);
+  t.xhi_map = find_map(x, x->pairmap_of, Xhi, plan.nb / 8 - 1);
+  t.xlo_map = find_map(x, x->pairmap_of, Xlo, plan.nb / 8 - 1);
   if (!t.xhi_map || !t.xlo_map) return no_map(x);
   t.part = x->gemm_part; t.part_rows = x->TM;
   t.ss_part = x->ss_rows; t.eps = c.rms_eps; t.d = c.d_model;
@@ -468,8 +468,8 @@ bool gemm(ada_ctx *x, int epi, const bf16 *W0, const bf16 *W1, const bf16 *W2, i
   const bf16 *Ws[3] = {W0, W1, W2};
   for (int i = 0; i < 3; ++i)
     if (Ws[i] && !(t.wmap[i] = find_map(x, x->tcmap_of, Ws[i]))) return no_map(x);
-  t.xhi_map = chunk ? find_map(x, x->pairmap_of, Xhi, kTcRowsMax / 32 - 1) : find_map(x, x->tcmap_of, Xhi);
-  t.xlo_map = chunk ? find_map(x, x->pairmap_of, Xlo, kTcRowsMax / 32 - 1) : find_map(x, x->tcmap_of, Xlo);
+  t.xhi_map = find_map(x, x->pairmap_of, Xhi);
+  t.xlo_map = find_map(x, x->pairmap_of, Xlo);
   if (!t.xhi_map || !t.xlo_map) return no_map(x);
   t.epi = epi; t.nseg = nseg; t.Nseg = Nseg; t.K = K;
   const int tiles = tc_tiles(epi, nseg, Nseg);
@@ -643,9 +643,9 @@ bool build_maps(ada_ctx *x, std::vector<TensorMap128> &maps) {
   return ok;
 }
 
-// Tensor maps of the multi-row tensor-core GEMMs: every weight matrix with a box of 64 k x 128 rows, the four
-// activation planes with a box of 64 k x 88 rows; tcmap_of finds a map by the base pointer of its tensor.  Prompt passes:
-// gate and up in boxes of 64 rows, the planes in boxes of 32, 64, 96 and 128 rows (pairmap_of finds the first of the four).
+// Tensor maps of the multi-row tensor-core GEMMs: every weight matrix with a box of 64 k x 128 rows; tcmap_of finds a map by the base
+// pointer of its tensor.  Gate and up of prompts in boxes of 64 rows, the four activation planes in boxes of 8, 16, .. 128 rows
+// (pairmap_of finds the first of the sixteen).
 bool build_tc_maps(ada_ctx *x, std::vector<TensorMap128> &maps) {
   void *sym = nullptr;
   cudaDriverEntryPointQueryResult q;
@@ -671,8 +671,6 @@ bool build_tc_maps(ada_ctx *x, std::vector<TensorMap128> &maps) {
   add(x->eagle_fc, d, 2 * d, 128);
   add(x->lm_head, V, d, 128);
   const size_t rows = x->prompt_rows;
-  add(x->xhi, rows, x->ldx, kTcRows); add(x->xlo, rows, x->ldx, kTcRows);
-  add(x->x2hi, rows, x->ldx2, kTcRows); add(x->x2lo, rows, x->ldx2, kTcRows);
   // the cache pools as rows of head_dim 16-bit elements, whose chunks are stored swizzled already (attention of prompts)
   auto add_pool = [&](const void *base, size_t rows) {
     ok = ok && next < x->n_tcmaps && encode_map(fn, &maps[next], base, rows, c.head_dim, 64, false);
@@ -690,10 +688,10 @@ bool build_tc_maps(ada_ctx *x, std::vector<TensorMap128> &maps) {
   auto gate_up = [&](const LayerW &a) { add_pair(a.wg, F, d, 64); add_pair(a.wu, F, d, 64); };
   for (int l = 0; l < c.n_layers; ++l) gate_up(x->layers[l]);
   gate_up(x->eagle);
-  for (unsigned box = 32; box <= 128; box += 32) add_pair(x->xhi, rows, x->ldx, box);
-  for (unsigned box = 32; box <= 128; box += 32) add_pair(x->xlo, rows, x->ldx, box);
-  for (unsigned box = 32; box <= 128; box += 32) add_pair(x->x2hi, rows, x->ldx2, box);
-  for (unsigned box = 32; box <= 128; box += 32) add_pair(x->x2lo, rows, x->ldx2, box);
+  for (unsigned box = 8; box <= 128; box += 8) add_pair(x->xhi, rows, x->ldx, box);
+  for (unsigned box = 8; box <= 128; box += 8) add_pair(x->xlo, rows, x->ldx, box);
+  for (unsigned box = 8; box <= 128; box += 8) add_pair(x->x2hi, rows, x->ldx2, box);
+  for (unsigned box = 8; box <= 128; box += 8) add_pair(x->x2lo, rows, x->ldx2, box);
   return ok;
 }
 

@@ -8,15 +8,15 @@
 // (grid.y splits); level-2 to shared-memory traffic then stays below 1.7 times the weight bytes.
 //
 //   warp 0   producer, one thread: per 64 k one stage = weight boxes (TMA tiled loads, 128-byte swizzle, box 64 k x 128
-//            rows) + the hi plane box and the lo plane box of the activations (64 k x ROWS rows each, stacked so that
-//            they form one K-major operand of 2 ROWS rows); 4 stages of 54 KB (ROWS = 88) or 3 of 64 KB (ROWS = 128),
+//            rows) + the hi plane box and the lo plane box of the activations (64 k x the pass's rows rounded up to eight, stacked so
+//            that they form one K-major operand of twice as many rows); 4 stages of 54 KB (ROWS = 88) or 3 of 64 KB (ROWS = 128),
 //            mbarrier transaction counts
-//   warp 1   one elected thread issues tcgen05.mma (M = 128, N = 2 ROWS, K = 16) per m tile and 16 k straight from the
-//            TMA-written tiles; accumulators in tensor memory (m tile i in columns [256 i, 256 i + 2 ROWS));
+//   warp 1   one elected thread issues tcgen05.mma (M = 128, N = 2 x rows, K = 16) per m tile and 16 k straight from the
+//            TMA-written tiles; accumulators in tensor memory (m tile i in columns [256 i, 256 i + N));
 //            tcgen05.commit frees the stage and, at the end, signals the accumulators
 //   warp 2   owns the tensor-memory allocation (512 columns)
 //   warps 4..11  epilogue: thread = one weight row (tensor-memory lane), tcgen05.ld eight pass rows at a time,
-//            column t (hi) + column ROWS + t (lo)
+//            column t (hi) + column N / 2 + t (lo)
 //
 // Every CTA leaves its sums in a scratch buffer and a reduction kernel, launched next, adds the K splits in split
 // order and runs everything up to the next GEMM's input over the whole grid (k_reduce_h, k_reduce_qkv,
@@ -32,23 +32,21 @@ constexpr int kTcRowsMax = 128;                      // rows of a prompt pass th
 constexpr int kTcABytes = 128 * 128;                 // one weight box: 128 rows x 64 k bf16
 constexpr int kTcThreads = 12 * 32;
 constexpr int kTcTmemCols = 512;
-// Shapes of the two instantiations: ROWS = 88 (N = 176, four 54 KB stages) and ROWS = 128 (N = 256, the largest N of one
+// Shapes of the two instantiations: ROWS = 88 (N up to 176, four 54 KB stages) and ROWS = 128 (N up to 256, the largest N of one
 // product and exactly the 2 x 256 accumulator columns; three 64 KB stages).
 template <int ROWS>
 struct TcShape {
-  static constexpr int kN = 2 * ROWS;                          // MMA N: hi rows then lo rows
   static constexpr int kBBytes = ROWS * 128;                   // one plane box
   static constexpr int kStageBytes = 2 * kTcABytes + 2 * kBBytes;
   static constexpr int kStages = ROWS <= 88 ? 4 : 3;
   static constexpr int kSmemBytes = 1024 + kStages * kStageBytes + 256;
-  static_assert(kBBytes % 1024 == 0, "the lo plane must start on a swizzle-atom boundary");
   static_assert(kSmemBytes <= 227 * 1024, "shared memory budget");
-  static_assert(kN <= 256 && kN % 16 == 0, "N of one product");
+  static_assert(ROWS <= 128 && ROWS % 8 == 0, "N of one product is twice the rows");
 };
 
 struct GemmTcArgs {
   const TensorMap128 *wmap[3];   // box {64 k, 128 rows}; STORE: up to 3 row segments; SWIGLU: gate, up
-  const TensorMap128 *xhi_map, *xlo_map;   // planes [128][ld]: box {64 k, ROWS rows}
+  const TensorMap128 *xhi_map, *xlo_map;   // planes: sixteen maps each, box {64 k, 8, 16, .. 128 rows}
   int epi;                    // EPI_STORE / EPI_RESID / EPI_SWIGLU (sums go to `part`) / EPI_ARGMAX
   int nseg, Nseg, K;
   int S;                      // K splits (grid.y)
@@ -91,7 +89,7 @@ __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.
 template <int ROWS>
 __global__ void __launch_bounds__(kTcThreads, 1) k_gemm_tc(const GemmTcArgs a) {
   using Sh = TcShape<ROWS>;
-  constexpr int kTcStages = Sh::kStages, kTcStageBytes = Sh::kStageBytes, kTcBBytes = Sh::kBBytes, kTcN = Sh::kN;
+  constexpr int kTcStages = Sh::kStages, kTcStageBytes = Sh::kStageBytes;
   pdl_launch_dependents();   // the next kernel may start its prologue; it waits for this grid to complete before it reads
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const bool sw = a.epi == EPI_SWIGLU;
@@ -118,21 +116,26 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_gemm_tc(const GemmTcArgs a) {
   // tensor memory is allocated and the CTA meets at the barrier below.
   const TensorMap128 *m0 = sw || seg == 0 ? a.wmap[0] : seg == 1 ? a.wmap[1] : a.wmap[2];   // (indexed, the arguments are copied to memory)
   const TensorMap128 *m1 = sw ? a.wmap[1] : m0;
-  const unsigned tx = (unsigned)(mtiles * kTcABytes + 2 * kTcBBytes);
   // level-2 policies: the weights pass through once (evict first), every CTA of a launch reads the same plane boxes (evict
   // last); what is read again soon -- planes, partial sums -- then stays in level 2 while 400 MB of weights stream by
   // (128-row layer: 131.6 -> 106.2 us for the four GEMMs)
   const uint64_t pol_w = l2_policy_evict_first(), pol_x = l2_policy_evict_last();
-  auto load_weights = [&](int kb, int s) {   // arms the stage's barrier for the whole stage
+  // Of the planes come the pass's rows, rounded up to eight (nrow), and the products have as many columns: with 88 rows whatever the pass's
+  // a CTA took 54 KB a box from level 2 in the time that HBM gives it 32 KB of weights, which is all that level 2 can hand out (40 bytes a
+  // clock and SM).  Eight sequences of 7B, verify of 48 rows: 4710 -> 4440 us, of the middle model 1113 -> 1080; prompts of 49, 77 and 128 rows,
+  // four layers of 7B: 721, 771, 836 -> 677, 738, 833.
+  int nrow;
+  auto load_weights = [&](int kb, int s) {   // their bytes, before the rows are known; load_planes arms the barrier for the stage
     unsigned char *st = smem + (size_t)s * kTcStageBytes;
-    mbar_expect_tx(&full[s], tx);
+    mbar_expect_more(&full[s], (unsigned)(mtiles * kTcABytes));
     tma_load_2d_hint(st, m0, kb * 64, row0, &full[s], pol_w);     // rows past the matrix and k past K read as zero
     if (mtiles > 1) tma_load_2d_hint(st + kTcABytes, m1, kb * 64, row1, &full[s], pol_w);
   };
   auto load_planes = [&](int kb, int s) {
     unsigned char *st = smem + (size_t)s * kTcStageBytes;
-    tma_load_2d_hint(st + 2 * kTcABytes, a.xhi_map, kb * 64, a.xrow0, &full[s], pol_x);
-    tma_load_2d_hint(st + 2 * kTcABytes + kTcBBytes, a.xlo_map, kb * 64, a.xrow0, &full[s], pol_x);
+    mbar_expect_tx(&full[s], (unsigned)(2 * nrow * 128));
+    tma_load_2d_hint(st + 2 * kTcABytes, a.xhi_map + (nrow / 8 - 1), kb * 64, a.xrow0, &full[s], pol_x);
+    tma_load_2d_hint(st + 2 * kTcABytes + nrow * 128, a.xlo_map + (nrow / 8 - 1), kb * 64, a.xrow0, &full[s], pol_x);
   };
   // Weights depend on no earlier kernel: the first stages' weight boxes are requested before this grid waits for
   // the grid before it (programmatic dependent launch), the activation boxes after; the tensor memory is allocated
@@ -145,6 +148,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_gemm_tc(const GemmTcArgs a) {
   __syncthreads();
   const bool ahead = ahead_s != 0;
   int T;
+  auto rows_of = [](int T) { return min(ROWS, max(8, (T + 7) & ~7)); };
   if (tid == 0) {
     *abort_s = 0;
     for (int i = 0; i < kTcStages; ++i) { mbar_init(&full[i], 1); mbar_init(&empty[i], 1); }
@@ -155,6 +159,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_gemm_tc(const GemmTcArgs a) {
       for (int i = 0; i < nfirst; ++i) load_weights(kb0 + i, i);
     pdl_wait();
     T = a.use_lm_rows ? a.pass->lmT : a.pass->T;
+    nrow = rows_of(T);
 #pragma unroll 1
     for (int i = 0; i < nfirst && (ahead || T > 0); ++i) {
       if (!ahead) load_weights(kb0 + i, i);
@@ -164,6 +169,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_gemm_tc(const GemmTcArgs a) {
     if (warp == 2 && ahead) tmem_alloc(tmem_slot, kTcTmemCols);
     pdl_wait();
     T = a.use_lm_rows ? a.pass->lmT : a.pass->T;
+    nrow = rows_of(T);
     if (warp == 2 && !ahead && T > 0) tmem_alloc(tmem_slot, kTcTmemCols);
   }
   const bool idle = T <= 0;   // a pass without rows: requested stages are awaited, nothing is computed or stored
@@ -187,7 +193,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_gemm_tc(const GemmTcArgs a) {
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------- tensor-core issuer
-    constexpr uint32_t idesc = umma_idesc_mn(128u, (uint32_t)kTcN);
+    const uint32_t idesc = umma_idesc_mn(128u, 2u * __reduce_max_sync(0xffffffffu, (uint32_t)nrow));   // hi rows, then lo rows
     // operands from values that are the same in all lanes as far as the compiler can see, and no loops over a whole box:
     // products whose operands have to be fetched from a lane first issue at 80 clocks each (eight sequences, 7B: verify
     // 5464 -> 5361 us)
@@ -248,7 +254,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_gemm_tc(const GemmTcArgs a) {
       for (int i = 0; i < 8; ++i) y[i] = 0.f;
       if (!active_warp || kb1 <= kb0) return;     // (warp-uniform)
       tmem_ld8(taddr + (uint32_t)(8 * j), hi);
-      tmem_ld8(taddr + (uint32_t)(ROWS + 8 * j), lo);
+      tmem_ld8(taddr + (uint32_t)(nrow + 8 * j), lo);
 #pragma unroll
       for (int i = 0; i < 8; ++i) y[i] = hi[i] + lo[i];
     };
@@ -269,7 +275,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_gemm_tc(const GemmTcArgs a) {
         uint32_t hi[32], lo[32];
         if (have) {
           tmem_ld32_issue(paddr + (uint32_t)c0, hi);
-          tmem_ld32_issue(paddr + (uint32_t)(ROWS + c0), lo);
+          tmem_ld32_issue(paddr + (uint32_t)(nrow + c0), lo);
           tmem_ld_wait();
         } else {
 #pragma unroll

@@ -192,6 +192,10 @@ __device__ __forceinline__ void mbar_expect_tx(uint64_t *bar, unsigned bytes) {
                "r"(bytes)
                : "memory");
 }
+// ... without the arrival: bytes that the phase awaits beyond those of the arrival to come
+__device__ __forceinline__ void mbar_expect_more(uint64_t *bar, unsigned bytes) {
+  asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
+}
 __device__ __forceinline__ bool mbar_try(uint64_t *bar, unsigned parity) {
   unsigned ok;
   asm volatile(
