@@ -238,11 +238,13 @@ size_t part_need_tc(int epi, int nseg, int Nseg, int K) {
 }
 
 // Tile of a prompt GEMM: prompt rows per CTA, token tiles, K splits.  Estimated time of a candidate = waves of 74 pairs x
-// (64-k boxes of an item x the slower of the products, 8 nb clocks per box, and the loads, about 48 bytes per clock and
+// (64-k boxes of an item x the slower of the products, 8 nb clocks per box, and the loads, about 40 bytes per clock and
 // SM, + an item's start and end), not less than the weights at the HBM rate, + what the splits' sums cost.  The load rate is
-// that of the kernel (750 clocks a box at nb = 64, 820 at 96, little more than the products' time at 128).  At 60 bytes tiles
-// of 64 rows came out too cheap: a prompt of 512 tokens 14.4 -> 13.4 ms (7B), 333 tokens 10.7 -> 10.3; 16 layers of 2048: 333
-// tokens 2033 -> 1932 us, 129 tokens 1563 -> 1496, 640 tokens 2785 -> 2820.
+// that of the kernel with all SMs loading (812 clocks a box at nb = 64; 1010 at 128, the products' time, on 96 SMs).  Prompt rows per
+// CTA in steps of eight, so that a tile ends where the prompt does: in steps of 32 (and 48 bytes) four layers of 7B took 988 us for 130
+// tokens -> 923, 205 1151 -> 1065, 333 1578 -> 1541, 400 1863 -> 1700, 512 1936 -> 1921, 600 2627 -> 2250, 850 3287 -> 3038; of 13B, 205
+// tokens 1529 -> 1432, 600 3798 -> 3496; of 2048, 333 tokens 661 -> 658, 400 770 -> 705.  A step that is no multiple of 32 has to be 1 %
+// faster: where the two come out alike the wider tile was (13B, 512 tokens: 2777 against 2818).
 // 64-k boxes per accumulator, so that a prompt's features are no further from 64-bit sums than with the 128-row kernel, whose K
 // splits get shorter with K.  Two layers, 333 tokens, 128-row kernel in chunks -> pairs: d_model 4096 6.8e-6 -> 6.3e-6 with 4
 // boxes, 2048 4.54e-6 -> 4.48e-6 with 4 (4.89e-6 with 8), 1024 1.99e-6 -> 2.01e-6 and 256 2.64e-7 -> 2.58e-7 with 2 (2.76e-7 with 4).  With
@@ -257,17 +259,17 @@ PairPlan plan_pair(int T, int weight_tiles, int N, int K, bool may_split, size_t
   PairPlan cut = best;
   double best_us = 1e30, cut_us = 1e30;
   const int kboxes = (K + 63) / 64;
-  for (int nb = 32; nb <= 128; nb += 32) {
+  for (int nb = 32; nb <= 128; nb += 8) {
     const int tt = (T + 2 * nb - 1) / (2 * nb);
+    const double clk_box = fmax(8.0 * nb, (16384.0 + 256.0 * nb) / 40.0) * (nb % 32 ? 1.01 : 1.0);
     for (int S = 1; S <= (may_split ? 8 : 1) && S <= kboxes && (S == 1 || (S * T <= kPairSplitRows && S * (size_t)T <= split_rows)); ++S) {
       const int items = tt * weight_tiles * S, waves = (items + kPairs - 1) / kPairs;
-      const double clk_box = fmax(8.0 * nb, (16384.0 + 256.0 * nb) / 48.0);
       double us = waves * ((double)((kboxes + S - 1) / S) * clk_box / 1900.0 + 2.0);
       us = fmax(us, 2.0 * N * (double)K / 6.4e6) + (S > 1 ? 8.0 * S * (double)T * N / 4.0e6 : 0.0);
       if (us < best_us) { best_us = us; best = PairPlan{nb, tt, S, items}; }
     }
     // All whole waves but one, the rest cut into runs of accumulators as long for every pair.  The cut tiles' sums are put at 10 us at nb
-    // = 128, and the cut has to come out below 0.92 of the time (weights of several token tiles come from HBM more than once).  GEMMs
+    // = 128, and the cut has to come out below 0.9 of the time (weights of several token tiles come from HBM more than once).  GEMMs
     // that may be split along K only at the widest tiles and with one for every pair at least: more cuts a tile, or narrower tiles,
     // cost more than an idle part of a wave (13B down of 640 rows 160 -> 188 us).  Four layers and the head, prompts of 130, 205, 256, 333,
     // 512 and 1000 tokens, whole tiles -> so: 7B 1119, 1285, 1317, 1660, 2015 -> 1012, 1182, 1210, 1620, 1975 us (1000: not cut), 13B
@@ -275,14 +277,13 @@ PairPlan plan_pair(int T, int weight_tiles, int N, int K, bool may_split, size_t
     const int kruns = (kboxes + chunk - 1) / chunk, items = tt * weight_tiles;
     const size_t sums = (may_split ? (size_t)T * N : 0) + (size_t)kPairs * 2 * 128 * 2 * nb;
     if (sums <= scratch && items * kruns >= kPairs && (!may_split || (nb == 128 && items >= kPairs))) {
-      const double clk_box = fmax(8.0 * nb, (16384.0 + 256.0 * nb) / 48.0);
       const int waves = std::max(0, items / kPairs - 1), rest = items - waves * kPairs;
       double us = waves * (kboxes * clk_box / 1900.0 + 2.0) + (double)((rest * kruns + kPairs - 1) / kPairs) * chunk * clk_box / 1900.0 + 2.0 + 10.0 * nb / 128.0;
       us = fmax(us, 2.0 * N * (double)K / 6.4e6);
       if (us < cut_us) { cut_us = us; cut = PairPlan{nb, tt, 1, waves * kPairs}; }
     }
   }
-  return cut_us < 0.92 * best_us ? cut : best;
+  return cut_us < 0.9 * best_us ? cut : best;
 }
 
 // Rows of a prompt chunk (and of the row scratch) that an engine asks for; ada_init takes the most, down to 128, that the

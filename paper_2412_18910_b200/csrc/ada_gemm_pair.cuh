@@ -60,7 +60,7 @@ struct GemmPairArgs {
   const TensorMap128 *xhi_map, *xlo_map;   // planes, box {64 k, nb rows}
   int nseg, Nseg, K;
   int T;                                   // rows of the pass (known on the host)
-  int nb;                                  // prompt rows per CTA and tile: 32, 64, 96 or 128
+  int nb;                                  // prompt rows per CTA and tile: 32, 40, .. 128
   int token_tiles, weight_tiles, S;        // S: K splits (PART only)
   int chunk;                               // 64-k boxes per accumulator
   int whole;                               // tiles (and splits) dealt whole; the rest (S = 1) in equal runs to all pairs
@@ -395,10 +395,10 @@ __global__ void __launch_bounds__(kPairThreads, 1) k_gemm_pair(const GemmPairArg
         if (kb0 > 0) {
           float *o = a.cut + (size_t)blockIdx.x * N * 128 + at;
 #pragma unroll
-          for (int blk = 0; blk < 4; ++blk)
-            if (blk * 32 < a.nb) {
+          for (int blk = 0; blk < 16; ++blk)
+            if (blk * 8 < a.nb) {
 #pragma unroll
-              for (int i = 0; i < 32; ++i) __stcg(o + (size_t)(blk * 32 + i) * 128, sum[blk][i]);
+              for (int i = 0; i < 8; ++i) __stcg(o + (size_t)(blk * 8 + i) * 128, sum[blk >> 2][(blk & 3) * 8 + i]);
             }
           __syncwarp();
           if (lane == 0) asm volatile("st.release.gpu.global.s32 [%0], 1;" ::"l"(a.cut_flags + blockIdx.x * 8 + ew) : "memory");
@@ -424,7 +424,7 @@ __global__ void __launch_bounds__(kPairThreads, 1) k_gemm_pair(const GemmPairArg
               if (blk * 32 < a.nb) {
                 float v[32];
 #pragma unroll
-                for (int i = 0; i < 32; ++i) v[i] = __ldcg(q + (size_t)(blk * 32 + i) * 128);
+                for (int i = 0; i < 32; ++i) v[i] = blk * 32 + (i & ~7) < a.nb ? __ldcg(q + (size_t)(blk * 32 + i) * 128) : 0.f;
 #pragma unroll
                 for (int i = 0; i < 32; ++i) sum[blk][i] += v[i];
               }
@@ -497,7 +497,7 @@ __global__ void __launch_bounds__(kPairThreads, 1) k_gemm_pair(const GemmPairArg
 #pragma unroll
           for (int k = 0; k < 4; ++k) c[k] = cs[k];
           if ((b16 + 1) * 16 < a.nb) rotary(tb + 16);
-          if (row >= a.Nseg || i >= Tl) continue;
+          if (row >= a.Nseg || i >= min(Tl, (ch + 1) * a.nb)) continue;
           if constexpr (sw) {
             __nv_bfloat162 hi[4], lo[4];
 #pragma unroll

@@ -42,3 +42,32 @@ def test_cut_tiles(shape, lengths, monkeypatch):
     off = _errors(sh, [100] + lengths, monkeypatch)
     for m in lengths:
         assert off[m] < 1.05 * off[100], (m, off)
+
+
+def test_rows_of_the_multi_row_gemms():
+    """Prompts of 49 to 128 rows bring only as many rows of the planes as they have, in steps of eight: a row's features do not depend on
+    how many rows come after it, bit for bit."""
+    from paper_2412_18910_b200 import Engine
+    sh = si.scaled(si.SHAPES["tiny"], n_layers=2, vocab=272, d_model=2048, n_heads=16, head_dim=128, d_ffn=1424)
+    ids = si.uniform_ids(31, "rows", 128, sh.vocab)
+    e = Engine(sh, si.make_weights(sh), kv_capacity=256)
+    try:
+        feats = {}
+        for m in (128, 49, 127, 56, 57, 64, 88, 89, 120, 121):
+            e.prefill(0, ids[:m])
+            feats[m] = e.ada_debug_buffer(0, torch.float32, (1, 256, sh.d_model))[0, :m].clone()
+            assert torch.equal(feats[m], feats[128][:m]), m
+        assert e.ada_get_counters()["status"] == 0
+    finally:
+        e.close()
+
+
+@pytest.mark.parametrize("shape,lengths", [   # tiles of 32 to 128 prompt rows per thread block, full and with rows to spare, whole and cut
+    (dict(d_model=2048, n_heads=32, head_dim=64, d_ffn=5632), [130, 144, 145, 209, 230, 241, 333, 401, 433, 600, 850]),
+    (dict(d_model=4096, n_heads=32, head_dim=128, d_ffn=11008), [130, 145, 205, 209, 333, 401, 610]),
+])
+def test_tile_widths(shape, lengths, monkeypatch):
+    sh = si.scaled(si.SHAPES["tiny"], n_layers=1, vocab=272, **shape)
+    off = _errors(sh, [100] + lengths, monkeypatch)
+    for m in lengths:
+        assert off[m] < 1.05 * off[100], (m, off)
