@@ -480,11 +480,14 @@ bool gemm(ada_ctx *x, int epi, const bf16 *W0, const bf16 *W1, const bf16 *W2, i
   t.logits = logits; t.ldl = c.vocab; t.amax = x->amax;
   t.pass = x->pass; t.use_lm_rows = use_lm_rows; t.cnts = x->cnt;
   t.xrow0 = x->prompt_seq >= 0 && !chunk ? x->TM - 1 : 0;   // greedy choice of a prompt chunk: after its last row
-  const int rows = x->TM, part_rows = chunk ? kTcRowsMax : kTcRows;
+  // Prompts of up to 88 rows with the decode passes' four stages, more rows with three larger ones (four layers, 49, 77 and 88 rows with
+  // three -> four: 7B 675, 739, 753 -> 656, 717, 734 us, 13B 910, 998, 1028 -> 888, 963, 989).
+  const bool wide = chunk && x->TM > kTcRows;
+  const int rows = x->TM, part_rows = wide ? kTcRowsMax : kTcRows;
   const int d = c.d_model;
   const double wb = 2.0 * (double)Nseg * (double)K * (epi == EPI_SWIGLU ? 2 : nseg);
   timed(x, 0, wb, [&] {
-    if (chunk) launch_pdl(x, k_gemm_tc<kTcRowsMax>, dim3(tiles, t.S), kTcThreads, TcShape<kTcRowsMax>::kSmemBytes, t);
+    if (wide) launch_pdl(x, k_gemm_tc<kTcRowsMax>, dim3(tiles, t.S), kTcThreads, TcShape<kTcRowsMax>::kSmemBytes, t);
     else launch_pdl(x, k_gemm_tc<kTcRows>, dim3(tiles, t.S), kTcThreads, TcShape<kTcRows>::kSmemBytes, t);
     if (r.kind == Reduce::H) {
       reduce_h(x, t.S, part_rows, r);

@@ -1,5 +1,5 @@
 // Multi-row GEMM on the 5th-generation tensor cores for passes of up to ROWS rows (ROWS = 88: decode passes of a
-// ragged batch; ROWS = 128: prompts of 49 to 128 rows):
+// ragged batch and prompts of 49 to 88 rows; ROWS = 128: prompts of 89 to 128 rows):
 //   Y[t][n] = sum_k X[t][k] * W[n][k],  t < T <= ROWS,  W bf16 [N][K] streamed once from HBM.
 //
 // With this many rows the activation operand is no longer small next to the weights (88 rows x {hi, lo} = 22 KB per
