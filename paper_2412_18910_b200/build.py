@@ -8,7 +8,7 @@ _HERE = os.path.dirname(os.path.abspath(__file__))
 _ROOT = os.path.dirname(_HERE)
 LIB = os.path.join(_HERE, "libada.so")
 SOURCES = [os.path.join(_HERE, "csrc", "ada.cu"), os.path.join(_HERE, "csrc", "ada_static.cu")]
-DEPS = SOURCES + [os.path.join(_HERE, "csrc", "ada_kernels.cuh"), os.path.join(_HERE, "csrc", "ada_pass.cuh"), os.path.join(_HERE, "csrc", "ada_small.cuh"),
+DEPS = SOURCES + [os.path.join(_HERE, "csrc", "ada_kernels.cuh"), os.path.join(_HERE, "csrc", "ada_pass.cuh"), os.path.join(_HERE, "csrc", "ada_small.cuh"), os.path.join(_HERE, "csrc", "ada_small_shape.h"),
                   os.path.join(_HERE, "csrc", "ada_ring.h"), os.path.join(_HERE, "csrc", "ada_areas.h"), os.path.join(_HERE, "csrc", "ada_ldlp.cuh"), os.path.join(_HERE, "csrc", "ada_gemm_tc.cuh"), os.path.join(_HERE, "csrc", "ada_gemm_pair.cuh"), os.path.join(_HERE, "csrc", "ada_attn_rows.cuh"), os.path.join(_HERE, "csrc", "ada_attn_prompt.cuh"), os.path.join(_ROOT, "include", "ada.h")]
 
 

@@ -36,90 +36,9 @@
 // Every wait is bounded; a wait that gave up sets the status bit and the rest of the kernel runs without waiting.
 #pragma once
 #include "ada_pass.cuh"
+#include "ada_small_shape.h"
 
 namespace ada {
-
-constexpr int kSmCtas = 16;                 // CTAs of a cluster
-constexpr int kSmWarps = 8;
-constexpr int kSmThreads = kSmWarps * 32;
-constexpr int kSmHd = 64;                   // width of a head
-constexpr int kSmRowsMax = 16;              // rows of a sequence in one pass at most (n_max + 1)
-constexpr int kSmLmUnits = 8;               // units of 32 k of the LM head: two tiles of a warp stay in its registers
-constexpr int kSmLmRound = 2 * kSmWarps;    // its tiles that are there at a time
-// Vocabulary at most: beyond 4096 rows the LM head no longer stays in the registers, and sixteen SMs read it at 40 GB/s each.  Draft of
-// four + verify, k_pass -> here: 4096 rows 134 + 62 -> 55 + 46 us, 8192 142 + 64 -> 71 + 50, 16 384 144 + 67 -> 95 + 60, 32 768 150 +
-// 69 -> 155 + 83.
-constexpr int kSmVocabMax = 16384;
-constexpr int kSmRed = 20;                  // floats per row of a warp's 16 sums (an 8 x 4 fragment then stores into 32 banks)
-enum { SM_FC = 0, SM_QKV, SM_O, SM_GU, SM_DOWN, SM_LM, kSmKinds };                        // phases with products
-enum { SMX_X = 0, SMX_Q, SMX_A, SMX_O, SMX_AC, SMX_D, SMX_C, SMX_W, kSmBars = SMX_W + SM_LM };   // exchanges: fc, q k v, attention, O, gate/up, down, candidates; then the weights of a layer's phases
-
-// Shape of the work and places in shared memory (bytes from the aligned start), worked out on the host.
-struct SmallShape {
-  int ns;                                   // CTAs per head (whole ones)
-  int qt, gt, lt;                           // tiles of a CTA at most: QKV, gate/up (8 columns each), vocabulary (of d columns it has one)
-  int shift[SM_LM];                         // by kind of phase, log2 of the warps that share a tile's K
-  int cap_slots;                            // fresh cache rows kept in shared memory
-  const __nv_bfloat16 *w_fc, *w_lm;
-  int pages, hown, gains, rope, x[2], e, ac, q, fk, fv, cand, send[3], scratch, w[SM_LM], total;
-};
-
-__host__ __device__ inline int small_align(int x) { return (x + 127) & ~127; }
-
-// Rows that a chunk of activations is stored for: odd, so that the loads of eight lanes, two rows of four neighbouring chunks, fall into
-// different banks.
-__host__ __device__ inline int small_stride(int T) { return T | 1; }
-// Bytes of a CTA's 16 columns of an input X with the rows' partial sums of squares behind them: one copy to each CTA.
-__host__ __device__ inline int small_xblock(int T) { return 64 * small_stride(T) + ((4 * T + 15) & ~15); }
-constexpr int kSmSmemMax = 227 * 1024;
-// False if the kernel's plan does not hold the shape.
-__host__ inline bool small_shape(int L, int d, int H, int hd, int F, int V, int nmax, int pages_per_seq, SmallShape &z) {
-  if (H > kSmCtas || nmax + 1 > kSmRowsMax || hd != kSmHd || d > 16 * kSmCtas || V > kSmVocabMax) return false;
-  const int R = nmax + 1, Rs = small_stride(R), slots = 2 * nmax + 1;
-  z.ns = kSmCtas / H;
-  z.qt = (3 * hd / 16 + z.ns - 1) / z.ns;
-  z.gt = (F / 8 + kSmCtas - 1) / kSmCtas;
-  z.lt = (V / 16 + kSmCtas - 1) / kSmCtas;
-  // as many warps to a tile as there are, no more than K has units
-  const int tiles[SM_LM] = {1, z.qt, 1, z.gt, 1}, K[SM_LM] = {2 * d, d, d, d, F};
-  for (int k = 0; k < SM_LM; ++k) {
-    const int units = (K[k] + 31) / 32;
-    int l = 0;
-    while ((2 << l) * tiles[k] <= kSmWarps && (2 << l) <= units) ++l;
-    if (tiles[k] << l > kSmWarps) return false;
-    z.shift[k] = l;
-  }
-  z.cap_slots = slots;
-  const int part = R * hd * 4 + ((R * 8 + 15) & ~15);     // a CTA's partial sums of a head
-  int at = small_align(1024 + kSmWarps * kSmRowsMax * ((int)sizeof(Top2) + 4));   // barriers, row information; candidates of the warps
-  auto take = [&](int bytes) { const int p = at; at += small_align(bytes); return p; };
-  z.pages = take(pages_per_seq * 4);
-  z.hown = take(R * 16 * 4);
-  z.gains = take((2 * L + 1) * 16 * 4);
-  z.rope = take(slots * hd / 2 * 8);
-  for (int i = 0; i < 2; ++i) z.x[i] = take(d / 16 * small_xblock(R));
-  const int acb = 4 * Rs * F, rcv = H * z.ns * part;
-  z.ac = take(acb > rcv ? acb : rcv);
-  z.q = take(4 * Rs * hd);
-  z.fk = take(2 * hd * slots);
-  z.fv = take(2 * hd * slots);
-  z.cand = take(kSmCtas * R * 32);
-  int sb = part;
-  auto up = [&](int v) { if (v > sb) sb = v; };
-  up(small_xblock(R)); up(z.gt * 32 * Rs); up(z.qt * 64 * Rs); up(32 * R);
-  for (int i = 0; i < 3; ++i) z.send[i] = take(sb);
-  // the products' sums, behind them the embeddings (draft) or attention's result, whose readers write no sums of their own over them; the
-  // warps' partial sums of attention over both
-  const int red = small_align(kSmWarps * R * kSmRed * 4);
-  int sc = red + 4 * Rs * d;
-  auto upc = [&](int v) { if (v > sc) sc = v; };
-  upc(kSmWarps * R * (hd + 4) * 4); upc(kSmWarps * R * 2 * kSmRed * 4);
-  z.scratch = take(sc);
-  z.e = z.scratch + red;
-  for (int k = 0; k < SM_LM; ++k) z.w[k] = take(tiles[k] * 32 * K[k]);
-  z.total = at + 128;
-  return z.total <= kSmSmemMax;
-}
 
 __device__ __forceinline__ void mma_bf16_k16(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
   asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
@@ -233,6 +152,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(const __grid_constant__
   unsigned char *const sm = small_smem + ((128u - (smem_u32(small_smem) & 127u)) & 127u);
   uint64_t *bars = reinterpret_cast<uint64_t *>(sm);
   static_assert(kSmBars * 8 <= 112, "barriers");
+  static_assert(sizeof(Top2) + 4 <= kSmCandBytes, "candidates");
   volatile int *abort_s = reinterpret_cast<int *>(sm + 112);
   int *tok_s = reinterpret_cast<int *>(sm + 128);                       // tokens of the first rows
   int *choice_s = tok_s + kSmRowsMax;                                   // verify: the greedy choices
@@ -334,8 +254,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(const __grid_constant__
   uint32_t phases = 0;                               // per barrier the parity of its next completion (weights' among them)
   int sbuf = 0;
   uint32_t send = sm0 + z.send[0];
-  // A buffer is written again three exchanges later: each exchange but QKV's is awaited from every CTA, so by then all that was
-  // sent from it has arrived.
+  // A buffer is written again three exchanges later: by then all that was sent from it has arrived (see SMX_X).
   auto next_send = [&] { sbuf = sbuf == 2 ? 0 : sbuf + 1; send = sm0 + z.send[sbuf]; };
   auto arm = [&](int kind, int bytes) { if (tid == 0) mbar_expect_tx(bars + kind, (unsigned)bytes); };
   auto wait = [&](int kind) {
@@ -421,7 +340,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(const __grid_constant__
     constexpr bool ONE = decltype(one_const)::value;
     const int T = ONE ? 1 : T0, TS = ONE ? 1 : small_stride(T0), XB = ONE ? small_xblock(1) : small_xblock(T0);
     const int nkeys = pos + T;
-    const int PS = HD + 4, part_o = T * HD * 4, part = part_o + ((T * 8 + 15) & ~15);   // floats of a row of a warp's partial sums; bytes of a CTA's
+    const int PS = HD + 4, part_o = T * HD * 4, part = small_part(T);   // floats of a row of a warp's partial sums; bytes of a CTA's
     int l = 0;
     int arrive = -1;                                 // exchange that brings the phase's input (< 0: here already)
     // sums over the warps of a tile, of pass row r and weight row c
@@ -593,9 +512,9 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(const __grid_constant__
             if (c == 0) sts_f2(send + part_o + r * 8, M, L);
           }
         }
-        arm(SMX_A, p.H * z.ns * part);
+        arm(SMX_A, small_expect(z.heads, part));
         before_send();
-        if (has_head) copy_to_all(z.ac + rank * part, part, SMX_A);
+        copy_to_all(has_head ? z.ac + rank * part : kSmNone, has_head ? part : kSmNoneBytes, SMX_A);
         wait(SMX_A);
         // over the CTAs of each head, by every CTA for itself: O's input
         auto merge_head = [&](int r, int c) {
@@ -778,9 +697,9 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(const __grid_constant__
         }
         xs ^= 1;
         arrive = kind == SM_FC ? SMX_X : kind == SM_O ? SMX_O : SMX_D;
-        arm(arrive, nd * XB);
+        arm(arrive, small_expect(nd, XB));
         before_send();
-        if (has_d) copy_to_all(z.x[xs] + rank * XB, XB, arrive);
+        copy_to_all(has_d ? z.x[xs] + rank * XB : kSmNone, has_d ? XB : kSmNoneBytes, arrive);
       }
     };
     if constexpr (DRAFT) phase(std::integral_constant<int, SM_FC>{});
