@@ -1399,7 +1399,11 @@ extern "C" int ada_get_counters(ada_ctx *x, int64_t out[8]) {
 
 extern "C" int ada_reset_status(ada_ctx *x) {
   if (!x) return ADA_ERR_NULL;
-  if (cudaMemsetAsync(&x->cnt->status, 0, sizeof(int), x->stream) != cudaSuccess)
+  // and what a launch whose waits gave up may have left: flags of cut tiles that were set behind the wait, and arrivals of attention
+  // splits that were counted twice or not at all
+  if (cudaMemsetAsync(&x->cnt->status, 0, sizeof(int), x->stream) != cudaSuccess ||
+      cudaMemsetAsync(x->cut_flags, 0, sizeof(int) * 2 * kPairs * 8, x->stream) != cudaSuccess ||
+      cudaMemsetAsync(x->attn_cnt, 0, sizeof(int) * kMaxBatch * x->c.n_heads, x->stream) != cudaSuccess)
     return fail(x, ADA_ERR_CUDA, "ada_reset_status: memset failed");
   return ADA_OK;
 }

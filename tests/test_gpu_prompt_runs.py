@@ -44,6 +44,30 @@ def test_cut_tiles(shape, lengths, monkeypatch):
         assert off[m] < 1.05 * off[100], (m, off)
 
 
+def test_flags_that_a_wait_left_behind():
+    """A wait that gave up leaves the other pair's flag set (here: all of them): after ada_reset_status the same prompt has the same bits
+    again, and no sums of an earlier launch."""
+    from paper_2412_18910_b200 import Engine
+    sh = si.scaled(si.SHAPES["tiny"], n_layers=1, vocab=272, d_model=2048, n_heads=32, head_dim=64, d_ffn=11264)
+    e = Engine(sh, si.make_weights(sh), kv_capacity=CAP)
+    try:
+        feats = []
+        flags, counts = 2 * 74 * 8, 64       # the flags and the grid barrier's words lie, in 256 bytes each, before the phase clock
+        clock = e.ada_debug_buffer(9, torch.int64, (2560,)).data_ptr() - e.workspace.data_ptr()
+        at = clock - 4 * counts - (4 * flags + 255) // 256 * 256
+        left = e.workspace[at: at + 4 * flags].view(torch.int32)
+        for m in (205, 300, 205):
+            e.prefill(0, si.uniform_ids(29, "runs%d" % m, m, sh.vocab))
+            feats.append(e.ada_debug_buffer(0, torch.float32, (1, CAP, sh.d_model))[0, :m].clone())
+            assert not left.any()
+            left.fill_(1)
+            e.ada_reset_status()
+        assert torch.equal(feats[0], feats[2])
+        assert not left.any() and e.ada_get_counters()["status"] == 0
+    finally:
+        e.close()
+
+
 def test_rows_of_the_multi_row_gemms():
     """Prompts of 49 to 128 rows bring only as many rows of the planes as they have, in steps of eight: a row's features do not depend on
     how many rows come after it, bit for bit."""
