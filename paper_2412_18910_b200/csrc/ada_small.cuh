@@ -33,7 +33,9 @@
 //   gate/up   silu(gate) * up to everyone
 //   LM head   the CTAs' two largest logits to everyone (draft) or to the first CTA (verify)
 // Every output element depends only on its own row and on the shape: results do not depend on the rows or sequences beside it.
-// Every wait is bounded; a wait that gave up sets the status bit and the rest of the kernel runs without waiting.
+// Every wait is bounded; a wait that gave up sets the status bit (which ends the other CTAs' waits) and the rest of the kernel runs without
+// waiting.  What that CTA then reads may be anything, so it sends nothing more, arms no barrier again, whose phase may not be complete, takes
+// no token past the vocabulary, and the state of the sequence stays as it was; nobody leaves before all copies have landed.
 #pragma once
 #include "ada_pass.cuh"
 #include "ada_small_shape.h"
@@ -255,13 +257,17 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(const __grid_constant__
   int sbuf = 0;
   uint32_t send = sm0 + z.send[0];
   // A buffer is written again three exchanges later: by then all that was sent from it has arrived (see SMX_X).
-  auto next_send = [&] { sbuf = sbuf == 2 ? 0 : sbuf + 1; send = sm0 + z.send[sbuf]; };
-  auto arm = [&](int kind, int bytes) { if (tid == 0) mbar_expect_tx(bars + kind, (unsigned)bytes); };
+  int off = 0;                                       // this CTA has given up (looked at behind a barrier of the threads that waited)
+  auto next_send = [&] { sbuf = sbuf == 2 ? 0 : sbuf + 1; send = sm0 + z.send[sbuf]; off = *abort_s; };
+  auto arm = [&](int kind, int bytes) { if (tid == 0 && !off) mbar_expect_tx(bars + kind, (unsigned)bytes); };
   auto wait = [&](int kind) {
 #pragma unroll 1
     for (unsigned i = 0; !mbar_try_cluster(bars + kind, (phases >> kind) & 1u) && !*abort_s; ++i) {
       if (i > 64) __nanosleep(40);
-      if (i == kSpinLimit) { *abort_s = 1; atomicOr(&p.cnt->status, kStatTimeout); }
+      if ((i & 63) == 63 && (i >= kSpinLimit || (ld_acquire(reinterpret_cast<const unsigned *>(&p.cnt->status)) & kStatTimeout))) {
+        *abort_s = 1;
+        atomicOr(&p.cnt->status, kStatTimeout);
+      }
     }
     phases ^= 1u << kind;
   };
@@ -283,7 +289,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(const __grid_constant__
   const bool qsends = qe < qtiles * z.ns;
   const uint32_t qpeer = map_rank(sm0, (uint32_t)min(hh * z.ns + qe - qtile * z.ns, kSmCtas - 1));
   auto copy_to_all = [&](int to, int bytes, int kind) {
-    if (lane < kSmCtas / kSmWarps) bulk_s2c(peer + to, send, (unsigned)bytes, peer + 8 * kind);
+    if (lane < kSmCtas / kSmWarps && !off) bulk_s2c(peer + to, send, (unsigned)bytes, peer + 8 * kind);
   };
 
   // ---- the first rows' input (row r: token tok_s[r], position first + r).  Verify: embedding rows, as residual and as input.  Draft:
@@ -295,7 +301,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(const __grid_constant__
 #pragma unroll 1
     for (int e = tid; e < T * nd; e += kSmThreads) {
       const int r = e / nd, tile = e - r * nd;
-      const uint4 *ep = reinterpret_cast<const uint4 *>(p.embed + (size_t)tok_s[r] * d + tile * 16);
+      const uint4 *ep = reinterpret_cast<const uint4 *>(p.embed + (size_t)small_token(tok_s[r], p.V) * d + tile * 16);
       const uint4 *gp = reinterpret_cast<const uint4 *>(p.layers[0].na + tile * 16);
       const float4 *fp = reinterpret_cast<const float4 *>(p.feat + ((size_t)b * p.tok_stride + pos + r) * d + tile * 16);
       const uint32_t x = sm0 + z.x[xs] + tile * XB;
@@ -602,14 +608,14 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(const __grid_constant__
       if constexpr (kind == SM_QKV || kind == SM_GU) rms_rows();   // (the norm that the sums carry)
       __syncthreads();
       // ============================================================== what becomes of the sums
-      if (!DRAFT && l + 1 < p.n_layers) {            // the same phase's weights of the next layer
+      next_send();
+      if (!DRAFT && l + 1 < p.n_layers && !off) {    // the same phase's weights of the next layer
         wpend |= 1u << kind;
         if (warp == kSmWarps - 1) {
           asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
           fetch_weights(kind, p.layers + l + 1);
         }
       }
-      next_send();
       if constexpr (kind == SM_QKV) {
         const int n = qtiles * T;
 #pragma unroll 1
@@ -642,7 +648,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(const __grid_constant__
         if (has_head) arm(SMX_Q, 4 * HD * (T + TS));
         before_send();
         // a tile to every CTA of the head: of q 32 TS bytes a chunk, of k and v 16 bytes a row and chunk, behind those of the steps before
-        if (qsends) {
+        if (qsends && !off) {
           const int type = qm / NTI, i = qm & (NTI - 1), to = type == 0 ? z.q + i * 64 * TS : (type == 1 ? z.fk : z.fv) + (pos - fresh0) * NTI * 32 + i * 32 * T;
           bulk_s2c(qpeer + to, send + qtile * 64 * TS, type == 0 ? 64 * TS : 32 * T, qpeer + 8 * SMX_Q);
         }
@@ -823,11 +829,11 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(const __grid_constant__
           }
           continue;
         }
-        const int token = DRAFT && p.forced ? p.forced[out0 + r] : c.i1;
+        const int token = DRAFT && p.forced ? p.forced[out0 + r] : small_token(c.i1, p.V);
         if constexpr (DRAFT) {               // the embedding row of the next step
 #pragma unroll 1
           for (int c8 = lane; c8 < d / 8; c8 += 32) {
-            const uint4 er = *reinterpret_cast<const uint4 *>(p.embed + (size_t)token * d + c8 * 8);
+            const uint4 er = *reinterpret_cast<const uint4 *>(p.embed + (size_t)small_token(token, p.V) * d + c8 * 8);
             sts4(sm0 + z.e + c8 * 32, make_uint4(er.x, 0u, er.y, 0u));
             sts4(sm0 + z.e + c8 * 32 + 16, make_uint4(er.z, 0u, er.w, 0u));
           }
@@ -847,7 +853,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(const __grid_constant__
       if (takes) arm(SMX_C, kSmCtas * 32 * Tg);
       before_send();
       if (DRAFT) copy_to_all(z.cand + rank * 32 * Tg, 32 * Tg, SMX_C);
-      else if (tid == 0) bulk_s2c(peer + z.cand + rank * 32 * Tg, send, 32 * Tg, peer + 8 * SMX_C);   // (to CTA 0)
+      else if (tid == 0 && !off) bulk_s2c(peer + z.cand + rank * 32 * Tg, send, 32 * Tg, peer + 8 * SMX_C);   // (to CTA 0)
       // this CTA's columns of the feature rows: the target's, by position, or the head's own output
       if (has_d && (DRAFT || p.feat))        // (packed start positions keep no features)
 #pragma unroll 1
@@ -895,22 +901,29 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(const __grid_constant__
   }
   if (rank == 0 && tid == 0) {
     SeqState *const st = p.st + b;
+    const bool lost = *abort_s != 0;                 // (the choices may be anything: as if no pass had run)
     if (DRAFT) {
       if (refused) { st->n = 0; atomicOr(&p.cnt->status, kStatStale); }
-      if (nstep > 0) {
+      if (nstep > 0 && !lost) {
         st->dlen = q.len - 1;
         if (p.ddd_thr < 0.f) st->n = nlen;
       }
       if (p.steps_out) atomicMax(p.steps_out, nstep);
     } else {
-      if (nstep > 0) st->j_prev = fresh0;
+      if (nstep > 0) st->j_prev = lost ? -1 : fresh0;
       if (p.accept) small_accept(p, b, nstep > 0 ? tok_s + 1 : nullptr, nstep > 0 ? choice_s : nullptr);
     }
   }
-  // no CTA leaves while copies into its memory, or out of it, are under way: all that were sent have been awaited by their readers
-  await_copies(abort_s);
+  // No CTA leaves while copies into its memory, or out of it, are under way: all that were sent have been awaited by their readers.  Where one
+  // gave up it tells the others, and all of them stay, when the last has stopped sending, until what was sent has landed.
   __syncthreads();
-  asm volatile("barrier.cluster.arrive.relaxed.aligned;\n barrier.cluster.wait.aligned;" ::: "memory");   // (nothing is published here)
+  if (*abort_s) {
+    if (tid < kSmCtas) asm volatile("st.relaxed.cluster.shared::cluster.u32 [%0], 1;" ::"r"(map_rank(sm0 + 112, (uint32_t)tid)) : "memory");
+    asm volatile("fence.acq_rel.cluster;" ::: "memory");
+    __syncwarp();
+  }
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;\n barrier.cluster.wait.aligned;" ::: "memory");   // (nothing else is published here)
+  await_copies(abort_s);
 }
 
 }  // namespace ada

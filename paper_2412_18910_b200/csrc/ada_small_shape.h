@@ -44,6 +44,9 @@ enum { SM_FC = 0, SM_QKV, SM_O, SM_GU, SM_DOWN, SM_LM, kSmKinds };              
 //   barrier    its exchange     this CTA                           an exchange that this CTA sends when it has awaited the one before: a phase's
 //                               bytes may come before this CTA has armed it, but never while the phase before it is not complete
 //
+// A CTA whose wait gave up takes no part any more: it arms and sends nothing, all others' waits end by the status word, and all meet at the
+// kernel's end, where they are told and stay until every copy has landed.
+//
 // (tests/small_model.cpp runs the CTAs through it in any order.)
 enum { SMX_X = 0, SMX_Q, SMX_A, SMX_O, SMX_AC, SMX_D, SMX_C, SMX_W, kSmBars = SMX_W + SM_LM };
 
@@ -67,6 +70,8 @@ __host__ __device__ inline int small_stride(int T) { return T | 1; }
 __host__ __device__ inline int small_xblock(int T) { return 64 * small_stride(T) + ((4 * T + 15) & ~15); }
 // Bytes of a CTA's partial sums of its head: of each row hd sums, then of each row (maximum, sum).
 __host__ __device__ inline int small_part(int T) { return T * kSmHd * 4 + ((T * 8 + 15) & ~15); }
+// A token as an index of the vocabulary: a candidate is read from memory that others fill, and nobody has where a wait gave up.
+__host__ __device__ inline int small_token(int i, int V) { return (unsigned)i < (unsigned)V ? i : 0; }
 constexpr int kSmNone = 1008, kSmNoneBytes = 16;   // where, and how much, a CTA without a share sends
 // Bytes of an exchange whose first n CTAs send `bytes` each.
 __host__ __device__ inline int small_expect(int n, int bytes) { return n * bytes + (kSmCtas - n) * kSmNoneBytes; }

@@ -3,13 +3,21 @@
 //   - a copy lands on no bytes that its receiver has still to read for something earlier than what it brings
 //   - bytes reach a barrier in the phase that they are meant for
 //   - a CTA writes no buffer that a copy of its own has still to read
-//   - all CTAs come to the end
-// usage: small_model d heads F V n_max rows layers draft(0: verify, else steps) silent trials
+//   - all CTAs come to the end, and nothing is under way when they leave
+// Where a wait gives up (in any CTA, at any time; the status word then ends the other CTAs' waits) what arrives is of no use to anyone.  Checked
+// instead:
+//   - no barrier is armed again before its phase is complete
+//   - nothing is under way to or from a CTA that has left
+// usage: small_model d heads F V n_max rows layers draft(0: verify, else steps) silent trials [gives_up]
 //   silent 1: CTAs without a share say nothing (an order that must be found wrong for narrow models)
+//   gives_up 1: a wait of each trial gives up; 2: and its CTA goes on arming and sending; 3: it does not, but it alone stays for a while, before
+//   it meets the others at the end (2 and 3 must be found wrong)
+//        small_model token V i [i ...]   -> the vocabulary row that is read for candidate i
 // prints "ok" and returns 0, "refused" (3) for a shape that the kernel does not take, or the first violation (1)
 #include <algorithm>
 #include <cstdio>
 #include <cstdlib>
+#include <cstring>
 #include <random>
 #include <vector>
 #include "ada_small_shape.h"
@@ -120,10 +128,14 @@ static std::vector<Op> program(int rank) {
 static bool meet(int a, int an, int b, int bn) { return a < b + bn && b < a + an; }
 
 int main(int argc, char **argv) {
+  if (argc > 2 && !strcmp(argv[1], "token")) {
+    for (int i = 3; i < argc; ++i) printf("%d ", small_token((int)strtoll(argv[i], nullptr, 0), atoi(argv[2])));
+    return 0;
+  }
   if (argc < 11) return 2;
   d = atoi(argv[1]); H = atoi(argv[2]); F = atoi(argv[3]); V = atoi(argv[4]); nmax = atoi(argv[5]); rows = atoi(argv[6]); layers = atoi(argv[7]);
   steps = atoi(argv[8]); silent = atoi(argv[9]);
-  const int trials = atoi(argv[10]);
+  const int trials = atoi(argv[10]), gives_up = argc > 11 ? atoi(argv[11]) : 0;
   if (!small_shape(layers, d, H, H > 0 ? d / H : 0, F, V, nmax, 8, z)) { printf("refused\n"); return 3; }
   if (rows > nmax + 1 || steps > nmax) return 2;
   std::vector<Op> prog[kSmCtas];
@@ -144,12 +156,14 @@ int main(int argc, char **argv) {
     for (int c = 0; c < kSmCtas; ++c) prio[c] = c;
     std::shuffle(prio, prio + kSmCtas, rng);
     const unsigned land = trial % 3 == 0 ? 1 : trial % 3 == 1 ? 8 : 64, change = trial % 2 ? 40 : 4000;
+    bool status = false, given[kSmCtas] = {false};   // a wait has given up; in this CTA
+    int countdown = gives_up ? (int)(rng() % 50000) : -1;
     auto complete = [&](int c, int e) {
       Bar &b = bar[c][e];
       if (b.pending == 0 && b.tx == 0) { ++b.phase; b.pending = 1; }
     };
     auto reaches = [&](int c, int e, int inst, const char *what) {
-      if (bar[c][e].phase == inst) return true;
+      if (status || bar[c][e].phase == inst) return true;
       printf("trial %d: %s for instance %d of exchange %d come to CTA %d in phase %d\n", trial, what, inst, e, c, bar[c][e].phase);
       return false;
     };
@@ -160,7 +174,8 @@ int main(int argc, char **argv) {
         const int k = prio[i];
         if (pc[k] == prog[k].size()) continue;
         const Op &o = prog[k][pc[k]];
-        if (o.kind != WAIT || bar[k][o.ex].phase > o.inst) c = k;
+        if (o.kind != WAIT || bar[k][o.ex].phase > o.inst || given[k]) { c = k; continue; }
+        if (gives_up && (status ? fly.empty() || rng() % 16 == 0 : countdown-- <= 0)) { status = given[k] = true; c = k; }
       }
       if (!fly.empty() && (c < 0 || rng() % land == 0)) {
         const size_t i = rng() % fly.size();
@@ -169,7 +184,7 @@ int main(int argc, char **argv) {
         fly.pop_back();
         const auto &w = wait_at[f.dst][f.ex];
         const size_t known = f.inst < (int)w.size() ? w[f.inst] : prog[f.dst].size();
-        for (size_t k = pc[f.dst]; k < known; ++k) {
+        for (size_t k = pc[f.dst]; k < known && !status; ++k) {
           const Op &o = prog[f.dst][k];
           if (o.kind == READ && meet(o.at, o.bytes, f.to, f.bytes)) {
             printf("trial %d: exchange %d of CTA %d lands on what CTA %d has still to read\n", trial, f.ex, f.src, f.dst);
@@ -183,19 +198,31 @@ int main(int argc, char **argv) {
       }
       if (c < 0) break;
       const Op &o = prog[c][pc[c]++];
-      if (o.kind == WRITE) {
+      const bool off = given[c] && gives_up != 2;    // it takes no part any more
+      if (o.kind == WRITE && !status) {
         for (const Copy &f : fly)
           if (f.src == c && meet(o.at, o.bytes, f.at, f.bytes)) {
             printf("trial %d: CTA %d writes what its copy for exchange %d has still to read\n", trial, c, f.ex);
             return 1;
           }
-      } else if (o.kind == ARM) {
+      } else if (o.kind == ARM && !off) {
         if (!reaches(c, o.ex, o.inst, "its own bytes")) return 1;
+        if (bar[c][o.ex].pending == 0) { printf("trial %d: CTA %d arms exchange %d twice in a phase\n", trial, c, o.ex); return 1; }
         bar[c][o.ex].tx += o.bytes;
         --bar[c][o.ex].pending;
         complete(c, o.ex);
-      } else if (o.kind == SEND) {
+      } else if (o.kind == SEND && !off) {
         fly.push_back({c, o.at, o.bytes, o.dst, o.to, o.ex, o.inst});
+      }
+      // at the end all meet; where a wait gave up, all (3: only its CTA, and before they meet) stay until what is under way has landed
+      bool all = true;
+      for (int k = 0; k < kSmCtas; ++k) all = all && pc[k] == prog[k].size();
+      if (gives_up == 3 && given[c] && pc[c] == prog[c].size())
+        fly.erase(std::remove_if(fly.begin(), fly.end(), [&](const Copy &f) { return f.src == c || f.dst == c; }), fly.end());
+      if (all && gives_up < 3 && status) fly.clear();
+      if (all && !fly.empty()) {
+        printf("trial %d: a copy from CTA %d to CTA %d is under way when they have left\n", trial, fly[0].src, fly[0].dst);
+        return 1;
       }
     }
     for (int c = 0; c < kSmCtas; ++c)

@@ -36,3 +36,28 @@ def test_the_model_sees_what_is_not_ordered(model, shape):
     """Thread blocks without a share that say nothing: found for every model narrower than 256."""
     r = model(*shape, 2, 4, 0, 1, 200)
     assert r.returncode == 1 and "lands on" in r.stdout, r.stdout + r.stderr
+
+
+@pytest.mark.parametrize("shape", SHAPES)
+@pytest.mark.parametrize("draft", [False, True])
+def test_a_wait_that_gives_up(model, shape, draft):
+    """Its thread block takes no part any more, and nobody leaves before all copies have landed."""
+    n_max = shape[4]
+    for rows in {1, n_max + 1}:
+        r = model(*shape, rows, 1 if draft else 4, n_max if draft else 0, 0, 300, 1)
+        assert r.returncode == 0, (rows, r.stdout + r.stderr)
+
+
+@pytest.mark.parametrize("gives_up,draft,found", [(2, False, "twice"), (2, True, "twice"), (3, False, "have left")])
+def test_the_model_sees_a_thread_block_that_goes_on(model, gives_up, draft, found):
+    """Barriers armed twice where a thread block that gave up goes on, copies to thread blocks that have left where it alone stays for
+    them."""
+    r = model(*SHAPES[-3], 9, 1 if draft else 4, 8 if draft else 0, 0, 3000, gives_up)
+    assert r.returncode == 1 and found in r.stdout, r.stdout + r.stderr
+
+
+def test_candidates_that_nobody_wrote(model):
+    """Whatever lies in memory where a candidate should, the row that is read is one of the vocabulary's."""
+    i = [0, 1, 4095, 4096, 2**31 - 1, -1, -2**31, 0x7f800000, 0x3f800000]
+    r = model("token", 4096, *i)
+    assert r.returncode == 0 and [int(x) for x in r.stdout.split()] == [0, 1, 4095] + [0] * 6
