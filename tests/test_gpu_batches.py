@@ -1,6 +1,6 @@
-"""Batches of short sequences against one oracle run per sequence: the widths around the 48 rows of a persistent pass
-(tiny model, 9 rows a sequence: 2 to 5 sequences there, 6 and 8 on the multi-row path), passes whose rows fall on both
-sides of 8, 16 and 32, and lengths that differ inside a batch."""
+"""Batches of short sequences against one oracle run per sequence, and lengths that differ inside a batch.  The tiny model decodes on
+its cluster kernel, a cluster a sequence; test_gpu_routes.py runs the same widths, around the 48 rows of a persistent pass (9 rows a
+sequence: 2 to 5 sequences there, 6 and 8 on the multi-row path; rows on both sides of 8, 16 and 32), on a model that it does not take."""
 import numpy as np
 import pytest
 import torch
@@ -105,8 +105,8 @@ def test_step_ends_as_its_parts_do_when_sequences_fill_up():
 
 @pytest.mark.parametrize("batch", [5, 6, 8])
 def test_catch_up_rows_of_more_than_one_pass(tiny, batch):
-    """Drafts after nine tokens were committed in every sequence: 45, 54 and 72 catch-up rows, which the draft head takes in a
-    persistent pass of up to 48 rows or on the multi-row path."""
+    """Drafts after nine tokens were committed in every sequence: nine catch-up rows a cluster, or (test_gpu_routes.py) 45, 54 and 72,
+    which the draft head takes in a persistent pass of up to 48 rows or on the multi-row path."""
     import oracle
     from paper_2412_18910_b200 import Engine
     sh, w, _, m = tiny
@@ -160,8 +160,9 @@ def test_models_that_the_persistent_pass_does_not_hold(batch, wider):
 
 @pytest.mark.parametrize("vocab", [4096, 5120, 9216, 9728])
 def test_small_models_on_part_of_the_chip(vocab):
-    """Widths around the 64 thread blocks that the smallest models run on, between them and all of the chip, and on either
-    side of its 148 SMs (32 KB of the vocabulary matrix to a block)."""
+    """Vocabularies of several rounds of the cluster kernel.  On models that it does not take (test_gpu_routes.py): widths around the 64
+    thread blocks that the smallest run on, between them and all of the chip, and on either side of its 148 SMs (32 KB of the
+    vocabulary matrix to a block).  Prompts of 7 tokens are passes of those grids here too."""
     import oracle
     from paper_2412_18910_b200 import Engine
     sh = si.scaled(si.SHAPES["tiny"], vocab=vocab)

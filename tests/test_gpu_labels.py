@@ -1,6 +1,7 @@
 """Labels of packed start positions (ada_label_positions) against one label pass per position from a fresh prefill: groups
 of eight and a rest, start positions on both sides of a page boundary, drafts that reach into the next page, a sequence
-whose cache leaves room for some of them only, and a sequence that is not the first of its engine."""
+whose cache leaves room for some of them only, and a sequence that is not the first of its engine.  The tiny model's packed passes run
+on its cluster kernel; test_gpu_routes.py runs these on the multi-row path."""
 import pytest
 import torch
 
@@ -61,7 +62,7 @@ def test_packed_labels_equal_single_label_passes(tiny, plen, j0, count, cap, bat
     (180, 256, 1, False),     # no unused page beside a sequence that goes on: every position in the sequence's own pages
     (100, 192, 2, False),     # one unused page: the first positions packed, those that need two pages one by one
     (100, 512, 2, True),      # teacher forcing: one by one
-    (20, 512, 6, False)])     # packed, sequences on the multi-row path
+    (20, 512, 6, False)])     # packed, beside a batch of six
 def test_labels_leave_the_sequences_as_they_were(tiny, plen, cap, batch, forced):
     """Two engines decode the same prompts; one labels a range of prompt and decoded positions in between, after a verify whose
     outcome is accepted only then.  States, features, cache rows, drafts and choices are the same bits, and so is what follows."""

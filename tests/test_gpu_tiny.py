@@ -249,7 +249,8 @@ def test_launch_chain_equals_plain_stream_order_bit_for_bit(monkeypatch):
     """The multi-kernel path launches a layer's kernels with programmatic dependent launch (each may start while the
     one before it runs and waits inside before it touches that kernel's data).  With ADA_NO_PDL set at ada_init the
     same kernels run in plain stream order: prompt features, draft features, tokens and all verify logits of a ragged
-    batch must be the same bits, through the separate calls and through the step graph."""
+    batch must be the same bits, through the separate calls and through the step graph.  (The tiny model's prompts only: it decodes on
+    its cluster kernel.  test_gpu_routes.py has a model whose decode passes are the chain too.)"""
     from paper_2412_18910_b200 import Engine
     sh = si.SHAPES["tiny"]
     w = si.make_weights(sh)

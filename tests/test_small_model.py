@@ -61,3 +61,13 @@ def test_candidates_that_nobody_wrote(model):
     i = [0, 1, 4095, 4096, 2**31 - 1, -1, -2**31, 0x7f800000, 0x3f800000]
     r = model("token", 4096, *i)
     assert r.returncode == 0 and [int(x) for x in r.stdout.split()] == [0, 1, 4095] + [0] * 6
+
+
+def test_shapes_of_the_other_kernels(model):
+    """What the tests of the persistent pass and of the multi-row path run is refused by the cluster kernel's plan."""
+    import synth_inputs as si
+    from tests import test_gpu_routes
+    for shape in test_gpu_routes.SHAPES:
+        sh = si.scaled(si.SHAPES["tiny"], **shape)
+        r = model(sh.d_model, sh.n_heads, sh.d_ffn, sh.vocab, sh.n_max, 1, sh.n_layers, 0, 0, 1)
+        assert r.returncode == 3, (shape, r.stdout + r.stderr)
