@@ -90,9 +90,11 @@ size_t ada_workspace_bytes(const ada_config *cfg);
  * A verify pass of at most 48 rows (max_batch * (n_max + 1)) and 128 heads (max_batch * n_heads) is one persistent
  * kernel and so are all steps of a draft, launched cooperatively in thread-block clusters of two, one CTA per SM; ada_init checks that the
  * whole grid can be resident and uses the multi-kernel path otherwise.  Larger batches take that kernel
- * for the draft steps after the first.  Their other passes and the prompt of every engine run the
- * multi-kernel path with its tensor-core GEMMs, whose weight boxes are 128 rows high: d_model, d_ffn and
- * vocab must be at least 128 (ADA_ERR_BAD_CONFIG otherwise).  The environment variable ADA_PASS_NONCOOP
+ * for the draft steps after the first.  Small models (d_model up to 256 in heads of 64, d_ffn up to 1024, vocab up to 16384, n_max up to
+ * 15, as far as a layer fits the shared memory of 16 SMs) run verify passes and drafts of any batch in a cluster of 16 CTAs per
+ * sequence instead, where the device can hold one.  Prompts of up to 48 tokens are persistent passes in either case.
+ * All other passes and longer prompts run the multi-kernel path with its tensor-core GEMMs, whose weight boxes are 128 rows high:
+ * d_model, d_ffn and vocab must be at least 128 (ADA_ERR_BAD_CONFIG otherwise).  The environment variable ADA_PASS_NONCOOP
  * (any value) drops the cooperative launch attribute, for profilers that refuse it together with
  * clusters. */
 int ada_init(ada_ctx **out, const ada_config *cfg, const ada_weights *w, void *d_workspace,
@@ -211,7 +213,8 @@ int ada_selftest_bounded_wait(ada_ctx *ctx, int32_t mode, uint32_t spin_limit, i
  *         8 target choices of the last verify [max_batch][n_max+1] int32,
  *         9 phase clock of the last profiled target pass (batch 1, ada_profile on): 512 uint64
  *           nanosecond stamps, [0] = start, [i+1] = end of phase i (embedding, then per layer
- *           QKV, attention, O, gate/up, down, then the LM head). */
+ *           QKV, attention, O, gate/up, down, then the LM head), as the kernel's first CTA sees
+ *           them; written by the persistent pass and by the cluster kernel of small models. */
 int ada_debug_buffer(ada_ctx *ctx, int which, void **d_ptr, size_t *bytes);
 
 /* Measurement hook for roofline reports.  ada_profile(ctx, 1) clears the records and from then on

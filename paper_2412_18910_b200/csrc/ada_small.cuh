@@ -252,6 +252,16 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(const __grid_constant__
   }
   __syncthreads();
 
+  // phase clock of a profiled verify pass (of the first sequence): [0] its start, then the end of each phase
+  auto stamp = [&](int i) {
+    if (!DRAFT && p.phase_ns && blockIdx.x == 0 && tid == 0 && i < 512) {
+      unsigned long long t;
+      asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+      p.phase_ns[i] = t;
+    }
+  };
+  stamp(0);
+
   // ---- exchanges
   uint32_t phases = 0;                               // per barrier the parity of its next completion (weights' among them)
   int sbuf = 0;
@@ -333,6 +343,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(const __grid_constant__
       sts_f(x + 64 * TS + r * 4, ss);
     }
     __syncthreads();
+    stamp(1);
   }
 
   const int d4 = d >> 2, dr4 = kSmThreads / d4, dc4 = kSmThreads - dr4 * d4, r4 = tid / d4, c4 = tid - r4 * d4;   // walk over rows of d / 4
@@ -544,6 +555,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(const __grid_constant__
           }
         }
         __syncthreads();
+        stamp(5 * l + 3);                            // attention
         x = sm0 + z.e + t * 32 * TS;
         xu = 128 * TS;
       } else {
@@ -707,6 +719,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(const __grid_constant__
         before_send();
         copy_to_all(has_d ? z.x[xs] + rank * XB : kSmNone, has_d ? XB : kSmNoneBytes, arrive);
       }
+      stamp(5 * l + (kind == SM_QKV ? 2 : kind + 2));
     };
     if constexpr (DRAFT) phase(std::integral_constant<int, SM_FC>{});
 #pragma unroll 1
@@ -900,6 +913,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(const __grid_constant__
     cluster_sync_all();
   }
   if (rank == 0 && tid == 0) {
+    if (nstep > 0) stamp(5 * p.n_layers + 2);        // LM head and choice
     SeqState *const st = p.st + b;
     const bool lost = *abort_s != 0;                 // (the choices may be anything: as if no pass had run)
     if (DRAFT) {

@@ -79,3 +79,25 @@ def test_rows_do_not_depend_on_their_pass(tiny, prompt):
             e.close()
     for a, b in zip(*out):
         assert torch.equal(a, b)
+
+
+def test_phase_clock(tiny):
+    """ada_debug_buffer 9 of a profiled verify pass: its start, the embedding, five phases a layer, the LM head; nothing where no profile is
+    taken."""
+    from paper_2412_18910_b200 import Engine
+    sh, w, prompt, _ = tiny
+    e = Engine(sh, w, kv_capacity=512)
+    try:
+        e.prefill(0, prompt)
+        e.d_draft.zero_()
+        e.d_n.fill_(4)
+        clock = e.ada_debug_buffer(9, torch.int64, (2560,))
+        for profiled in (False, True):
+            clock.zero_()
+            e.ada_profile(profiled)
+            e.ada_verify(e.d_draft, e.d_n, e.d_target)
+            at = clock[: 5 * sh.n_layers + 3].tolist()
+            assert at == sorted(at) and (min(at) > 0) == profiled and not clock[len(at):].any()
+        assert e.ada_get_counters()["status"] == 0
+    finally:
+        e.close()
