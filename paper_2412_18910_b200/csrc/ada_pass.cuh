@@ -235,12 +235,11 @@ __device__ __forceinline__ void mbar_wait(uint64_t *bar, unsigned parity, Counte
   mbar_spin(bar, parity, cnt, abort_flag, limit);
 }
 // Where a wait gave up, copies into shared memory (this thread block's, or its peer's sums) may still be under way: the thread
-// block stays for a millisecond, in which they land.  Called once, at a kernel's end.  (In one round of the loop, which the compiler
-// otherwise writes out in 16 KB; k_pass was 0.3 % slower without those.)
-template <int UNROLL = 1>
+// block stays for a millisecond, in which they land.  Called once, at a kernel's end.  (The compiler would otherwise write the loop out in
+// 16 KB.)
 __device__ __forceinline__ void await_copies(volatile int *abort_flag) {
   if (*abort_flag)
-#pragma unroll UNROLL
+#pragma unroll 1
     for (int i = 0; i < 1000; ++i) __nanosleep(1000);
 }
 __device__ __forceinline__ void bulk_g2s_hint(void *dst, const void *src, unsigned bytes, uint64_t *bar, uint64_t pol) {
@@ -2086,7 +2085,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_pass(const __grid_constant_
   if (arrived) phase_await();   // (a prompt's pass of the draft head ends with its layer)
   }
   // let warp 2 free the tensor memory once every worker has made its last read
-  await_copies<1000>(abort_s);
+  await_copies(abort_s);
   tc_fence_before();
   named_bar(5, 32 + kNumCWarps * 32);
 }
