@@ -101,3 +101,25 @@ def test_phase_clock(tiny):
         assert e.ada_get_counters()["status"] == 0
     finally:
         e.close()
+
+
+def test_passes_behind_a_wait_that_gave_up(tiny):
+    """With the time-out bit in the status word every wait that takes long gives up: passes return, what they emit are tokens of the
+    vocabulary (or nothing), and behind ada_reset_status the same context decodes in lock step with the oracle."""
+    from paper_2412_18910_b200 import Engine
+    sh, w, prompt, m = tiny
+    e = Engine(sh, w, max_batch=1, kv_capacity=512)
+    try:
+        e.prefill(0, prompt)
+        e.ada_selftest_bounded_wait(0, 1000, torch.zeros(2, dtype=torch.int32, device=e.dev))
+        for _ in range(4):
+            assert all(0 <= t < sh.vocab for t in e.step()["emitted"][0])
+        assert e.ada_get_counters()["status"] & 4
+        e.ada_reset_status()
+        seq = m.new_seq(512)
+        assert seq.prefill(prompt) == e.prefill(0, prompt)
+        res = lockstep.run_lockstep(e, [seq], 4)
+        assert not res["failures"], res["failures"]
+        assert e.ada_get_counters()["status"] == 0
+    finally:
+        e.close()
