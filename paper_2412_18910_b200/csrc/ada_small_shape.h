@@ -76,7 +76,10 @@ constexpr int kSmNone = 1008, kSmNoneBytes = 16;   // where, and how much, a CTA
 // Bytes of an exchange whose first n CTAs send `bytes` each.
 __host__ __device__ inline int small_expect(int n, int bytes) { return n * bytes + (kSmCtas - n) * kSmNoneBytes; }
 constexpr int kSmSmemMax = 227 * 1024;
-// False if the kernel's plan does not hold the shape.
+// False if the kernel's plan does not hold the shape.  d_model up to 256 (a CTA has one tile of 16 columns of d) and heads of 64 are what
+// the plan was written for, not where k_pass gets faster: draft of four + verify of five rows at context 100, us, d_model 256 in four heads
+// 48 + 40 here, in two heads of 128 139 + 65 on k_pass, d_model 320 148 + 68; seven sequences 48 + 41, 182 + 112, 195 + 114; an eighth
+// makes a second round of clusters: 89 + 75, 184 + 110, 198 + 116.
 __host__ inline bool small_shape(int L, int d, int H, int hd, int F, int V, int nmax, int pages_per_seq, SmallShape &z) {
   if (H > kSmCtas || nmax + 1 > kSmRowsMax || hd != kSmHd || d > 16 * kSmCtas || V > kSmVocabMax) return false;
   const int R = nmax + 1, Rs = small_stride(R), slots = 2 * nmax + 1;
